@@ -231,7 +231,9 @@ ruqlp_status ruqlp_reserve(ruqlp_handle h, int64_t m, int64_t n, int d,
                            ruqlp_dtype compute, int64_t nnz);
 
 /* Workspace bytes a problem needs (0 on invalid sizes); nnz as for
- * ruqlp_reserve. */
+ * ruqlp_reserve.  (On a handle without a memory budget, dense FP32 problems
+ * also keep the skinny operand of a product split for the tensor cores: about
+ * 6 max(m, n) d bytes more.) */
 size_t ruqlp_workspace_bytes(int64_t m, int64_t n, int d, ruqlp_dtype compute,
                              int64_t nnz);
 

@@ -20,8 +20,18 @@ struct DevStatus {
   int32_t shifted;    // set by the Cholesky of the current orth when it shifted
   int32_t timeout;    // a bounded device wait ran out
   int32_t invalid;    // input checks on the device (CSR structure) failed
-  int32_t pad[3];
+  int32_t range;      // FP32 tensor-core products: RANGE_* bits
+  int32_t pad[2];
 };
+
+// What the FP32 tensor-core products met (k_f32tc.cu): an operand outside the
+// range of their split; an operand below 2^-50; a result below 2^-70.  The
+// product is formed again on the CUDA cores for the first, and for the other
+// two together.
+constexpr int32_t RANGE_OFF = 1, RANGE_SMALL = 2, RANGE_TINY = 4;
+__device__ __forceinline__ bool range_redo(int32_t r) {
+  return (r & RANGE_OFF) || (r & (RANGE_SMALL | RANGE_TINY)) == (RANGE_SMALL | RANGE_TINY);
+}
 
 template <typename T> __device__ __forceinline__ float to_f32(T v);
 template <> __device__ __forceinline__ float to_f32<float>(float v) { return v; }

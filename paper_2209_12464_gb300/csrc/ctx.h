@@ -32,6 +32,9 @@ struct ruqlp_ctx {
   int orth_simt = 0;    // 1: orth() Grams and Q = Y R^{-1} on CUDA cores
   int batch_orth_tc = 0;  // 1: batched BF16 items with dp <= 80 take the tensor-core passes
   int orth_tsqr = 0;    // 1: every orth() is a Householder TSQR
+  // room for the split skinny operand of FP32 products (k_f32tc.cu): handles
+  // under a memory budget do without it (same results)
+  bool f32_img = true;
   int tc_nsplit = 0;    // tensor-core products: column split (0 = tuned per shape)
   int test_withhold = 0;  // test hook: the next tensor-core products run out a wait
   bool tsqr_now = false;  // this run takes the TSQR orth() (fallback rerun)

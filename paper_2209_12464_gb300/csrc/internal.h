@@ -3,6 +3,7 @@
 
 #include <cuda.h>
 #include <functional>
+#include <vector>
 
 #include "common.cuh"
 
@@ -16,9 +17,11 @@ enum class Mul : int {
 };
 
 // C[M x N] = A[M x K] B[K x N]; all row-major with the given leading dims.
+// A non-null `redo` (DevStatus::range) makes the launch a no-op unless its
+// bits ask for the product to be formed again (range_redo).
 cudaError_t simt_gemm_nn(Ty ta, Ty tb, Ty tc, Mul mul, const void* A, int64_t lda,
                          const void* B, int64_t ldb, void* C, int64_t ldc, int64_t M,
-                         int64_t K, int64_t N, cudaStream_t st);
+                         int64_t K, int64_t N, cudaStream_t st, const int32_t* redo = nullptr);
 
 // C[M x N] = A^T B with A (K x M) and B (K x N) row-major.  With splits > 1
 // the K range is cut into `splits` slabs whose FP64 partial products go to
@@ -27,7 +30,7 @@ cudaError_t simt_gemm_nn(Ty ta, Ty tb, Ty tc, Mul mul, const void* A, int64_t ld
 cudaError_t simt_gemm_tn(Ty ta, Ty tb, Ty tc, Mul mul, const void* A, int64_t lda,
                          const void* B, int64_t ldb, void* C, int64_t ldc, int64_t M,
                          int64_t K, int64_t N, int splits, double* partial,
-                         const int32_t* gate, cudaStream_t st);
+                         const int32_t* gate, cudaStream_t st, const int32_t* redo = nullptr);
 
 // Number of K slabs simt_gemm_tn should use for a small M x N output.
 int tn_splits(int64_t M, int64_t K, int64_t N, int max_splits);
@@ -169,7 +172,9 @@ struct BMat {
   // Qout (FP32, leading dimension d) instead of the Y buffer (tensor-core
   // items with the CUDA-core solve and FP32 outputs: nothing reads Y after
   // that solve, the last product taking its BF16 parts)
-  int q_direct, pad2;
+  int q_direct;
+  int f32_tc[2];  // FP32 item: A X, A^T Y on the tensor cores (k_f32tc.cu)
+  void* Ximg;  // its split skinny operand (null without room for it)
   void* Qout;
   void* Lout;
   void* Pout;
@@ -291,6 +296,45 @@ cudaError_t tsqr(Ty t, const void* Y, int64_t ldy, int64_t M, int d, void* Q, in
 // of philox.cuh.
 cudaError_t omega_philox(uint64_t seed, int64_t n, int d, double* out, int64_t ldo,
                          cudaStream_t st);
+
+// FP32 products on the tensor cores (k_f32tc.cu): 128-row x 32-deep blocks,
+// column chunks of at most 224.  F32Split: nch chunks of w columns; P SMs;
+// KB K blocks; full_waves waves of whole items (a 128-row tile of a chunk),
+// then `tail` items in S slabs along K each.
+constexpr int F32_BM = 128, F32_BK = 32, F32_WMAX = 224;
+struct F32Split {
+  int nch, w, P, KB, full_waves, tail, S;
+};
+__host__ __device__ inline F32Split f32_columns(int dp) {
+  F32Split sp{};
+  sp.nch = (dp + F32_WMAX - 1) / F32_WMAX;
+  sp.w = ((dp + sp.nch - 1) / sp.nch + 15) / 16 * 16;
+  return sp;
+}
+F32Split f32_split(int64_t rows, int64_t K, int64_t m, int64_t n, int d, int dp);
+bool f32_tc_supported(int64_t K);
+// out (ld ldo, dp columns written) = A X or A^T X, A m x n FP32 (ld lda), X
+// FP32 (ld ldx, d columns, the first xcols >= d -- a multiple of 4 --
+// readable); frag: the Gram partials' buffer.  Sets st->range
+// when an operand is outside the split's range: the product must then be
+// formed again on the CUDA cores (a launch gated by that word).
+cudaError_t f32_gemm_tc(bool trans, const float* A, int64_t lda, int64_t m, int64_t n,
+                        const float* X, int64_t ldx, int xcols, int d, int dp, float* out,
+                        int64_t ldo, float* frag, void* img, DevStatus* st,
+                        cudaStream_t stream);
+// Bytes of the split X of a product over K rows (img above; null: every CTA
+// splits X itself, with the same result).
+size_t f32_img_bytes(int64_t K, int dp);
+// Batched: unit s of S of an item (tt: its index among the matrix's tail
+// items); f32_tiles appends a matrix's units and its split items.
+struct F32Tile {
+  int mat, item, tt, s, S;
+};
+void f32_tiles(int mat, const F32Split& sp, std::vector<F32Tile>& list,
+               std::vector<F32Tile>& fix);
+cudaError_t bf32_gemm_tc(bool trans, const BMat* T, const F32Tile* list, int n,
+                         const F32Tile* fix, int nfix, int src, int dst, int wmax, int count,
+                         bool img, int* err, cudaStream_t st);
 
 // Batched tensor-core products (BF16 A): tile list entries and launcher.
 struct BTcTile {

@@ -123,8 +123,9 @@ template <bool TRANS_A, typename TA, typename TB, typename TC, Mul MODE, bool PA
 __global__ void __launch_bounds__(NT)
 k_gemm(const TA* __restrict__ A, int64_t lda, const TB* __restrict__ B, int64_t ldb,
        TC* __restrict__ C, int64_t ldc, int64_t M, int64_t K, int64_t N, int64_t kslab,
-       const int32_t* __restrict__ gate) {
+       const int32_t* __restrict__ gate, const int32_t* __restrict__ redo) {
   if (gate != nullptr && *gate == 0) return;
+  if (redo != nullptr && !range_redo(*redo)) return;
   gemm_tile<TRANS_A, TA, TB, TC, MODE, PARTIAL>(A, lda, B, ldb, C, ldc, M, K, N, kslab,
                                                 blockIdx.x, blockIdx.y, blockIdx.z);
 }
@@ -136,6 +137,7 @@ k_gemm(const TA* __restrict__ A, int64_t lda, const TB* __restrict__ B, int64_t 
 template <bool TRANS_A, typename TA, typename TB, int SPLIT2 = 0>
 __global__ void __launch_bounds__(NT)
 k_bgemm(const BMat* __restrict__ T, const int* __restrict__ prefix, int count, int src, int dst) {
+  // FP32 items on the tensor cores come here only to be formed again
   const int t = blockIdx.x;
   int lo = 0, hi = count;  // largest i with prefix[i] <= t
   while (hi - lo > 1) {
@@ -143,6 +145,7 @@ k_bgemm(const BMat* __restrict__ T, const int* __restrict__ prefix, int count, i
     if (prefix[mid] <= t) lo = mid; else hi = mid;
   }
   const BMat& b = T[prefix[count + 1 + lo]];  // the launch order's item lo
+  if (b.f32_tc[TRANS_A ? 1 : 0] && !range_redo(b.status->range)) return;
   const int local = t - prefix[lo];
   const int ntn = (b.d + BN - 1) / BN;
   const int64_t Mout = TRANS_A ? b.n : b.m, K = TRANS_A ? b.m : b.n;
@@ -179,7 +182,7 @@ __global__ void k_reduce_partials(const double* __restrict__ P, int splits, int6
 template <bool TRANS_A, typename TA, typename TB, typename TC, Mul MODE>
 cudaError_t launch(const void* A, int64_t lda, const void* B, int64_t ldb, void* C, int64_t ldc,
                    int64_t M, int64_t K, int64_t N, int splits, double* partial,
-                   const int32_t* gate, cudaStream_t st) {
+                   const int32_t* gate, cudaStream_t st, const int32_t* redo = nullptr) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (splits < 1) splits = 1;
   int64_t kslab = ((K + splits - 1) / splits + BK - 1) / BK * BK;
@@ -189,12 +192,12 @@ cudaError_t launch(const void* A, int64_t lda, const void* B, int64_t ldb, void*
   dim3 grid(ceil_div(M, BM), ceil_div(N, BN), splits);
   if (splits == 1) {
     k_gemm<TRANS_A, TA, TB, TC, MODE, false><<<grid, NT, 0, st>>>(
-        (const TA*)A, lda, (const TB*)B, ldb, (TC*)C, ldc, M, K, N, kslab, gate);
+        (const TA*)A, lda, (const TB*)B, ldb, (TC*)C, ldc, M, K, N, kslab, gate, redo);
     count_launch();
     return cudaGetLastError();
   }
   k_gemm<TRANS_A, TA, TB, double, MODE, true><<<grid, NT, 0, st>>>(
-      (const TA*)A, lda, (const TB*)B, ldb, partial, N, M, K, N, kslab, gate);
+      (const TA*)A, lda, (const TB*)B, ldb, partial, N, M, K, N, kslab, gate, redo);
     count_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -219,11 +222,11 @@ int tn_splits(int64_t M, int64_t K, int64_t N, int max_splits) {
 #define RUQLP_DISPATCH(TRANS, TA_, TB_, TC_, MODE_, CTA, CTB, CTC)                         \
   if (ta == TA_ && tb == TB_ && tc == TC_ && mul == MODE_)                                 \
     return launch<TRANS, CTA, CTB, CTC, MODE_>(A, lda, B, ldb, C, ldc, M, K, N, splits,    \
-                                               partial, gate, st);
+                                               partial, gate, st, redo);
 
 cudaError_t simt_gemm_nn(Ty ta, Ty tb, Ty tc, Mul mul, const void* A, int64_t lda,
                          const void* B, int64_t ldb, void* C, int64_t ldc, int64_t M,
-                         int64_t K, int64_t N, cudaStream_t st) {
+                         int64_t K, int64_t N, cudaStream_t st, const int32_t* redo) {
   const int splits = 1;
   double* partial = nullptr;
   const int32_t* gate = nullptr;
@@ -264,7 +267,7 @@ cudaError_t bgemm(bool trans, Ty ta, Ty tb, const BMat* T, const int* prefix, in
 cudaError_t simt_gemm_tn(Ty ta, Ty tb, Ty tc, Mul mul, const void* A, int64_t lda,
                          const void* B, int64_t ldb, void* C, int64_t ldc, int64_t M,
                          int64_t K, int64_t N, int splits, double* partial,
-                         const int32_t* gate, cudaStream_t st) {
+                         const int32_t* gate, cudaStream_t st, const int32_t* redo) {
   if (splits > 1 && partial == nullptr) return cudaErrorInvalidValue;
   RUQLP_DISPATCH(true, Ty::F64, Ty::F64, Ty::F64, Mul::F64, double, double, double)
   RUQLP_DISPATCH(true, Ty::F32, Ty::F32, Ty::F32, Mul::F32, float, float, float)

@@ -130,9 +130,11 @@ inline int64_t round8(int64_t x) { return (x + 7) / 8 * 8; }
 
 // nnz >= 0: A is CSR with nnz nonzeros of val_bytes each (CSC copy kept too).
 // finish: room for Algorithm 1 step 5 (an m x dp buffer for Q P~).
+// img: room for the split skinny operand of an FP32 product (L.Bt).
 // tsqr: room for the Householder TSQR orth() (the rank-deficiency fallback).
 Layout layout_of(int64_t m, int64_t n, int d, Ty ct, int64_t nnz = -1, size_t val_bytes = 0,
-                 int finish = 0, bool gen_omega = false, int64_t lr_r = 0, bool tsqr = false) {
+                 int finish = 0, bool gen_omega = false, int64_t lr_r = 0, bool tsqr = false,
+                 bool img = false) {
   Layout L{};
   const int dp = round16(d);
   const size_t wes = ty_size(work_ty(ct));
@@ -169,6 +171,8 @@ Layout layout_of(int64_t m, int64_t n, int d, Ty ct, int64_t nnz = -1, size_t va
     L.Btl = L.Bt + one;
     L.frag = take(tc_frag_bytes(dp <= 256 ? dp : 256));  // per column chunk
   }
+  if (ct == Ty::F32 && nnz < 0 && img && f32_tc_supported(std::max(m, n)))
+    L.Bt = take(f32_img_bytes(std::max(m, n), dp));
   if (finish) L.T = take((size_t)m * dp * wes);
   if (finish == 2) {  // Jacobi SVD of L: W, V, S, order, norms, sweep count, sorted U and V
     L.svdW = take((size_t)d * d * wes);
@@ -291,6 +295,8 @@ struct Job {
   Ty ot;
   int finish_paper;  // 0 none, 1 qr(L) (Algorithm 1 step 5), 2 SVD of L (Remark 1)
   bool use_tc;  // BF16 products on the tensor cores (k_tc.cu)
+  bool f32_tc[2] = {false, false};  // FP32 A X, A^T Y on the tensor cores (k_f32tc.cu)
+  int x_cols = 0;       // readable columns of a caller's skinny operand (0: an arena buffer)
   // CSR input (work type FP32): A's arrays and the CSC copy in the arena
   bool csr = false;
   const int32_t* rowptr = nullptr;
@@ -488,6 +494,15 @@ ruqlp_status product(ruqlp_ctx* h, const Layout& Lo, const Job& J, bool trans, T
     return RUQLP_OK;
   }
   const Mul mul = (J.ct == Ty::F64) ? Mul::F64 : Mul::F32;
+  // FP32: the tensor-core product, then a launch that forms it again on the
+  // CUDA cores if an operand was outside the split's range (else a no-op)
+  const int32_t* redo = nullptr;
+  if (J.f32_tc[trans]) {
+    CK(f32_gemm_tc(trans, (const float*)J.A, J.lda, J.m, J.n, (const float*)Xin, ldx,
+                   J.x_cols ? J.x_cols : J.dp, J.d, J.dp, (float*)out, J.dp,
+                   (float*)(base + Lo.partial), Lo.Bt ? base + Lo.Bt : nullptr, h->status, st));
+    redo = &h->status->range;
+  }
   if (J.ct == Ty::BF16 && split2) {
     // the two-part operand, rounded as the tensor cores use it (h + l is exact
     // in FP32)
@@ -506,10 +521,11 @@ ruqlp_status product(ruqlp_ctx* h, const Layout& Lo, const Job& J, bool trans, T
     ldx = J.d;
   }
   if (!trans)
-    CK(simt_gemm_nn(J.ct, xt, J.wt, mul, J.A, J.lda, Xin, ldx, out, J.dp, Mout, K, J.d, st));
+    CK(simt_gemm_nn(J.ct, xt, J.wt, mul, J.A, J.lda, Xin, ldx, out, J.dp, Mout, K, J.d, st,
+                    redo));
   else
     CK(simt_gemm_tn(J.ct, xt, J.wt, mul, J.A, J.lda, Xin, ldx, out, J.dp, Mout, K, J.d, 1,
-                    nullptr, nullptr, st));
+                    nullptr, nullptr, st, redo));
   return RUQLP_OK;
 }
 
@@ -544,6 +560,8 @@ void fill_job(const ruqlp_matrix* A, const ruqlp_params* prm, const ruqlp_output
   } else {
     J.A = A->dense.data;
     J.lda = A->dense.ld;
+    J.f32_tc[0] = J.ct == Ty::F32 && f32_tc_supported(n);
+    J.f32_tc[1] = J.ct == Ty::F32 && f32_tc_supported(m);
   }
 }
 
@@ -578,7 +596,8 @@ ruqlp_status run_dense(ruqlp_ctx* h, const Job& J0) {
   const bool ts = h->tsqr_now || h->orth_tsqr;
   const Layout Lo = J.csr ? layout_of(J.m, J.n, J.d, J.ct, J.nnz, ty_size(J.tv), J.finish_paper,
                                       gen, J.lr_r, ts)
-                          : layout_of(J.m, J.n, J.d, J.ct, -1, 0, J.finish_paper, gen, 0, ts);
+                          : layout_of(J.m, J.n, J.d, J.ct, -1, 0, J.finish_paper, gen, 0, ts,
+                                      h->f32_img);
   ruqlp_status s = ensure_arena(h, Lo.total);
   if (s != RUQLP_OK) return s;
   CK(status_reset(h->status, h->stream));
@@ -787,8 +806,14 @@ size_t batch_item_bytes(const ruqlp_matrix* A, const ruqlp_params* prm) {
   const int64_t sl = std::max(gram_slabs(m, kMaxSplits, &slab), gram_slabs(n, kMaxSplits, &slab));
   const size_t per = (size_t)(3 * n + m) * dp * 4 + (size_t)sl * d * d * 8 + (size_t)d * d * 12 +
                      chol_tiles_bytes(d) + (size_t)2 * dp * std::max(m, n) * 2 + 8 * 256;
+  size_t units = 0;  // FP32 tensor-core units (with their split items)
+  if (prm->compute == RUQLP_F32)
+    for (const bool trans : {false, true}) {
+      const F32Split sp = f32_split(trans ? n : m, trans ? m : n, m, n, d, dp);
+      units += (size_t)sp.full_waves * sp.P + (size_t)sp.tail * (sp.S + 1);
+    }
   // plus its share of the metadata (table entry, prefixes, tile lists, maps)
-  return per + 4096 + (size_t)(ceil_div(m, 128) + ceil_div(n, 128)) * 8;
+  return per + 4096 + units * sizeof(F32Tile) + (size_t)(ceil_div(m, 128) + ceil_div(n, 128)) * 8;
 }
 
 bool batchable(const ruqlp_matrix* A, const ruqlp_params* prm) {
@@ -807,6 +832,7 @@ void copy_options(const ruqlp_ctx* from, ruqlp_ctx* to) {
   to->batch_orth_tc = from->batch_orth_tc;
   to->orth_tsqr = from->orth_tsqr;
   to->tc_nsplit = from->tc_nsplit;
+  to->f32_img = from->f32_img;  // the request loop enforces its parent's budget
 }
 
 ruqlp_status set_error(ruqlp_ctx* h, ruqlp_status s, const char* msg) {
@@ -838,6 +864,10 @@ struct BatchPlan {
   // trsmY, trsmN, gramY, gramN (wide items)
   std::vector<int> prefix[NPF];
   std::vector<BTcTile> tc_nn, tc_tn;  // tensor-core tile lists
+  // FP32 tensor-core units and split items, A X then A^T Y
+  std::vector<F32Tile> ft[2], ftfix[2];
+  size_t off_ft[2], off_ftfix[2];
+  int wmax_ft = 16;
   // tensor-core CholeskyQR items (orth_tc): their list (for k_btrinv) and,
   // over Y (m rows) and over Z (n rows), the Gram units (one row slab each)
   // and the Q = Y R^{-1} units with their per-CTA ranges
@@ -899,6 +929,9 @@ ruqlp_status batch_launches(ruqlp_ctx* h, const BatchPlan& bp, int count, int q,
   auto prod = [&](bool trans, int src, int dst, bool split2) -> ruqlp_status {
     ProfScope sp(ph, trans ? PROF_ATX : PROF_AX);
     const int pf = trans ? PF_TN : PF_NN;
+    CK(bf32_gemm_tc(trans, T, (const F32Tile*)(base + bp.off_ft[trans]), (int)bp.ft[trans].size(),
+                    (const F32Tile*)(base + bp.off_ftfix[trans]), (int)bp.ftfix[trans].size(),
+                    src, dst, bp.wmax_ft, count, h->f32_img, err, st));
     CK(bgemm(trans, ct, Ty::F32, T, pre(pf), tot(pf), count, src, dst, st, split2));
     const auto& list = trans ? bp.tc_tn : bp.tc_nn;
     if (!list.empty()) {  // Bt (and Btl) were written by the step that produced buf[src]
@@ -993,6 +1026,14 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
     const int d = dd[i], dp = round16(d);
     BMat& b = bp.table[i];
     b.use_tc = (ct0 == Ty::BF16 && !h->bf16_simt && tc_supported(D.data, D.ld, dp)) ? 1 : 0;
+    for (int x = 0; x < 2; ++x) {
+      const int64_t rows = x ? n : m, K = x ? m : n;
+      b.f32_tc[x] = (ct0 == Ty::F32 && f32_tc_supported(K)) ? 1 : 0;
+      if (!b.f32_tc[x]) continue;
+      bp.wmax_ft = std::max(bp.wmax_ft, f32_columns(dp).w);
+      f32_tiles(i, f32_split(rows, K, m, n, d, dp), bp.ft[x], bp.ftfix[x]);
+    }
+    const bool img = h->f32_img && (b.f32_tc[0] || b.f32_tc[1]);
     // option batch_orth_tc: BF16 items of width dp <= 80 run their
     // CholeskyQR passes on the tensor cores (a rule on the dtype, the
     // options and d only, so an item decides the same alone and in any
@@ -1015,6 +1056,7 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
     oGf[i] = take((size_t)d * d * 4);
     oT[i] = take(chol_tiles_bytes(d));
     oB[i] = b.use_tc ? take((size_t)2 * dp * b.ldbt * 2) : 0;  // Bt, then Btl
+    if (img) oB[i] = take(f32_img_bytes(std::max(m, n), dp));
     oS[i] = b.orth_tc ? take(bo_st_bytes(d)) : 0;
     if (b.orth_tc) bp.dmax_otc = std::max(bp.dmax_otc, d);
     bp.dmax = std::max(bp.dmax, d);
@@ -1035,6 +1077,17 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
       n_nn += ceil_div(A[i].dense.m, 128);
       n_tn += ceil_div(A[i].dense.n, 128);
     }
+  for (int x = 0; x < 2; ++x) {
+    // longest contraction first, as the BF16 tile lists
+    std::stable_sort(bp.ft[x].begin(), bp.ft[x].end(), [&](const F32Tile& a, const F32Tile& b) {
+      auto cost = [&](const F32Tile& t) {
+        return (x ? A[t.mat].dense.m : A[t.mat].dense.n) / t.S;
+      };
+      return cost(a) > cost(b);
+    });
+    bp.off_ft[x] = take(sizeof(F32Tile) * bp.ft[x].size());
+    bp.off_ftfix[x] = take(sizeof(F32Tile) * bp.ftfix[x].size());
+  }
   bp.off_tc_nn = take(sizeof(BTcTile) * std::max<size_t>(n_nn, 1));
   bp.off_tc_tn = take(sizeof(BTcTile) * std::max<size_t>(n_tn, 1));
   {
@@ -1124,6 +1177,7 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
     b.tiles = (float*)(base + oT[i]);
     b.Bt = b.use_tc ? (void*)(base + oB[i]) : nullptr;
     b.Btl = b.use_tc ? (void*)(base + oB[i] + (size_t)b.dp * b.ldbt * 2) : nullptr;
+    b.Ximg = h->f32_img && (b.f32_tc[0] || b.f32_tc[1]) ? (void*)(base + oB[i]) : nullptr;
     b.St = b.orth_tc ? (void*)(base + oS[i]) : nullptr;
     b.omega = prm[i].omega;
     b.seed = prm[i].omega_seed;
@@ -1175,6 +1229,7 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
     key.push_back(bp.table[i].n);
     key.push_back(bp.table[i].d);
     key.push_back(bp.table[i].use_tc);
+    key.push_back(bp.table[i].f32_tc[0] + 2 * bp.table[i].f32_tc[1]);
     key.push_back(bp.table[i].orth_tc);
   }
   ruqlp_ctx::BatchEntry* g = nullptr;
@@ -1219,6 +1274,10 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
   put(bp.off_table, bp.table.data(), sizeof(BMat) * count);
   for (int k = 0; k < NPF; ++k)
     put(bp.off_prefix[k], bp.prefix[k].data(), sizeof(int) * (2 * count + 1));
+  for (int x = 0; x < 2; ++x) {
+    put(bp.off_ft[x], bp.ft[x].data(), sizeof(F32Tile) * bp.ft[x].size());
+    put(bp.off_ftfix[x], bp.ftfix[x].data(), sizeof(F32Tile) * bp.ftfix[x].size());
+  }
   put(bp.off_tc_nn, bp.tc_nn.data(), sizeof(BTcTile) * bp.tc_nn.size());
   put(bp.off_tc_tn, bp.tc_tn.data(), sizeof(BTcTile) * bp.tc_tn.size());
   put(bp.off_maps, g->maps.data(), g->maps.size());
@@ -1320,6 +1379,7 @@ ruqlp_status ruqlp_create(ruqlp_handle* out, const ruqlp_config* cfg) {
   h->stream = (cudaStream_t)cfg->cuda_stream;
   h->budget = cfg->hbm_budget_bytes;
   h->max_slots = cfg->max_slots > 0 ? cfg->max_slots : 8;
+  h->f32_img = h->budget == 0;
   if (cudaSetDevice(h->device) != cudaSuccess ||
       cudaMalloc(&h->status, sizeof(DevStatus)) != cudaSuccess ||
       cudaMallocHost(&h->status_host, sizeof(DevStatus)) != cudaSuccess) {
@@ -1423,7 +1483,9 @@ ruqlp_status ruqlp_reserve(ruqlp_handle h, int64_t m, int64_t n, int d, ruqlp_dt
   if (!h) return RUQLP_ERR_INVALID;
   const size_t b = ruqlp_workspace_bytes(m, n, d, compute, nnz);
   if (b == 0) return fail(h, RUQLP_ERR_INVALID, "invalid sizes for ruqlp_reserve");
-  return ensure_arena(h, b);
+  return ensure_arena(h, nnz < 0 && compute == RUQLP_F32 && h->f32_img
+                             ? layout_of(m, n, d, Ty::F32, -1, 0, 0, false, 0, false, true).total
+                             : b);
 }
 
 ruqlp_status ruqlp_decompose(ruqlp_handle h, const ruqlp_matrix* A, const ruqlp_params* prm,
@@ -1499,7 +1561,8 @@ static ruqlp_status decompose_host_once(ruqlp_handle h, const ruqlp_matrix* A,
   const bool ts = h->tsqr_now || h->orth_tsqr;
   const Layout Lo = J.csr ? layout_of(m, n, d, J.ct, J.nnz, ty_size(J.tv), J.finish_paper, gen,
                                       0, ts)
-                          : layout_of(m, n, d, J.ct, -1, 0, J.finish_paper, gen, 0, ts);
+                          : layout_of(m, n, d, J.ct, -1, 0, J.finish_paper, gen, 0, ts,
+                                      h->f32_img);
   size_t off = align_up(Lo.total, 256);
   auto take = [&](size_t bytes) {
     const size_t o = off;
@@ -1612,7 +1675,7 @@ ruqlp_status ruqlp_sketch(ruqlp_handle h, const ruqlp_matrix* A, int trans, cons
              tc_supported(J.A, J.lda, std::min(J.dp, 256));
   const int64_t Mout = trans ? n : m;
   const Layout Lo = J.csr ? layout_of(m, n, d, J.ct, J.nnz, ty_size(J.tv), false, false, J.lr_r)
-                          : layout_of(m, n, d, J.ct);
+                          : layout_of(m, n, d, J.ct, -1, 0, 0, false, 0, false, h->f32_img);
   s = ensure_arena(h, Lo.total);
   if (s != RUQLP_OK) return s;
   CK(status_reset(h->status, h->stream));
@@ -1623,9 +1686,14 @@ ruqlp_status ruqlp_sketch(ruqlp_handle h, const ruqlp_matrix* A, int trans, cons
   void* stage = (char*)h->arena + (trans ? Lo.Z : Lo.Y);
   const void* Xuse = X;
   int64_t ldxu = ldx;
-  if (J.csr && ((ldx % 4) || ((uintptr_t)X & 15))) {  // 128-bit gathers need aligned rows
+  // the SpMM's 128-bit gathers and the FP32 tensor-core product's 128-bit loads
+  // need aligned rows
+  const bool f32_tc = J.f32_tc[trans != 0];
+  J.x_cols = f32_tc ? d : 0;
+  if (((J.csr || f32_tc) && ((ldx % 4) || ((uintptr_t)X & 15))) || (f32_tc && d % 4)) {
     void* Xa = (char*)h->arena + (trans ? Lo.Y : Lo.X);  // m x dp or n x dp
     const int64_t K = trans ? m : n;
+    J.x_cols = 0;
     CK(copy_cast_2d(J.wt, X, ldx, J.wt, Xa, J.dp, K, d, h->stream));
     Xuse = Xa;
     ldxu = J.dp;
