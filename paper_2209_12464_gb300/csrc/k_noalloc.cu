@@ -87,8 +87,8 @@ extern "C" ruqlp_status ruqlp_gram_noalloc(const void* Y, int64_t M, int d, int6
   int splits = tn_splits(d, M, d, 64);
   const int64_t fit = kScratchDoubles / ((int64_t)d * d);
   if (splits > fit) splits = (int)fit;
-  // Every slab writes all d x d entries of its partial, so nothing in the
-  // scratch has to start at zero; the previous call's contents are overwritten.
+  // Every slab writes the entries of its partial that the reduction reads, so
+  // nothing in the scratch has to start at zero; the previous call's contents are overwritten.
   const cudaError_t e = simt_gemm_tn(ty, ty, Ty::F64, Mul::F64, Y, ldy, Y, ldy, G, d, d, M, d,
                                      splits, scratch, nullptr, (cudaStream_t)cuda_stream);
   return e == cudaSuccess ? RUQLP_OK : RUQLP_ERR_CUDA;

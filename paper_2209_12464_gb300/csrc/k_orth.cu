@@ -5,6 +5,8 @@
 // triangular solve Q = Y R^{-1}, and small layout helpers.
 #include <math.h>
 
+#include <algorithm>
+
 #include "../../include/ruqlp.h"
 #include "internal.h"
 
@@ -43,6 +45,7 @@ k_chol(const double* __restrict__ G, int d, double shift_rel, int force_shift,
   __shared__ int s_rankdef;
   __shared__ int s_far;
   __shared__ double s_shift;
+  __shared__ TF s_t[512];  // row k / pivot (d <= 512)
   const bool check_on = check == 1 || (check == 2 && status->shifted == 0);
   TF* W = PACKED ? reinterpret_cast<TF*>(smem_d) : reinterpret_cast<TF*>(R);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -67,32 +70,43 @@ k_chol(const double* __restrict__ G, int d, double shift_rel, int force_shift,
     if (tid == 0) s_bad = 0;
     __syncthreads();
     for (int k = 0; k < d; ++k) {
-      if (tid == 0) {
+      // the chain per column is one division: t = row k / pivot, then a_ij -=
+      // a_ki t_j; the square roots wait until the end (with them and the
+      // row's division in the chain a 30-column FP64 factor took 42 us)
+      if (warp == 0) {
         TF piv = W[uidx<PACKED>(k, k, d)];
-        if (check_on && attempt == 0 && !(piv >= TF(0.5) && piv <= TF(2))) s_far = 1;
+        __syncwarp();
+        if (lane == 0 && check_on && attempt == 0 && !(piv >= TF(0.5) && piv <= TF(2))) s_far = 1;
         if (!(piv > TF(0)) || !isfinite((double)piv)) {
           if (attempt == 0) {
             s_bad = 1;
           } else {
             piv = (TF)s_shift;
-            s_rankdef = 1;
+            if (lane == 0) {
+              s_rankdef = 1;
+              W[uidx<PACKED>(k, k, d)] = piv;
+            }
           }
         }
-        W[uidx<PACKED>(k, k, d)] = sqrt(piv);
+        const TF inv = TF(1) / piv;
+        for (int j = k + 1 + lane; j < d; j += 32) s_t[j] = W[uidx<PACKED>(k, j, d)] * inv;
       }
       __syncthreads();
       if (s_bad) break;
-      const TF rkk = W[uidx<PACKED>(k, k, d)];
-      for (int j = k + 1 + tid; j < d; j += blockDim.x) W[uidx<PACKED>(k, j, d)] /= rkk;
-      __syncthreads();
       for (int i = k + 1 + warp; i < d; i += nwarps) {
-        const TF rki = W[uidx<PACKED>(k, i, d)];
-        for (int j = i + lane; j < d; j += 32)
-          W[uidx<PACKED>(i, j, d)] -= rki * W[uidx<PACKED>(k, j, d)];
+        const TF aki = W[uidx<PACKED>(k, i, d)];
+        for (int j = i + lane; j < d; j += 32) W[uidx<PACKED>(i, j, d)] -= aki * s_t[j];
       }
       __syncthreads();
     }
     if (!s_bad) break;
+  }
+  __syncthreads();
+  for (int i = warp; i < d; i += nwarps) {  // row i of R = row i / sqrt(pivot)
+    const TF r = sqrt(W[uidx<PACKED>(i, i, d)]);
+    __syncwarp();
+    for (int j = i + lane; j < d; j += 32)
+      W[uidx<PACKED>(i, j, d)] = j == i ? r : W[uidx<PACKED>(i, j, d)] / r;
   }
   __syncthreads();
   // R (full FP64, zero lower part) and its working-type copy; in global mode
@@ -136,6 +150,7 @@ k_trsm(const T* __restrict__ Y, int64_t ldy, const T* __restrict__ R, T* __restr
   if (gate != nullptr && *gate == 0) return;
   extern __shared__ unsigned char smem_raw[];
   T* S = reinterpret_cast<T*>(smem_raw);
+  __shared__ T s_inv[512];  // 1 / R_jj (d <= 512)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t r0 = (int64_t)blockIdx.x * rows;
   const int nr = (int)min((int64_t)rows, M - r0);
@@ -143,9 +158,10 @@ k_trsm(const T* __restrict__ Y, int64_t ldy, const T* __restrict__ R, T* __restr
     const int r = e / d, c = e % d;
     S[(int64_t)r * d + c] = Y[(r0 + r) * ldy + c];
   }
+  for (int j = tid; j < d; j += blockDim.x) s_inv[j] = T(1) / R[(int64_t)j * d + j];
   __syncthreads();
   for (int j = 0; j < d; ++j) {
-    const T inv = T(1) / R[(int64_t)j * d + j];
+    const T inv = s_inv[j];
     for (int r = warp; r < nr; r += 8) {
       T* srow = S + (int64_t)r * d;
       const T xj = srow[j] * inv;
@@ -242,8 +258,10 @@ cudaError_t trsm_right_upper(Ty ty, const void* Y, int64_t ldy, const void* R, v
   if (M <= 0 || d <= 0) return cudaSuccess;
   const size_t es = ty_size(ty);
   int rows = (int)((200 * 1024) / ((size_t)d * es));
-  if (rows > 64) rows = 64;
-  rows = rows / 8 * 8;
+  // at most 64 rows per CTA, fewer when that leaves SMs idle (1000 x 30 in FP64:
+  // 16 CTAs of 64 rows 66 us; the rows are independent, so the result is the same)
+  rows = std::min(rows, std::min(64, std::max(8, ceil_div(M, 4 * sm_count()))));
+  rows = std::max(rows / 8 * 8, std::min(rows, 8));
   if (rows < 8) return cudaErrorInvalidValue;
   const size_t sm = (size_t)rows * d * es;
   const int grid = ceil_div(M, rows);

@@ -6,6 +6,7 @@
 // 4 x 4 sub-tile.  K is walked in 16-wide slabs staged in shared memory.
 // Out-of-range rows/columns are zero-filled on load and skipped on store, so
 // any M, K, N works (ragged tails included).
+#include <algorithm>
 #include <type_traits>
 
 #include "internal.h"
@@ -157,15 +158,243 @@ k_bgemm(const BMat* __restrict__ T, const int* __restrict__ prefix, int count, i
       ((K + BK - 1) / BK) * BK, local / ntn, local % ntn, 0);
 }
 
+// FP64 products of one matrix with tiles fitted to the shape.  A CTA computes a
+// BM x BN tile (BN any multiple of NI), each thread MI x NI of it, an FMA chain
+// over K per entry.
+// Products (PART = false): a cluster of S CTAs shares a tile; CTA s sums K slab
+// s, and the slab sums are added in slab order through distributed shared
+// memory.  Partial sums (PART = true, C = A^T B of a few columns): CTA (pair,
+// slab) writes its tile of slab's M x N sum; tiles are the pairs (i, j) of
+// equal column chunks, with sym only j >= i.
+// The FP64 units do two DFMA per clock and SM, so an FP64 product is bound by
+// them (1.19 TFLOP/s); neighbouring CTAs of an SM hide the loads.
+struct FitShape {
+  int bm, bn;     // tile
+  int nch, nchm;  // column chunks, row chunks (partial sums)
+  int64_t kslab;  // K per slab
+  int S;          // slabs (products: CTAs per cluster)
+  bool sym;
+};
+constexpr int FIT_BN = 64;       // widest tile of a product
+constexpr int FIT_BN_PART = 44;  // ... of a partial sum (square tiles)
+constexpr int FIT_BK = 32;       // K per staged block
+
+template <int N>
+__device__ __forceinline__ void fit_ld(const double* p, double (&v)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; i += 2) {
+    const double2 x = *reinterpret_cast<const double2*>(p + i);
+    v[i] = x.x;
+    v[i + 1] = x.y;
+  }
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+template <bool TRANS_A, typename T, int MI, int NI, bool PART>
+__global__ void __launch_bounds__(512)
+k_fit(const T* __restrict__ A, int64_t lda, const T* __restrict__ B, int64_t ldb,
+      double* __restrict__ C, int64_t ldc, int64_t M, int64_t K, int64_t N, FitShape f,
+      const int32_t* __restrict__ gate) {
+  constexpr int BK = FIT_BK, PAD = 2;  // rows stay on 16 bytes
+  extern __shared__ __align__(16) unsigned char fit_smem[];
+  if (gate != nullptr && *gate == 0) return;  // (the same for a whole cluster)
+  const int bm = f.bm, bn = f.bn, t = threadIdx.x, nt = blockDim.x;
+  const int pa = bm + PAD, pb = bn + PAD;
+  double* As = reinterpret_cast<double*>(fit_smem);  // [BK][pa]
+  double* Bs = As + BK * pa;                     // [BK][pb]
+  // the block is a multiple of 32 threads: those past the tile only load
+  const int nx = bn / NI;
+  const bool live = t < (bm / MI) * nx;
+  const int tx = live ? t % nx : 0, ty = live ? t / nx : 0;
+  int64_t m0, n0;
+  int slab;
+  if (PART) {
+    int i = 0, j = blockIdx.x;
+    if (f.sym) {
+      while (j >= f.nch - i) { j -= f.nch - i; ++i; }
+      j += i;
+    } else {
+      i = j / f.nch;
+      j -= i * f.nch;
+    }
+    m0 = (int64_t)i * bm;
+    n0 = (int64_t)j * bn;
+    slab = blockIdx.y;
+  } else {
+    m0 = (int64_t)(blockIdx.x / f.S) * bm;
+    n0 = (int64_t)blockIdx.y * bn;
+    slab = blockIdx.x % f.S;  // rank in the cluster
+  }
+  const int64_t kz0 = (int64_t)slab * f.kslab, kz1 = min(K, kz0 + f.kslab);
+  const int warp = t >> 5, lane = t & 31, nw = nt >> 5;
+  double acc[MI][NI];
+#pragma unroll
+  for (int i = 0; i < MI; ++i)
+#pragma unroll
+    for (int j = 0; j < NI; ++j) acc[i][j] = 0.0;
+  for (int64_t k0 = kz0; k0 < kz1; k0 += BK) {
+    if (TRANS_A) {  // a warp per k, lanes along m
+#pragma unroll 4
+      for (int c = warp; c < BK; c += nw)
+        for (int r = lane; r < bm; r += 32)
+          As[c * pa + r] = (m0 + r < M && k0 + c < kz1) ? (double)(A[(k0 + c) * lda + m0 + r])
+                                                        : 0.0;
+    } else {  // 16 consecutive k per row
+      for (int e = t; e < bm * BK; e += nt) {
+        const int r = e / BK, c = e % BK;
+        As[c * pa + r] = (m0 + r < M && k0 + c < kz1) ? (double)(A[(m0 + r) * lda + k0 + c])
+                                                      : 0.0;
+      }
+    }
+#pragma unroll 4
+    for (int c = warp; c < BK; c += nw)
+      for (int r = lane; r < bn; r += 32)
+        Bs[c * pb + r] = (n0 + r < N && k0 + c < kz1) ? (double)(B[(k0 + c) * ldb + n0 + r])
+                                                      : 0.0;
+    __syncthreads();
+    if (live) {
+#pragma unroll 16
+      for (int kk = 0; kk < BK; ++kk) {
+        double a[MI], b[NI];
+        fit_ld(As + kk * pa + ty * MI, a);
+        fit_ld(Bs + kk * pb + tx * NI, b);
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+          for (int j = 0; j < NI; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+      }
+    }
+    __syncthreads();
+  }
+  if (PART || f.S == 1) {
+    double* Cz = PART ? C + (int64_t)slab * M * ldc : C;
+    if (!live) return;
+#pragma unroll
+    for (int i = 0; i < MI; ++i) {
+      const int64_t gm = m0 + ty * MI + i;
+#pragma unroll
+      for (int j = 0; j < NI; ++j) {
+        const int64_t gn = n0 + tx * NI + j;
+        if (gm < M && gn < N) Cz[gm * ldc + gn] = acc[i][j];
+      }
+    }
+    return;
+  }
+  // slab sums to shared memory; CTA s adds the entries s, s + S, ... of all slabs
+  double* W = reinterpret_cast<double*>(fit_smem);
+  if (live) {
+#pragma unroll
+    for (int i = 0; i < MI; ++i)
+#pragma unroll
+      for (int j = 0; j < NI; ++j) W[(ty * MI + i) * bn + tx * NI + j] = acc[i][j];
+  }
+  cluster_barrier();
+  const uint32_t w0 = (uint32_t)__cvta_generic_to_shared(W);
+  for (int e = t * f.S + slab; e < bm * bn; e += nt * f.S) {
+    const int r = e / bn, c = e - r * bn;
+    if (m0 + r >= M || n0 + c >= N) continue;
+    double v[8];
+#pragma unroll
+    for (int z = 0; z < 8; ++z) {
+      v[z] = 0.0;
+      if (z < f.S) {
+        uint32_t p;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                     : "=r"(p)
+                     : "r"(w0 + e * (uint32_t)sizeof(double)), "r"(z));
+        asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v[z]) : "r"(p) : "memory");
+      }
+    }
+    double s = v[0];
+#pragma unroll
+    for (int z = 1; z < 8; ++z)
+      if (z < f.S) s += v[z];
+    C[(m0 + r) * ldc + n0 + c] = s;
+  }
+  cluster_barrier();  // no CTA leaves while others read its slab
+}
+
+size_t fit_smem_bytes(const FitShape& f, bool reduce) {
+  const size_t stage = (size_t)FIT_BK * (f.bm + f.bn + 4) * sizeof(double);
+  return reduce ? std::max(stage, (size_t)f.bm * f.bn * sizeof(double)) : stage;
+}
+
+// Chunks of N columns: equal, at most `widest`, multiples of ni.
+void fit_columns(int64_t N, int ni, int widest, FitShape& f) {
+  f.nch = ceil_div(N, widest);
+  f.bn = ceil_div(ceil_div(N, f.nch), ni) * ni;
+}
+
+int fit_threads(const FitShape& f, int mi, int ni) {
+  return ceil_div((f.bm / mi) * (f.bn / ni), 32) * 32;
+}
+
+// A product: the tile rows and the K split are taken that leave the fullest SM
+// the least work, the CTAs (ceil(M / bm) nch S of bm bn K / S multiply-adds)
+// being dealt evenly.  8192 x 4096 at d = 72: 9.49 ms in 64 x 64 tiles of all K
+// (128 padded columns), 4.26 ms in 64 x 36 tiles and 8 slabs (1.13 TFLOP/s of
+// the 1.19 the FP64 units do); 1000 x 800 at d = 30: 990 us (16 CTAs) to 76 us.
+template <bool TRANS_A>
+cudaError_t fit_launch(const double* A, int64_t lda, const double* B, int64_t ldb, double* C,
+                       int64_t ldc, int64_t M, int64_t K, int64_t N, const int32_t* gate,
+                       cudaStream_t st) {
+  constexpr int MI = 4, NI = 2;
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  FitShape f{};
+  fit_columns(N, NI, FIT_BN, f);
+  const int64_t P = sm_count();
+  double best = 1e300;
+  for (int b = 16 * MI; b >= 4 * MI; b /= 2) {
+    for (int s = 1; s <= 8; s *= 2) {
+      if (s > 1 && K < (int64_t)64 * s) break;
+      const int64_t units = (int64_t)ceil_div(M, b) * f.nch * s;
+      // shorter tiles load more per multiply-add (measured at 8192 x 4096, d =
+      // 72, in 8 slabs: 4.26, 4.79 and 5.57 ms with 64, 32 and 16 rows); one CTA
+      // per SM waits for its loads (1000 x 800, d = 30: 184 us with 128 CTAs of
+      // 64 rows, 121 with 256 of 32)
+      const double cost = (double)((units + P - 1) / P) * b / s *
+                          (b == 16 * MI ? 1.0 : b == 8 * MI ? 1.11 : 1.3) *
+                          (units <= P ? 1.5 : 1.0);
+      if (cost < best * 0.999) {
+        best = cost;
+        f.bm = b;
+        f.S = s;
+      }
+    }
+  }
+  f.kslab = ((K + f.S - 1) / f.S + FIT_BK - 1) / FIT_BK * FIT_BK;
+  const size_t sm = fit_smem_bytes(f, f.S > 1);
+  auto kern = k_fit<TRANS_A, double, MI, NI, false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(ceil_div(M, f.bm) * f.S), f.nch);
+  cfg.blockDim = dim3(fit_threads(f, MI, NI));
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim = {(unsigned)f.S, 1, 1};
+  cfg.attrs = attr;
+  cfg.numAttrs = f.S > 1 ? 1 : 0;
+  e = cudaLaunchKernelEx(&cfg, kern, A, lda, B, ldb, C, ldc, M, K, N, f, gate);
+  count_launch();
+  return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
 // C[i][j] = sum_z P[z][i][j] in z order (deterministic), cast to TC.
+// sym: only the entries with j >= i were formed.
 template <typename TC>
 __global__ void k_reduce_partials(const double* __restrict__ P, int splits, int64_t M, int64_t N,
                                   TC* __restrict__ C, int64_t ldc,
-                                  const int32_t* __restrict__ gate) {
+                                  const int32_t* __restrict__ gate, bool sym = false) {
   if (gate != nullptr && *gate == 0) return;
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= M * N) return;
   const int64_t i = idx / N, j = idx % N;
+  if (sym && j < i) idx = j * N + i;
   double s = 0.0;  // split order, eight independent loads in flight
   int z = 0;
   for (; z + 8 <= splits; z += 8) {
@@ -177,6 +406,35 @@ __global__ void k_reduce_partials(const double* __restrict__ P, int splits, int6
   }
   for (; z < splits; ++z) s += P[(int64_t)z * M * N + idx];
   C[i * ldc + j] = Cvt<TC>::from(s);
+}
+
+// C = A^T B (FP64 sums; M x N small) in `splits` K slabs, or its upper
+// triangle's tiles mirrored when A = B: the square tiles' chunks fit N (one of
+// 30 columns at d = 30, five of 44 at d = 220), half of the off-diagonal work
+// is left out.
+template <typename T, typename TC>
+cudaError_t fit_partial(const void* A, int64_t lda, const void* B, int64_t ldb, void* C,
+                        int64_t ldc, int64_t M, int64_t K, int64_t N, int splits, double* partial,
+                        const int32_t* gate, cudaStream_t st) {
+  FitShape f{};
+  fit_columns(N, 2, FIT_BN_PART, f);
+  f.bm = f.bn;
+  f.nchm = ceil_div(M, f.bm);
+  f.sym = A == B && lda == ldb && M == N;
+  f.kslab = ((K + splits - 1) / splits + 15) / 16 * 16;
+  f.S = (int)((K + f.kslab - 1) / f.kslab);
+  const size_t sm = fit_smem_bytes(f, false);
+  const int pairs = f.sym ? f.nch * (f.nch + 1) / 2 : f.nchm * f.nch;
+  k_fit<true, T, 2, 2, true>
+      <<<dim3(pairs, f.S), fit_threads(f, 2, 2), sm, st>>>((const T*)A, lda, (const T*)B, ldb,
+                                                           partial, N, M, K, N, f, gate);
+  count_launch();
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_reduce_partials<TC><<<ceil_div(M * N, 256), 256, 0, st>>>(partial, f.S, M, N, (TC*)C, ldc, gate,
+                                                              f.sym);
+  count_launch();
+  return cudaGetLastError();
 }
 
 template <bool TRANS_A, typename TA, typename TB, typename TC, Mul MODE>
@@ -211,8 +469,8 @@ cudaError_t launch(const void* A, int64_t lda, const void* B, int64_t ldb, void*
 
 int tn_splits(int64_t M, int64_t K, int64_t N, int max_splits) {
   const int64_t tiles = (int64_t)ceil_div(M, BM) * ceil_div(N, BN);
-  int64_t s = (2 * 152 + tiles - 1) / tiles;        // about two CTAs per SM
-  const int64_t kmax = (K + 4 * BK - 1) / (4 * BK);  // at least 64 rows per slab
+  int64_t s = (4 * 152 + tiles - 1) / tiles;  // about four CTAs per SM
+  const int64_t kmax = (K + BK - 1) / BK;     // at least 16 rows per slab
   if (s > kmax) s = kmax;
   if (s > max_splits) s = max_splits;
   if (s < 1) s = 1;
@@ -230,7 +488,9 @@ cudaError_t simt_gemm_nn(Ty ta, Ty tb, Ty tc, Mul mul, const void* A, int64_t ld
   const int splits = 1;
   double* partial = nullptr;
   const int32_t* gate = nullptr;
-  RUQLP_DISPATCH(false, Ty::F64, Ty::F64, Ty::F64, Mul::F64, double, double, double)
+  if (ta == Ty::F64 && tb == Ty::F64 && tc == Ty::F64 && mul == Mul::F64)
+    return fit_launch<false>((const double*)A, lda, (const double*)B, ldb, (double*)C, ldc, M, K, N,
+                                                                     gate, st);
   RUQLP_DISPATCH(false, Ty::F32, Ty::F32, Ty::F32, Mul::F32, float, float, float)
   RUQLP_DISPATCH(false, Ty::BF16, Ty::F32, Ty::F32, Mul::F32, __nv_bfloat16, float, float)
   RUQLP_DISPATCH(false, Ty::BF16, Ty::BF16, Ty::F32, Mul::F32, __nv_bfloat16, __nv_bfloat16, float)
@@ -269,7 +529,15 @@ cudaError_t simt_gemm_tn(Ty ta, Ty tb, Ty tc, Mul mul, const void* A, int64_t ld
                          int64_t K, int64_t N, int splits, double* partial,
                          const int32_t* gate, cudaStream_t st, const int32_t* redo) {
   if (splits > 1 && partial == nullptr) return cudaErrorInvalidValue;
-  RUQLP_DISPATCH(true, Ty::F64, Ty::F64, Ty::F64, Mul::F64, double, double, double)
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  if (splits > 1 && mul == Mul::F64 && tc == Ty::F64 && ta == tb && ta != Ty::BF16)
+    return ta == Ty::F64 ? fit_partial<double, double>(A, lda, B, ldb, C, ldc, M, K, N, splits,
+                                                       partial, gate, st)
+                         : fit_partial<float, double>(A, lda, B, ldb, C, ldc, M, K, N, splits,
+                                                      partial, gate, st);
+  if (ta == Ty::F64 && tb == Ty::F64 && tc == Ty::F64 && mul == Mul::F64)
+    return fit_launch<true>((const double*)A, lda, (const double*)B, ldb, (double*)C, ldc, M, K, N,
+                                                                    gate, st);
   RUQLP_DISPATCH(true, Ty::F32, Ty::F32, Ty::F32, Mul::F32, float, float, float)
   RUQLP_DISPATCH(true, Ty::BF16, Ty::F32, Ty::F32, Mul::F32, __nv_bfloat16, float, float)
   RUQLP_DISPATCH(true, Ty::BF16, Ty::BF16, Ty::F32, Mul::F32, __nv_bfloat16, __nv_bfloat16, float)
