@@ -130,11 +130,12 @@ cudaError_t transpose_to_bf16(Ty ts, const void* src, int64_t lds, int64_t rows,
 
 // CSR products (k_csr.cu), values FP32 or BF16, dense operands FP32.
 // csr_validate ORs into *flag: 1 bad rowptr, 2 bad / unsorted / duplicate
-// column index.  csr_transpose builds the CSR of A^T (colptr n+1, rowidx and
+// column index, and counts the columns into scratch[0..n).  csr_transpose (after
+// it, with the same scratch) builds the CSR of A^T (colptr n+1, rowidx and
 // cvals nnz) with rows sorted inside each column (deterministic); scratch:
 // 2n ints; *flag |= 4 if a column has more than 1024 nonzeros.
 cudaError_t csr_validate(const int32_t* rowptr, const int32_t* colidx, int64_t m, int64_t n,
-                         int64_t nnz, int* flag, cudaStream_t st);
+                         int64_t nnz, int* flag, int32_t* scratch, cudaStream_t st);
 cudaError_t csr_transpose(Ty tv, const int32_t* rowptr, const int32_t* colidx, const void* vals,
                           int64_t m, int64_t n, int64_t nnz, int32_t* colptr, int32_t* rowidx,
                           void* cvals, int32_t* scratch, int* flag, cudaStream_t st);
@@ -311,6 +312,16 @@ __host__ __device__ inline F32Split f32_columns(int dp) {
   sp.w = ((dp + sp.nch - 1) / sp.nch + 15) / 16 * 16;
   return sp;
 }
+// A stage (K block) of the split X: three parts of [32 k][64 columns] BF16 boxes
+// with 128-byte swizzle; the byte offset of (k, column) within a part.
+constexpr uint32_t F32_BOX = F32_BK * 128;
+__host__ __device__ inline uint32_t f32_xstage(int w) {
+  return 3 * (uint32_t)((w + 63) / 64) * F32_BOX;
+}
+__host__ __device__ inline uint32_t f32_img_off(int k, int col) {
+  return (uint32_t)(col >> 6) * F32_BOX + (uint32_t)k * 128 +
+         ((uint32_t)(((col & 63) >> 3) ^ (k & 7)) << 4) + (uint32_t)((col & 7) * 2);
+}
 F32Split f32_split(int64_t rows, int64_t K, int64_t m, int64_t n, int d, int dp);
 bool f32_tc_supported(int64_t K);
 // out (ld ldo, dp columns written) = A X or A^T X, A m x n FP32 (ld lda), X
@@ -322,6 +333,11 @@ cudaError_t f32_gemm_tc(bool trans, const float* A, int64_t lda, int64_t m, int6
                         const float* X, int64_t ldx, int xcols, int d, int dp, float* out,
                         int64_t ldo, float* frag, void* img, DevStatus* st,
                         cudaStream_t stream);
+// out = A X with X given split (img, one column chunk: dp <= 224, K < 512 rows);
+// out may be A (lda = ldo): a tile's rows are read before they are written.
+// err: timeout word.
+cudaError_t f32_mul_img(const float* A, int64_t lda, int64_t M, int K, int dp, const void* img,
+                        float* out, int64_t ldo, int* err, cudaStream_t stream);
 // Bytes of the split X of a product over K rows (img above; null: every CTA
 // splits X itself, with the same result).
 size_t f32_img_bytes(int64_t K, int dp);

@@ -28,56 +28,97 @@ template <> __device__ __forceinline__ float val_f32<__nv_bfloat16>(__nv_bfloat1
 
 // flag bit 1: rowptr not a valid prefix (rowptr[0] != 0, decreasing, or
 // rowptr[m] != nnz); bit 2: column index out of range or not strictly
-// increasing inside a row.
+// increasing inside a row.  The valid columns are counted on the way (counts,
+// zeroed before): one warp per row, so the indices are read once, coalesced
+// (20M nonzeros: 185 us as a thread per row and a counting pass).
 __global__ void k_csr_validate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
-                               int64_t m, int64_t n, int64_t nnz, int* flag) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+                               int64_t m, int64_t n, int64_t nnz, int* flag,
+                               int32_t* __restrict__ counts) {
+  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (i > m) return;
-  if (i == 0 && rowptr[0] != 0) atomicOr(flag, 1);
+  if (i == 0 && lane == 0 && rowptr[0] != 0) atomicOr(flag, 1);
   if (i == m) {
-    if ((int64_t)rowptr[m] != nnz) atomicOr(flag, 1);
+    if (lane == 0 && (int64_t)rowptr[m] != nnz) atomicOr(flag, 1);
     return;
   }
   const int32_t a = rowptr[i], b = rowptr[i + 1];
-  if (b < a || a < 0 || (int64_t)b > nnz) { atomicOr(flag, 1); return; }
-  int32_t prev = -1;
-  for (int32_t e = a; e < b; ++e) {
-    const int32_t c = colidx[e];
-    if (c <= prev || (int64_t)c >= n) { atomicOr(flag, 2); return; }
-    prev = c;
+  if (b < a || a < 0 || (int64_t)b > nnz) {
+    if (lane == 0) atomicOr(flag, 1);
+    return;
   }
+  bool bad = false;
+  int32_t before = -1;  // the last index of the chunk before
+  for (int32_t e0 = a; e0 < b; e0 += 32) {
+    const bool in = e0 + lane < b;
+    const int32_t c = in ? colidx[e0 + lane] : 0x7fffffff;
+    int32_t prev = __shfl_up_sync(0xffffffffu, c, 1);
+    if (lane == 0) prev = before;
+    if (in) {
+      if (c <= prev || c < 0 || (int64_t)c >= n) bad = true;
+      else atomicAdd(&counts[c], 1);
+    }
+    before = __shfl_sync(0xffffffffu, c, 31);
+  }
+  if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(flag, 2);
 }
 
-__global__ void k_col_count(const int32_t* __restrict__ colidx, int64_t nnz, int32_t* counts) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nnz;
-       e += (int64_t)gridDim.x * blockDim.x)
-    atomicAdd(&counts[colidx[e]], 1);
-}
-
-// exclusive scan of counts[0..n) into ptr[0..n], one CTA of 1024 threads
-__global__ void __launch_bounds__(1024) k_scan(const int32_t* __restrict__ counts, int64_t n,
-                                               int32_t* __restrict__ ptr, int32_t* __restrict__ cursor) {
-  __shared__ int32_t part[1024];
-  const int t = threadIdx.x;
-  const int64_t per = (n + 1023) / 1024;
-  const int64_t a = t * per, b = min(n, a + per);
-  int32_t s = 0;
-  for (int64_t i = a; i < b; ++i) s += counts[i];
-  part[t] = s;
+// Exclusive scan of counts[0..n) into ptr[0..n]: block sums of 1024 counts,
+// then every block adds the sums before it and scans its own.
+constexpr int SCAN_BLOCK = 1024;
+__device__ __forceinline__ int32_t block_sum(int32_t v, int32_t* red) {  // 256 threads
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  for (int off = 1; off < 1024; off <<= 1) {  // inclusive scan of the parts
-    const int32_t v = (t >= off) ? part[t - off] : 0;
-    __syncthreads();
-    part[t] += v;
-    __syncthreads();
+  int32_t s = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) s += red[w];
+  __syncthreads();
+  return s;
+}
+__global__ void __launch_bounds__(256) k_scan_sums(const int32_t* __restrict__ counts, int64_t n,
+                                                   int32_t* __restrict__ sums) {
+  __shared__ int32_t red[8];
+  int32_t v = 0;
+  for (int q = 0; q < 4; ++q) {
+    const int64_t i = (int64_t)blockIdx.x * SCAN_BLOCK + q * 256 + threadIdx.x;
+    if (i < n) v += counts[i];
   }
-  int32_t run = (t == 0) ? 0 : part[t - 1];
-  for (int64_t i = a; i < b; ++i) {
-    ptr[i] = run;
-    cursor[i] = run;
-    run += counts[i];
+  v = block_sum(v, red);
+  if (threadIdx.x == 0) sums[blockIdx.x] = v;
+}
+__global__ void __launch_bounds__(256) k_scan(const int32_t* __restrict__ counts,
+                                              const int32_t* __restrict__ sums, int64_t n,
+                                              int32_t* __restrict__ ptr) {
+  __shared__ int32_t red[8];
+  int32_t v = 0;
+  for (int i = threadIdx.x; i < (int)blockIdx.x; i += 256) v += sums[i];
+  const int32_t base = block_sum(v, red);
+  const int64_t i0 = (int64_t)blockIdx.x * SCAN_BLOCK + 4 * threadIdx.x;
+  int32_t c[4], t = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    c[q] = i0 + q < n ? counts[i0 + q] : 0;
+    t += c[q];
   }
-  if (t == 1023) ptr[n] = part[1023];
+  int32_t run = t;  // inclusive scan of the threads' sums
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t x = __shfl_up_sync(0xffffffffu, run, o);
+    if (lane >= o) run += x;
+  }
+  if (lane == 31) red[w] = run;
+  __syncthreads();
+  run += base - t;
+  for (int k = 0; k < w; ++k) run += red[k];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (i0 + q < n) ptr[i0 + q] = run;
+    run += c[q];
+    if (i0 + q + 1 == n) ptr[n] = run;
+  }
 }
 
 template <typename TV>
@@ -95,9 +136,13 @@ __global__ void k_csc_scatter(const int32_t* __restrict__ rowptr, const int32_t*
   }
 }
 
-// Sort each column's (row, value) entries by row: one warp per column,
-// bitonic sort of up to 1024 entries in shared memory.  flag bit 4: a
-// column holds more than 1024 nonzeros.
+// Sort each column's (row, value) entries by row, one warp per column, up to
+// 1024 entries in shared memory (flag bit 4: a column holds more).  The rows
+// (distinct) are dealt to 32 buckets between the column's least and largest
+// row; an entry's place is its bucket's start plus the number of smaller rows
+// in the bucket (6 of 200 on average: 748 -> 80 us for 100000 columns against
+// the bitonic network, which stays for columns whose fullest bucket holds more
+// than 64).
 constexpr int SORT_MAX = 1024;
 template <typename TV>
 __global__ void __launch_bounds__(128)
@@ -105,6 +150,7 @@ k_csc_sort(const int32_t* __restrict__ colptr, int64_t n, int32_t* __restrict__ 
            TV* __restrict__ cvals, int* flag) {
   __shared__ int32_t keys[4][SORT_MAX];
   __shared__ TV sv[4][SORT_MAX];
+  __shared__ int32_t s_at[4][32];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t c = (int64_t)blockIdx.x * 4 + w;
   if (c >= n) return;
@@ -114,6 +160,58 @@ k_csc_sort(const int32_t* __restrict__ colptr, int64_t n, int32_t* __restrict__ 
   if (len > SORT_MAX) {
     if (lane == 0) atomicOr(flag, 4);
     return;
+  }
+  {
+    int32_t lo = 0x7fffffff, hi = 0;
+    for (int i = lane; i < len; i += 32) {
+      const int32_t k = rowidx[a + i];
+      lo = min(lo, k);
+      hi = max(hi, k);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    const float scale = 32.f / ((float)(hi - lo) + 1.f);  // (monotone in the row)
+    auto bucket = [&](int32_t k) { return min(31, (int)((float)(k - lo) * scale)); };
+    s_at[w][lane] = 0;
+    __syncwarp();
+    for (int i = lane; i < len; i += 32) atomicAdd(&s_at[w][bucket(rowidx[a + i])], 1);
+    __syncwarp();
+    const int cnt = s_at[w][lane];
+    int end = cnt;  // inclusive scan
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, end, o);
+      if (lane >= o) end += x;
+    }
+    if (__reduce_max_sync(0xffffffffu, cnt) <= 64) {
+      s_at[w][lane] = end - cnt;
+      __syncwarp();
+      for (int i0 = 0; i0 < len; i0 += 32) {  // by bucket, in any order
+        const int i = i0 + lane;
+        if (i < len) {
+          const int32_t k = rowidx[a + i];
+          const int pos = atomicAdd(&s_at[w][bucket(k)], 1);
+          keys[w][pos] = k;
+          sv[w][pos] = cvals[a + i];
+        }
+      }
+      __syncwarp();
+      for (int i0 = 0; i0 < len; i0 += 32) {
+        const int i = i0 + lane;
+        const int32_t k = i < len ? keys[w][i] : lo;
+        const int bk = bucket(k);
+        const int e1 = __shfl_sync(0xffffffffu, end, bk);
+        const int e0 = e1 - __shfl_sync(0xffffffffu, cnt, bk);
+        if (i < len) {
+          int r = e0;
+          for (int j = e0; j < e1; ++j) r += keys[w][j] < k ? 1 : 0;
+          rowidx[a + r] = k;
+          cvals[a + r] = sv[w][i];
+        }
+      }
+      return;
+    }
+    __syncwarp();
   }
   int p2 = 1;
   while (p2 < len) p2 <<= 1;
@@ -219,8 +317,11 @@ cudaError_t add_rows_f32(float* out, int64_t ldo, const float* t, int64_t ldt, i
 }
 
 cudaError_t csr_validate(const int32_t* rowptr, const int32_t* colidx, int64_t m, int64_t n,
-                         int64_t nnz, int* flag, cudaStream_t st) {
-  k_csr_validate<<<ceil_div(m + 1, 256), 256, 0, st>>>(rowptr, colidx, m, n, nnz, flag);
+                         int64_t nnz, int* flag, int32_t* scratch, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(scratch, 0, (size_t)n * sizeof(int32_t), st);
+  if (e != cudaSuccess) return e;
+  k_csr_validate<<<ceil_div((m + 1) * 32, 256), 256, 0, st>>>(rowptr, colidx, m, n, nnz, flag,
+                                                              scratch);
   count_launch();
   return cudaGetLastError();
 }
@@ -228,16 +329,17 @@ cudaError_t csr_validate(const int32_t* rowptr, const int32_t* colidx, int64_t m
 cudaError_t csr_transpose(Ty tv, const int32_t* rowptr, const int32_t* colidx, const void* vals,
                           int64_t m, int64_t n, int64_t nnz, int32_t* colptr, int32_t* rowidx,
                           void* cvals, int32_t* scratch, int* flag, cudaStream_t st) {
-  int32_t* counts = scratch;        // n
+  int32_t* counts = scratch;        // n, from csr_validate
   int32_t* cursor = scratch + n;    // n
-  cudaError_t e = cudaMemsetAsync(counts, 0, (size_t)n * sizeof(int32_t), st);
-  if (e != cudaSuccess) return e;
-  if (nnz > 0) {
-    k_col_count<<<1216, 256, 0, st>>>(colidx, nnz, counts);
-    count_launch();
-  }
-  k_scan<<<1, 1024, 0, st>>>(counts, n, colptr, cursor);
+  const int nblk = ceil_div(n, SCAN_BLOCK);
+  k_scan_sums<<<nblk, 256, 0, st>>>(counts, n, cursor);
   count_launch();
+  k_scan<<<nblk, 256, 0, st>>>(counts, cursor, n, colptr);
+  count_launch();
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(cursor, colptr, (size_t)n * sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
+  if (e != cudaSuccess) return e;
   const int gw = ceil_div(m * 32, 256);
   const int gs = ceil_div(n, 4);
   if (tv == Ty::F32) {

@@ -576,7 +576,8 @@ ruqlp_status prepare_csr(ruqlp_ctx* h, const Layout& Lo, Job& J) {
   int* flag = &h->status->invalid;
   // the structure is checked (and the result read) before any kernel indexes
   // with the column indices
-  CK(csr_validate(J.rowptr, J.colidx, J.m, J.n, J.nnz, flag, h->stream));
+  CK(csr_validate(J.rowptr, J.colidx, J.m, J.n, J.nnz, flag, (int32_t*)(base + Lo.cscratch),
+                  h->stream));
   CK(cudaMemcpyAsync(h->status_host, h->status, sizeof(DevStatus), cudaMemcpyDeviceToHost,
                      h->stream));
   CK(cudaStreamSynchronize(h->stream));
