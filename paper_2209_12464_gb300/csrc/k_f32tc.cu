@@ -5,8 +5,8 @@
 //   out[n x dp] = A^T[n x m] X     (A MN-major)
 //
 // Every FP32 value is split on the fly into three BF16 parts, x = h + m + l
-// exactly (h rounded to nearest, m and l the next bits: 8 + 8 + 7 significant
-// bits), and a x is formed as the six part products
+// exactly (h and m rounded to nearest, l the rest: 8 + 8 + 7 significant bits),
+// and a x is formed as the six part products
 //   l h + h l + m m + m h + h m + h h
 // (the dropped m l, l m, l l are below 2^-25 |a x|), accumulated in FP32.
 //
@@ -63,12 +63,14 @@ constexpr int FT_THREADS = 512;
 constexpr int FT_CT = 256;                       // converter threads
 constexpr int FT_CW = FT_CT / 32;                // converter warps
 constexpr uint32_t FT_APART = F32_BM * F32_BK * 2;  // one part of an A block
-constexpr uint32_t FT_BOX = F32_BK * 128;        // [32 k][64 columns] BF16
+constexpr uint32_t FT_BOX = F32_BOX;
 constexpr int FT_NA = 2;                         // stages of split A blocks
 constexpr int FT_NC = F32_WMAX / 16;             // accumulator chunks per thread
 constexpr int FT_XV = F32_BK * F32_WMAX / 4 / FT_CT;  // X float4s per thread and block
 constexpr int FT_AHEAD = 4;                      // A blocks in flight per CTA
 constexpr uint32_t FT_RAW = F32_BM * F32_BK * 4; // one raw A block
+constexpr int FT_SP = 20;                        // epilogue staging pitch (floats)
+constexpr uint32_t FT_STG = 4 * 32 * FT_SP * 4;
 constexpr int FT_REG_CTL = 56, FT_REG_CONV = 104, FT_REG_EPI = 248;
 
 // One unit of work: a 128-row output tile, columns [col0, col0 + w), K blocks
@@ -98,12 +100,9 @@ struct FtParams {
   float* frag;
   int d, xcols, dp, vec;
   F32Split sp;
-  DevStatus* st;
+  DevStatus* st;  // null: no range notes
+  int* err;
 };
-
-__host__ __device__ inline uint32_t ft_xstage(int w) {
-  return 3 * (uint32_t)((w + 63) / 64) * FT_BOX;
-}
 
 __device__ __forceinline__ void ft_columns(const F32Split& sp, int item, int dp, FtUnit& u) {
   u.tile = item / sp.nch;
@@ -143,7 +142,7 @@ struct FtSingle {
     ft_columns(sp, item, p->dp, u);
     u.img = p->img == nullptr
                 ? nullptr
-                : p->img + (int64_t)(u.col0 / sp.w) * sp.KB * ft_xstage(sp.w);
+                : p->img + (int64_t)(u.col0 / sp.w) * sp.KB * f32_xstage(sp.w);
     u.kb0 = (int)((int64_t)sp.KB * s / S);
     u.kb1 = (int)((int64_t)sp.KB * (s + 1) / S);
     if (S == 1) {
@@ -186,7 +185,7 @@ struct FtBatch {
     ft_columns(sp, e.item, b.dp, u);
     u.img = b.Ximg == nullptr
                 ? nullptr
-                : (const uint8_t*)b.Ximg + (int64_t)(u.col0 / sp.w) * KB * ft_xstage(sp.w);
+                : (const uint8_t*)b.Ximg + (int64_t)(u.col0 / sp.w) * KB * f32_xstage(sp.w);
     u.kb0 = (int)((int64_t)KB * e.s / e.S);
     u.kb1 = (int)((int64_t)KB * (e.s + 1) / e.S);
     if (e.S == 1) {
@@ -200,33 +199,11 @@ struct FtBatch {
   }
 };
 
-// Packed FP32 pairs (one instruction for two values).
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
-  float2 r;
-  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
-      "sub.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
-      : "=f"(r.x), "=f"(r.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return r;
-}
-
 __device__ __forceinline__ void add2(float& a, float& b, float x, float y) {
   asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%0, %1};\n\tmov.b64 y, {%2, %3};\n\t"
       "add.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
       : "+f"(a), "+f"(b)
       : "f"(x), "f"(y));
-}
-
-// Two values as h + m + l, each part packed as a BF16 pair.
-__device__ __forceinline__ void split3(float2 x, uint32_t& h, uint32_t& m, uint32_t& l) {
-  const uint32_t hx = (__float_as_uint(x.x) + 0x8000u) & 0xFFFF0000u;
-  const uint32_t hy = (__float_as_uint(x.y) + 0x8000u) & 0xFFFF0000u;
-  h = __byte_perm(hx, hy, 0x7632);
-  const float2 r1 = sub2(x, make_float2(__uint_as_float(hx), __uint_as_float(hy)));
-  m = __byte_perm(__float_as_uint(r1.x), __float_as_uint(r1.y), 0x7632);
-  const float2 r2 = sub2(r1, make_float2(__uint_as_float(__float_as_uint(r1.x) & 0xFFFF0000u),
-                                         __uint_as_float(__float_as_uint(r1.y) & 0xFFFF0000u)));
-  l = __byte_perm(__float_as_uint(r2.x), __float_as_uint(r2.y), 0x7632);
 }
 
 // The three parts of four consecutive values at shared address a, a + pitch,
@@ -243,7 +220,7 @@ __device__ __forceinline__ void put4(uint32_t a, uint32_t pitch, const float4& v
 }
 
 __device__ __forceinline__ void note(DevStatus* st, int32_t bits) {
-  if ((*(volatile int32_t*)&st->range & bits) != bits) atomicOr(&st->range, bits);
+  if (st != nullptr && (*(volatile int32_t*)&st->range & bits) != bits) atomicOr(&st->range, bits);
 }
 // Magnitudes met: the largest |x| (NaN kept) and the smallest nonzero one as
 // twice its bits less one (zero wraps to the top, so it never counts as small).
@@ -303,9 +280,7 @@ struct XPlace {
     c = (lane & 7) * 4;
   }
   __device__ __forceinline__ uint32_t off(int q) const {
-    const int col = c + 32 * q;
-    return (uint32_t)(col >> 6) * FT_BOX + (uint32_t)k * 128 +
-           ((uint32_t)(((col & 63) >> 3) ^ (k & 7)) << 4) + (uint32_t)((col & 7) * 2);
+    return f32_img_off(k, c + 32 * q);
   }
 };
 
@@ -316,7 +291,7 @@ __device__ __forceinline__ void split_block(const float* X, int64_t ldx, int64_t
                                             int xcols, int kb, int col0, int w, uint8_t* img, DevStatus* st) {
   const XPlace xp(threadIdx.x);
   const int64_t row = (int64_t)kb * F32_BK + xp.k;
-  const uint32_t part = ft_xstage(w) / 3;
+  const uint32_t part = f32_xstage(w) / 3;
   Range rx;
   for (int q = 0; 32 * q < (w + 63) / 64 * 64; ++q) {
     const int c = xp.c + 32 * q;
@@ -338,7 +313,7 @@ __device__ __forceinline__ void split_block(const float* X, int64_t ldx, int64_t
 __global__ void __launch_bounds__(FT_CT) k_f32_split(const __grid_constant__ FtParams p) {
   pdl_launch();
   pdl_wait();
-  const uint32_t xs = ft_xstage(p.sp.w);
+  const uint32_t xs = f32_xstage(p.sp.w);
   split_block(p.X, p.ldx, p.K, p.d, p.xcols, blockIdx.x, blockIdx.y * p.sp.w, p.sp.w,
               const_cast<uint8_t*>(p.img) + ((int64_t)blockIdx.y * p.sp.KB + blockIdx.x) * xs,
               p.st);
@@ -354,7 +329,7 @@ __global__ void __launch_bounds__(FT_CT) k_bf32_split(const BMat* __restrict__ T
   for (int x = blockIdx.x; x < KB * sp.nch; x += gridDim.x) {
     const int ch = x / KB, kb = x - ch * KB;
     split_block(bbuf(b, src), b.dp, K, b.d, b.dp, kb, ch * sp.w, sp.w,
-                (uint8_t*)b.Ximg + (int64_t)x * ft_xstage(sp.w), b.status);
+                (uint8_t*)b.Ximg + (int64_t)x * f32_xstage(sp.w), b.status);
   }
 }
 
@@ -366,13 +341,15 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - raw);
-  // shared memory: split A stages, split X stages, raw A blocks, barriers
+  // shared memory: split A stages, split X stages, raw A blocks, the epilogue's
+  // staging, barriers
   // fa / ea (A full: converter warps; empty: MMA commit), fx / ex (X), tfull,
   // tempty, drain; then the TMEM address
-  const uint32_t xstage = ft_xstage(wmax), xpart = xstage / 3;
+  const uint32_t xstage = f32_xstage(wmax), xpart = xstage / 3;
   const uint32_t x_base = base + FT_NA * 3 * FT_APART;
   const uint32_t raw_base = x_base + NX * xstage;
-  const uint32_t bar = raw_base + FT_AHEAD * FT_RAW;
+  const uint32_t stg_base = raw_base + FT_AHEAD * FT_RAW;
+  const uint32_t bar = stg_base + FT_STG;
   auto fa = [&](int i) { return bar + 8u * i; };
   auto ea = [&](int i) { return bar + 8u * (FT_NA + i); };
   auto fx = [&](int i) { return bar + 8u * (2 * FT_NA + i); };
@@ -472,7 +449,7 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
       uint32_t ph = 1;
       for (int i = 0; i < nunits && ok; ++i) {
         const FtUnit u = w.get(i);
-        const uint32_t bytes = ft_xstage(u.xw);
+        const uint32_t bytes = f32_xstage(u.xw);
         const uint32_t part = bytes / 3;
         const uint8_t* src = u.img + (int64_t)u.kb0 * bytes;
         for (int kb = u.kb0; kb < u.kb1; ++kb) {
@@ -635,7 +612,7 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(FT_REG_EPI));
     // ---------------- epilogue ----------------
     const int g = warp & 3;  // TMEM lane quarter of this warp
-    const int row = g * 32 + lane;
+    float* const stg = (float*)(base_ptr + (stg_base - base)) + g * 32 * FT_SP;
     const uint32_t lanes = (uint32_t)(g * 32) << 16;
     bool ok = true;
     int it = 0;
@@ -667,23 +644,32 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
         if (lane == 0) mbar_arrive(tempty(a));
       }
       if (!ok) break;
-      if ((int64_t)u.tile * F32_BM + row < u.rows) {
-        float* dst = u.out + (int64_t)row * u.ldo;
-        float least = 1.f;
+      // 16 columns at a time through a staging block, so that a store covers
+      // whole 64-byte row segments (a lane storing its own row takes 32 of the
+      // L1's cycles per instruction: 3600 clocks a tile at 112 columns)
+      const int left = (int)min((int64_t)F32_BM, u.rows - (int64_t)u.tile * F32_BM) - g * 32;
+      float least = 1.f;
 #pragma unroll
-        for (int c = 0; c < FT_NC; ++c) {
-          if (c * 16 >= u.w) break;
-          float4* d4 = reinterpret_cast<float4*>(dst + c * 16);
+      for (int c = 0; c < FT_NC; ++c) {
+        if (c * 16 >= u.w) break;
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            d4[j] = make_float4(acc[c][4 * j], acc[c][4 * j + 1], acc[c][4 * j + 2],
-                                acc[c][4 * j + 3]);
+        for (int j = 0; j < 4; ++j)
+          *reinterpret_cast<float4*>(stg + lane * FT_SP + 4 * j) = make_float4(
+              acc[c][4 * j], acc[c][4 * j + 1], acc[c][4 * j + 2], acc[c][4 * j + 3]);
+        __syncwarp();
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (u.col0 + c * 16 + j < u.d) least = fminf(least, fabsf(acc[c][j]));
+        for (int r = 0; r < 4; ++r) {
+          const int rr = r * 8 + (lane >> 2), cc = (lane & 3) * 4;
+          if (rr < left)
+            *reinterpret_cast<float4*>(u.out + (int64_t)(g * 32 + rr) * u.ldo + c * 16 + cc) =
+                *reinterpret_cast<const float4*>(stg + rr * FT_SP + cc);
         }
-        if (least < 8.470329e-22f) note(u.st, RANGE_TINY);  // 2^-70
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (u.col0 + c * 16 + j < u.d) least = fminf(least, fabsf(acc[c][j]));
       }
+      if (lane < left && least < 8.470329e-22f) note(u.st, RANGE_TINY);  // 2^-70
     }
     if (!ok) *abort_flag = 1;
   }
@@ -700,7 +686,7 @@ template <bool TRANS, bool IMG>
 __global__ void __launch_bounds__(FT_THREADS, 1)
 k_f32_tc(const __grid_constant__ FtParams p, int stages) {
   const FtSingle w{&p};
-  ft_body<TRANS, IMG>(w, stages, p.sp.w, &p.st->timeout);
+  ft_body<TRANS, IMG>(w, stages, p.sp.w, p.err);
 }
 
 template <bool TRANS, bool IMG>
@@ -761,7 +747,7 @@ __global__ void __launch_bounds__(256) k_bf32_fixup(const F32Tile* __restrict__ 
 }
 
 size_t ft_smem(int nx, int w) {
-  return 1024 + FT_NA * 3 * FT_APART + FT_AHEAD * FT_RAW + (size_t)nx * ft_xstage(w) +
+  return 1024 + FT_NA * 3 * FT_APART + FT_AHEAD * FT_RAW + FT_STG + (size_t)nx * f32_xstage(w) +
          8 * (2 * FT_NA + 2 * nx + 5) + 16;
 }
 // X stages: as many as fit (2 at 224 columns), at most 6.
@@ -809,8 +795,11 @@ F32Split f32_split(int64_t rows, int64_t K, int64_t m, int64_t n, int d, int dp)
 // Whether a product over K rows runs on the tensor cores.  The CUDA-core
 // kernel takes 47 us + 0.115 us K per call (its 64 x 64 tiles walk K one after
 // another), this one 58 us + 0.035 us K with its three launches: they meet near
-// K = 140 (256 x 256, d = 72: 72 against 58 us; 128 x 128, d = 30: 61 against 63).
-bool f32_tc_supported(int64_t K) { return K >= 192; }
+// K = 140 (256 x 256, d = 72: 72 against 58 us; 128 x 128, d = 30: 61 against
+// 63; 64 x 64: 49 against 59).  The line is at 128 because a batch, which pays
+// the launches anyway, gains from every item (a batch of 64: 1750 us with the
+// items of K < 192 on the CUDA cores, 1640 without).
+bool f32_tc_supported(int64_t K) { return K >= 128; }
 
 cudaError_t f32_gemm_tc(bool trans, const float* A, int64_t lda, int64_t m, int64_t n,
                         const float* X, int64_t ldx, int xcols, int d, int dp, float* out,
@@ -835,6 +824,7 @@ cudaError_t f32_gemm_tc(bool trans, const float* A, int64_t lda, int64_t m, int6
   p.vec = (lda & 3) == 0 && ((uintptr_t)A & 15) == 0;
   p.sp = f32_split(p.rows, p.K, m, n, d, dp);
   p.st = st;
+  p.err = &st->timeout;
   const int stages = ft_stages(p.sp.w);
   const size_t smem = ft_smem(stages, p.sp.w);
   auto kern = img ? (trans ? k_f32_tc<true, true> : k_f32_tc<false, true>)
@@ -856,9 +846,35 @@ cudaError_t f32_gemm_tc(bool trans, const float* A, int64_t lda, int64_t m, int6
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
+cudaError_t f32_mul_img(const float* A, int64_t lda, int64_t M, int K, int dp, const void* img,
+                        float* out, int64_t ldo, int* err, cudaStream_t stream) {
+  if ((ldo & 3) || ((uintptr_t)out & 15) || K >= 512 || dp > F32_WMAX) return cudaErrorInvalidValue;
+  FtParams p{};
+  p.A = A;
+  p.lda = lda;
+  p.rows = M;
+  p.K = K;
+  p.img = (const uint8_t*)img;
+  p.out = out;
+  p.ldo = ldo;
+  p.d = K;
+  p.dp = dp;
+  p.vec = (lda & 3) == 0 && ((uintptr_t)A & 15) == 0;
+  p.sp = f32_split(M, K, M, K, K, dp);  // (one slab: K < 512)
+  p.err = err;
+  const int stages = ft_stages(p.sp.w);
+  const size_t smem = ft_smem(stages, p.sp.w);
+  cudaError_t e = ft_prepare(k_f32_tc<false, true>, smem);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(k_f32_tc<false, true>, dim3(p.sp.full_waves > 0 ? p.sp.P : p.sp.tail),
+                 dim3(FT_THREADS), smem, stream, p, stages);
+  count_launch();
+  return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
 size_t f32_img_bytes(int64_t K, int dp) {
   const F32Split sp = f32_columns(dp);
-  return (size_t)sp.nch * ceil_div(K, F32_BK) * ft_xstage(sp.w);
+  return (size_t)sp.nch * ceil_div(K, F32_BK) * f32_xstage(sp.w);
 }
 
 void f32_tiles(int mat, const F32Split& sp, std::vector<F32Tile>& list,

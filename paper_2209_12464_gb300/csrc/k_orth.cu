@@ -178,13 +178,37 @@ k_trsm(const T* __restrict__ Y, int64_t ldy, const T* __restrict__ R, T* __restr
   }
 }
 
+// Four columns per thread, with vector loads and stores where the rows of both
+// sides start on them (vec), and 32-bit index arithmetic below 2^31 groups
+// (20000 x 220 FP32: 12.9 us with one element and a 64-bit division per thread).
+template <typename T> struct alignas(4 * sizeof(T)) Quad { T v[4]; };
 template <typename TS, typename TD>
 __global__ void k_copy_cast(const TS* __restrict__ src, int64_t lds, TD* __restrict__ dst,
-                            int64_t ldd, int64_t rows, int64_t cols) {
+                            int64_t ldd, int64_t rows, int cols, bool vec) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= rows * cols) return;
-  const int64_t i = idx / cols, j = idx % cols;
-  dst[i * ldd + j] = Cvt<TD>::from(src[i * lds + j]);
+  const int g = (cols + 3) / 4;
+  int64_t i;
+  int j;
+  if (rows * g < (int64_t)1 << 31) {
+    const uint32_t q = (uint32_t)idx / (uint32_t)g;
+    i = q;
+    j = (int)((uint32_t)idx - q * (uint32_t)g) * 4;
+  } else {
+    i = idx / g;
+    j = (int)(idx - i * g) * 4;
+  }
+  if (i >= rows) return;
+  const TS* s = src + i * lds + j;
+  TD* o = dst + i * ldd + j;
+  if (vec && j + 4 <= cols) {
+    const Quad<TS> x = *reinterpret_cast<const Quad<TS>*>(s);
+    Quad<TD> y;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) y.v[u] = Cvt<TD>::from(x.v[u]);
+    *reinterpret_cast<Quad<TD>*>(o) = y;
+  } else {
+    for (int u = 0; u < 4 && j + u < cols; ++u) o[u] = Cvt<TD>::from(s[u]);
+  }
 }
 
 // dst = h + bf16(v - h), h = bf16(v): v rounded to the sum of its two BF16
@@ -302,12 +326,13 @@ cudaError_t round2_bf16_2d(Ty ts, const void* src, int64_t lds, float* dst, int6
 
 cudaError_t copy_cast_2d(Ty ts, const void* src, int64_t lds, Ty td, void* dst, int64_t ldd,
                          int64_t rows, int64_t cols, cudaStream_t st) {
-  const int64_t tot = rows * cols;
-  if (tot <= 0) return cudaSuccess;
-  const int grid = ceil_div(tot, 256);
+  if (rows <= 0 || cols <= 0) return cudaSuccess;
+  const int grid = ceil_div(rows * ((cols + 3) / 4), 256);
+  const size_t as = 4 * ty_size(ts), ad = 4 * ty_size(td);
+  const bool vec = lds % 4 == 0 && ldd % 4 == 0 && (uintptr_t)src % as == 0 && (uintptr_t)dst % ad == 0;
 #define RUQLP_CC(TS_, TD_, CS, CD)                                                           \
   if (ts == TS_ && td == TD_) {                                                              \
-    k_copy_cast<CS, CD><<<grid, 256, 0, st>>>((const CS*)src, lds, (CD*)dst, ldd, rows, cols); \
+    k_copy_cast<CS, CD><<<grid, 256, 0, st>>>((const CS*)src, lds, (CD*)dst, ldd, rows, (int)cols, vec); \
     count_launch();                                                                          \
     return cudaGetLastError();                                                               \
   }

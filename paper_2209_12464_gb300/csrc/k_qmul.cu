@@ -91,7 +91,9 @@ constexpr int TI_STRIPS = TB / TI_W;    // strips per 32-column block
 // n = 32 J + W h .. of St[3][dp][KPX] (K padded to KPX).  Every tile the
 // column needs (R_IK for I < K <= J, S_KK for K <= J) is loaded at once;
 // acc_I is accumulated in the slot of S_IJ and turned into S_IJ in place.
-template <int KPX>
+// IMG: instead, the parts go to the image of the FP32 product's X stages
+// (f32_img_off; K padded to 32 nb).
+template <int KPX, bool IMG = false>
 __device__ __forceinline__ void trinv_body(const float* __restrict__ tiles, int d, int dp, int J,
                                            int h, __nv_bfloat16* __restrict__ St, float* sm) {
   constexpr int W = TI_W, RI = W / 4, RS = 128 / W;
@@ -170,6 +172,25 @@ __device__ __forceinline__ void trinv_body(const float* __restrict__ tiles, int 
     }
     __syncthreads();
   }
+  if (IMG) {
+    const int n = J * TB + h * W;
+    const uint32_t part = f32_xstage(dp) / 3;
+    for (int k = t; n < dp && k < nb * TB; k += TI_THREADS) {
+      const int kb = k / TB;
+      float v[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        v[c] = (kb <= J && k < d && n + c < d) ? Scol[(size_t)kb * TILE_F + (k % TB) * TP + h * W + c]
+                                               : 0.f;
+      uint32_t hp[2], mp[2], lp[2];
+      split3_bf16x4(v, hp, mp, lp);
+      uint8_t* o = (uint8_t*)St + (size_t)kb * 3 * part + f32_img_off(k % TB, n);
+      *reinterpret_cast<uint2*>(o) = make_uint2(hp[0], hp[1]);
+      *reinterpret_cast<uint2*>(o + part) = make_uint2(mp[0], mp[1]);
+      *reinterpret_cast<uint2*>(o + 2 * part) = make_uint2(lp[0], lp[1]);
+    }
+    return;
+  }
   // St[p][n][k] = part p of S[k][n], n = 32 J + c: lane = k within a
   // 32-row block, so a warp writes 64 contiguous bytes per row n
   for (int e = warp; e < W * (KPX / TB); e += nw) {
@@ -191,10 +212,12 @@ __device__ __forceinline__ void trinv_body(const float* __restrict__ tiles, int 
 
 // grid = TI_STRIPS nb CTAs (block column J = blockIdx.x / TI_STRIPS, strip
 // blockIdx.x % TI_STRIPS), S^T parts K-padded to 256.
+template <bool IMG>
 __global__ void __launch_bounds__(TI_THREADS)
 k_trinv(const float* __restrict__ tiles, int d, int dp, __nv_bfloat16* __restrict__ St) {
+  static_assert(TI_W == 4, "the image takes four columns at a time");
   extern __shared__ __align__(16) float sm[];
-  trinv_body<KP>(tiles, d, dp, blockIdx.x / TI_STRIPS, blockIdx.x % TI_STRIPS, St, sm);
+  trinv_body<KP, IMG>(tiles, d, dp, blockIdx.x / TI_STRIPS, blockIdx.x % TI_STRIPS, St, sm);
 }
 
 // Batched: grid (TI_STRIPS x block columns, items); item list[blockIdx.y] of the table,
@@ -219,6 +242,12 @@ constexpr uint32_t QM_ASTAGE = 3 * QM_APART;     // 48 KB
 constexpr uint32_t QM_BPART = 256 * 128;         // B part: [256 rows][64 BF16], 32 KB
 constexpr uint32_t QM_BBOX = 64 * 128;           // one TMA box of a part: 64 rows, 8 KB
 constexpr uint32_t QM_B = 3 * QM_BPART;          // 96 KB
+// dp <= 128: both chunks' S parts (9 boxes, 72 KB) stay resident instead of
+// being loaded again for every sub-tile: chunk 0's part q at 2 q boxes, chunk
+// 1's at 6 + q boxes
+__device__ __forceinline__ uint32_t qm_res_off(int c, int q) {
+  return (c == 0 ? 2u * q : 6u + q) * QM_BBOX;
+}
 constexpr int QM_SP = 20;                        // epilogue staging pitch (floats)
 constexpr uint32_t QM_STG = QM_CONV * 32 * QM_SP * 4;  // 20 KB
 constexpr uint32_t QM_BAR = 2 * QM_ASTAGE + QM_B + QM_STG;
@@ -301,6 +330,7 @@ k_qmul_tc(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ QmPar
 
   const int dp = p.dp, d = p.d;
   const int nsteps = (dp + 63) / 64;  // K chunks
+  const bool res = nsteps <= 2;       // S stays resident
   // this CTA's rows [r_begin, r_end), in groups of gs (1 or 2) 128-row
   // sub-tiles.  gs = 2: sub-tile s uses A stage s and accumulator s.  gs = 1:
   // the steps alternate between the A stages and the groups between the
@@ -326,7 +356,16 @@ k_qmul_tc(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ QmPar
       const uint64_t pol = policy_evict_last();
       bool pending = false;
       uint32_t pend_par = 0;
-      for (int j = 0; j < total; ++j) {
+      if (res && total > 0) {  // S once, for all of this CTA's sub-tiles
+        mbar_expect_tx(b_full, 3u * (uint32_t)(nsteps == 1 ? (dp + 63) / 64 : 3) * QM_BBOX);
+        for (int c = 0; c < nsteps; ++c)
+          for (int q = 0; q < 3; ++q)
+            for (int b = 0; b < (dp - 64 * c + 63) / 64; ++b)
+              tma_load_2d(sB + qm_res_off(c, q) + b * QM_BBOX, &tmS, b_full, 64 * c,
+                          q * dp + 64 * c + 64 * b, pol);
+        pending = true;
+      }
+      for (int j = 0; j < total && !res; ++j) {
         const int c = j % nsteps;
         const int nbox = (dp - 64 * c + 63) / 64;  // 64-row boxes per part
         if (j >= 1 && !mbar_wait(b_empty, (uint32_t)((j - 1) & 1), abort_flag)) {
@@ -361,7 +400,7 @@ k_qmul_tc(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ QmPar
         tc_fence_after();
         for (int c = 0; c < nsteps; ++c) {
           const int j = g * nsteps + c;
-          if (!mbar_wait(b_full, (uint32_t)(j & 1), abort_flag)) {
+          if (!mbar_wait(b_full, res ? 0u : (uint32_t)(j & 1), abort_flag)) {
             ok = false;
             break;
           }
@@ -381,7 +420,8 @@ k_qmul_tc(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ QmPar
 #pragma unroll
               for (int q = 0; q < 6; ++q) {
                 const uint64_t ad = ad0 + (uint64_t)((pa[q] * QM_APART + kk * 32) >> 4);
-                const uint64_t bd = bd0 + (uint64_t)((pb[q] * QM_BPART + kk * 32) >> 4);
+                const uint32_t bo = res ? qm_res_off(c, pb[q]) : pb[q] * QM_BPART;
+                const uint64_t bd = bd0 + (uint64_t)((bo + kk * 32) >> 4);
                 mma_bf16(dcol, ad, bd, id, (c > 0 || kk > 0 || q > 0) ? 1u : 0u);
               }
             }
@@ -389,7 +429,7 @@ k_qmul_tc(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ QmPar
             if (c == nsteps - 1) mma_commit(acc_full(set));
           }
           if (!ok) break;
-          mma_commit(b_empty);
+          if (!res) mma_commit(b_empty);
         }
       }
       if (!ok) s_abort = 1;
@@ -574,14 +614,22 @@ cudaError_t qmul_tc(const float* Y, int64_t ldy, const float* tiles, int64_t M, 
   const int dp = (d + 15) / 16 * 16;
   const int nb = (d + TB - 1) / TB;
   const size_t ti_smem = (size_t)(nb + nb * (nb - 1) / 2 + nb + 4) * TILE_F * sizeof(float);
+  // Without the transposed BF16 copy, narrow Q = Y S is an FP32 product
+  // (k_f32tc.cu), whose load ring and separate epilogue warps keep more of Y in
+  // flight (200000 x 110: 9 us less per pass, with a third of the rounding
+  // error); at 20000 x 220 its 157 tiles make two rounds over 152 SMs (40 us
+  // against 28 with k_qmul_tc's equal ranges), so wider Y stays here
+  const bool plain = Bt == nullptr && dp <= 128 && f32_img_bytes(d, dp) <= qmul_st_bytes(d);
+  auto trinv = plain ? k_trinv<true> : k_trinv<false>;
   cudaError_t e =
-      cudaFuncSetAttribute(k_trinv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ti_smem);
+      cudaFuncSetAttribute(trinv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ti_smem);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(k_trinv, dim3(TI_STRIPS * nb), dim3(TI_THREADS), ti_smem, st, tiles, d, dp,
+  e = launch_pdl(trinv, dim3(TI_STRIPS * nb), dim3(TI_THREADS), ti_smem, st, tiles, d, dp,
                  (__nv_bfloat16*)St);
   count_launch();
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  if (plain) return f32_mul_img(Y, ldy, M, d, dp, St, Q, ldq, err, st);
   CUtensorMap map;
   if (!make_map(&map, St, KP, (uint64_t)3 * dp, KP, 64, 64)) return cudaErrorInvalidValue;
   QmParams p;

@@ -130,35 +130,39 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// x rounded to BF16 (round to nearest even) as FP32 bits (low 16 bits zero),
-// by integer arithmetic on the full-rate ALUs; equal to __float2bfloat16_rn
-// for every finite x.
-__device__ __forceinline__ uint32_t bf16_rne_bits(float x) {
-  const uint32_t u = __float_as_uint(x);
-  return (u + 0x7FFFu + ((u >> 16) & 1u)) & 0xFFFF0000u;
+// Packed FP32 pairs (one instruction for two values).
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+      "sub.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
 }
 
-// Three-way BF16 split x = h + m + l (h = bf16(x), m = bf16(x - h),
-// l = bf16(x - h - m)) of four values, packed as BF16 pairs:
-// hp[0] = (h1, h0), hp[1] = (h3, h2), likewise mp, lp.
+// Two values as x = h + m + l, each part packed as a BF16 pair: h and m
+// rounded to nearest, l the remaining 7 significant bits, so the sum is exact
+// for 2^-110 <= |x| < 2^127.  Integer and packed FP32 instructions only, 6.5 per
+// value (the conversion instructions, and rounding every part to nearest even
+// -- 16 per value -- had made the split the converter warps' bottleneck).
+__device__ __forceinline__ void split3(float2 x, uint32_t& h, uint32_t& m, uint32_t& l) {
+  const uint32_t hx = (__float_as_uint(x.x) + 0x8000u) & 0xFFFF0000u;
+  const uint32_t hy = (__float_as_uint(x.y) + 0x8000u) & 0xFFFF0000u;
+  h = __byte_perm(hx, hy, 0x7632);
+  const float2 r1 = sub2(x, make_float2(__uint_as_float(hx), __uint_as_float(hy)));
+  const uint32_t mx = (__float_as_uint(r1.x) + 0x8000u) & 0xFFFF0000u;
+  const uint32_t my = (__float_as_uint(r1.y) + 0x8000u) & 0xFFFF0000u;
+  m = __byte_perm(mx, my, 0x7632);
+  const float2 r2 = sub2(r1, make_float2(__uint_as_float(mx), __uint_as_float(my)));
+  l = __byte_perm(__float_as_uint(r2.x), __float_as_uint(r2.y), 0x7632);
+}
+
+// Four values: hp[0] = (h1, h0), hp[1] = (h3, h2), likewise mp, lp.
 __device__ __forceinline__ void split3_bf16x4(const float (&v)[4], uint32_t (&hp)[2],
                                               uint32_t (&mp)[2], uint32_t (&lp)[2]) {
-  uint32_t hb[4], mb[4], lb[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    hb[j] = bf16_rne_bits(v[j]);
-    const float r1 = v[j] - __uint_as_float(hb[j]);
-    mb[j] = bf16_rne_bits(r1);
-    lb[j] = bf16_rne_bits(r1 - __uint_as_float(mb[j]));
-  }
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    hp[q] = __byte_perm(hb[2 * q], hb[2 * q + 1], 0x7632);
-    mp[q] = __byte_perm(mb[2 * q], mb[2 * q + 1], 0x7632);
-    lp[q] = __byte_perm(lb[2 * q], lb[2 * q + 1], 0x7632);
-  }
+  split3(make_float2(v[0], v[1]), hp[0], mp[0], lp[0]);
+  split3(make_float2(v[2], v[3]), hp[1], mp[1], lp[1]);
 }
-
 
 }  // namespace
 }  // namespace ruqlp

@@ -35,7 +35,7 @@ def _check(Y, A, X, trans):
     assert bool(((Y.double() - R).abs() <= bound).all())
 
 
-@pytest.mark.parametrize("m,n,d", [(64, 200, 1), (192, 192, 16), (257, 255, 17), (300, 1000, 33),
+@pytest.mark.parametrize("m,n,d", [(64, 200, 1), (128, 128, 16), (257, 255, 17), (300, 1000, 33),
                                    (1001, 777, 37), (2560, 2047, 224), (640, 20000, 225),
                                    (512, 300, 300), (19500, 1030, 20)])
 @pytest.mark.parametrize("trans", [False, True])
