@@ -146,11 +146,14 @@ cudaError_t spmm_csr(Ty tv, const int32_t* ptr, const int32_t* idx, const void* 
 // ---- batched execution (ruqlp_decompose_batch) ----------------------------
 // One entry of the device problem table: matrix A_i, its FP32 work buffers
 // (ld dp) and its outputs.
+// BMat::flags: FP32 items whose A X, A^T Y run on the tensor cores (k_f32tc.cu)
+enum : int { BM_F32_AX = 1, BM_F32_ATY = 2 };
 enum BufId : int { B_X = 0, B_Y = 1, B_Z = 2, B_P = 3 };
 struct BMat {
   const void* A;
   int64_t lda, m, n;
-  int d, dp, ot, pad;
+  int d, dp, ot;
+  int flags;  // BM_* bits
   float* X;  // n x dp
   float* Y;  // m x dp
   float* Z;  // n x dp
@@ -161,7 +164,8 @@ struct BMat {
   float* tiles;
   const double* omega;  // NULL: generated from seed (philox.cuh)
   uint64_t seed;
-  void* Bt;        // dp x ldbt BF16 (tensor-core items): the transposed skinny operand
+  void* Bt;        // dp x ldbt BF16 (tensor-core items): the transposed skinny operand;
+                   // FP32 items: the split skinny operand's image (null without room for it)
   void* Btl;       // its low BF16 part (same layout), for the two-part B^T = A^T Q
   int64_t ldbt;
   // orth_tc: this item's CholeskyQR runs on the tensor cores (bgram_tc,
@@ -173,9 +177,7 @@ struct BMat {
   // Qout (FP32, leading dimension d) instead of the Y buffer (tensor-core
   // items with the CUDA-core solve and FP32 outputs: nothing reads Y after
   // that solve, the last product taking its BF16 parts)
-  int q_direct;
-  int f32_tc[2];  // FP32 item: A X, A^T Y on the tensor cores (k_f32tc.cu)
-  void* Ximg;  // its split skinny operand (null without room for it)
+  int q_direct, pad2;
   void* Qout;
   void* Lout;
   void* Pout;
@@ -205,7 +207,8 @@ int bgram_tiles(int64_t M, int d, bool sym, int max_slabs);
 // one CTA per row slab, upper-triangle blocks only); bgram_sym_ctas is an
 // item's CTA count (0 for wider items, whose tiles go to bgram).
 int bgram_sym_ctas(int64_t M, int d, int max_slabs);
-cudaError_t bgram_sym(const BMat* T, const int* prefix, int total, int count, int src,
+// src2 != src: the upper triangle of buf[src]^T buf[src2] instead.
+cudaError_t bgram_sym(const BMat* T, const int* prefix, int total, int count, int src, int src2,
                       int max_slabs, cudaStream_t st);
 // Batched CholeskyQR passes on the tensor cores (k_borth.cu, k_qmul.cu) for
 // items with orth_tc (dp <= BO_DPMAX).  Work comes as units (a row range of
@@ -231,10 +234,10 @@ cudaError_t bgram_tc(const BMat* T, const BoUnit* units, const int* uoff, int gr
 cudaError_t btrinv(const BMat* T, const int* list, int n, int dmax, cudaStream_t st);
 cudaError_t bqmul_tc(const BMat* T, const BoUnit* units, const int* uoff, int grid, int src,
                      int dst, int make_bt, int* err, cudaStream_t st);
-// reduce = false: only the CUDA-core tiles (bgram_reduce adds the slabs
-// later, e.g. together with bgram_tc's)
+// The CUDA-core tiles of the other items; bgram_reduce adds the slabs of all
+// (together with bgram_sym's and bgram_tc's).
 cudaError_t bgram(const BMat* T, const int* prefix, int total, int count, int src, int src2,
-                  int max_slabs, int dmax, cudaStream_t st, bool reduce = true);
+                  int max_slabs, cudaStream_t st);
 cudaError_t bgram_reduce(const BMat* T, int count, int src, int src2, int max_slabs, int dmax,
                          cudaStream_t st);
 int btrsm_blocks(int64_t M);
@@ -341,10 +344,18 @@ cudaError_t f32_mul_img(const float* A, int64_t lda, int64_t M, int K, int dp, c
 // Bytes of the split X of a product over K rows (img above; null: every CTA
 // splits X itself, with the same result).
 size_t f32_img_bytes(int64_t K, int dp);
-// Batched: unit s of S of an item (tt: its index among the matrix's tail
-// items); f32_tiles appends a matrix's units and its split items.
+// Batched: unit s of S of an item (8 bytes); f32_tiles appends a matrix's
+// units and its split items.
 struct F32Tile {
-  int mat, item, tt, s, S;
+  uint64_t v;
+  __host__ __device__ static F32Tile make(int mat, int item, int s, int S) {
+    return {(uint64_t)(uint32_t)mat << 40 | (uint64_t)(uint32_t)item << 16 |
+            (uint64_t)(uint32_t)s << 8 | (uint64_t)(uint32_t)S};
+  }
+  __host__ __device__ int mat() const { return (int)(v >> 40); }
+  __host__ __device__ int item() const { return (int)(v >> 16 & 0xFFFFFF); }
+  __host__ __device__ int s() const { return (int)(v >> 8 & 0xFF); }
+  __host__ __device__ int S() const { return (int)(v & 0xFF); }
 };
 void f32_tiles(int mat, const F32Split& sp, std::vector<F32Tile>& list,
                std::vector<F32Tile>& fix);

@@ -8,7 +8,7 @@ namespace ruqlp {
 namespace {
 
 // X_i (n x dp, FP32) <- Omega_i (n x d, FP64), zero padding columns; for
-// tensor-core items also Bt_i = bf16(X_i)^T (dp x ldbt, K-major), the first
+// tensor-core items instead Bt_i = bf16(X_i)^T (dp x ldbt, K-major), the first
 // product's B operand.  64-row blocks through a shared tile, so both the
 // row-major and the transposed writes are coalesced; a thread issues its
 // eight loads of a 64 x 32 chunk before any store.
@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(256) k_bcast_omega(const BMat* __restrict__ T)
       for (int q = 0; q < OB / 8; ++q) {
         const int64_t r = r0 + ty + 8 * q;
         t[ty + 8 * q][tx] = v[q];
-        if (r < n && c < dp) X[r * dp + c] = v[q];
+        if (Bt == nullptr && r < n && c < dp) X[r * dp + c] = v[q];
       }
       if (Bt == nullptr) continue;
       __syncthreads();

@@ -156,19 +156,28 @@ struct FtSingle {
   }
 };
 
+// An item's index among the tail items (past the whole waves of `sms` items).
+__device__ __forceinline__ int tail_index_of(int64_t rows, int nch, int item, int sms) {
+  const int items = (int)((rows + F32_BM - 1) / F32_BM) * nch;
+  return item - items / sms * sms;
+}
+
 // Batch: CTA c takes entries c, c + P, ... of a host-built list.
 struct FtBatch {
   const F32Tile* list;
   int n;
   const BMat* T;
-  int src, dst;
+  int src, dst, sms;
   bool trans;
+  __device__ int tail_index(int64_t rows, int nch, int item) const {
+    return tail_index_of(rows, nch, item, sms);
+  }
   __device__ int count() const {
     return (int)blockIdx.x < n ? (n - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   }
   __device__ FtUnit get(int i) const {
     const F32Tile e = list[blockIdx.x + (int64_t)i * gridDim.x];
-    const BMat& b = T[e.mat];
+    const BMat& b = T[e.mat()];
     FtUnit u;
     u.A = (const float*)b.A;
     u.lda = b.lda;
@@ -182,17 +191,18 @@ struct FtBatch {
     u.st = b.status;
     const F32Split sp = f32_columns(b.dp);
     const int KB = (int)((u.K + F32_BK - 1) / F32_BK);
-    ft_columns(sp, e.item, b.dp, u);
-    u.img = b.Ximg == nullptr
+    ft_columns(sp, e.item(), b.dp, u);
+    u.img = b.Bt == nullptr
                 ? nullptr
-                : (const uint8_t*)b.Ximg + (int64_t)(u.col0 / sp.w) * KB * f32_xstage(sp.w);
-    u.kb0 = (int)((int64_t)KB * e.s / e.S);
-    u.kb1 = (int)((int64_t)KB * (e.s + 1) / e.S);
-    if (e.S == 1) {
+                : (const uint8_t*)b.Bt + (int64_t)(u.col0 / sp.w) * KB * f32_xstage(sp.w);
+    const int s = e.s(), S = e.S();
+    u.kb0 = (int)((int64_t)KB * s / S);
+    u.kb1 = (int)((int64_t)KB * (s + 1) / S);
+    if (S == 1) {
       u.out = bbuf(b, dst) + (int64_t)u.tile * F32_BM * b.dp + u.col0;
       u.ldo = b.dp;
     } else {
-      u.out = (float*)b.partial + (int64_t)(e.tt * e.S + e.s) * F32_BM * sp.w;
+      u.out = (float*)b.partial + (int64_t)(tail_index(u.rows, sp.nch, e.item()) * S + s) * F32_BM * sp.w;
       u.ldo = sp.w;
     }
     return u;
@@ -322,14 +332,14 @@ __global__ void __launch_bounds__(FT_CT) k_f32_split(const __grid_constant__ FtP
 // Batch: block (x, i) takes K block x (and every gridDim.x after) of item i.
 __global__ void __launch_bounds__(FT_CT) k_bf32_split(const BMat* __restrict__ T, int src) {
   const BMat& b = T[blockIdx.y];
-  if (b.Ximg == nullptr) return;
+  if (!(b.flags & (src == B_Y ? BM_F32_ATY : BM_F32_AX))) return;
   const F32Split sp = f32_columns(b.dp);
   const int64_t K = src == B_Y ? b.m : b.n;
   const int KB = (int)((K + F32_BK - 1) / F32_BK);
   for (int x = blockIdx.x; x < KB * sp.nch; x += gridDim.x) {
     const int ch = x / KB, kb = x - ch * KB;
     split_block(bbuf(b, src), b.dp, K, b.d, b.dp, kb, ch * sp.w, sp.w,
-                (uint8_t*)b.Ximg + (int64_t)x * f32_xstage(sp.w), b.status);
+                (uint8_t*)b.Bt + (int64_t)x * f32_xstage(sp.w), b.status);
   }
 }
 
@@ -692,8 +702,8 @@ k_f32_tc(const __grid_constant__ FtParams p, int stages) {
 template <bool TRANS, bool IMG>
 __global__ void __launch_bounds__(FT_THREADS, 1)
 k_bf32_tc(const F32Tile* __restrict__ list, int n, const BMat* __restrict__ T, int src, int dst,
-          int stages, int wmax, int* err) {
-  const FtBatch w{list, n, T, src, dst, TRANS};
+          int sms, int stages, int wmax, int* err) {
+  const FtBatch w{list, n, T, src, dst, sms, TRANS};
   ft_body<TRANS, IMG>(w, stages, wmax, err);
 }
 
@@ -735,14 +745,15 @@ __global__ void __launch_bounds__(256) k_f32_fixup(const __grid_constant__ FtPar
 // Batch: block x is the x-th split item of the list's fix-up entries.
 __global__ void __launch_bounds__(256) k_bf32_fixup(const F32Tile* __restrict__ list,
                                                     const BMat* __restrict__ T, int dst,
-                                                    bool trans) {
+                                                    bool trans, int sms) {
   const F32Tile e = list[blockIdx.x];
-  const BMat& b = T[e.mat];
+  const BMat& b = T[e.mat()];
+  const int64_t rows = trans ? b.n : b.m;
   const F32Split sp = f32_columns(b.dp);
   FtUnit u;
-  ft_columns(sp, e.item, b.dp, u);
-  f32_fixup((const float*)b.partial, e.tt, e.S, sp.w, u.w,
-            (trans ? b.n : b.m) - (int64_t)u.tile * F32_BM,
+  ft_columns(sp, e.item(), b.dp, u);
+  f32_fixup((const float*)b.partial, tail_index_of(rows, sp.nch, e.item(), sms), e.S(), sp.w, u.w,
+            rows - (int64_t)u.tile * F32_BM,
             bbuf(b, dst) + (int64_t)u.tile * F32_BM * b.dp + u.col0, b.dp);
 }
 
@@ -880,10 +891,10 @@ size_t f32_img_bytes(int64_t K, int dp) {
 void f32_tiles(int mat, const F32Split& sp, std::vector<F32Tile>& list,
                std::vector<F32Tile>& fix) {
   const int whole = sp.full_waves * sp.P;
-  for (int i = 0; i < whole; ++i) list.push_back({mat, i, 0, 0, 1});
+  for (int i = 0; i < whole; ++i) list.push_back(F32Tile::make(mat, i, 0, 1));
   for (int tt = 0; tt < sp.tail; ++tt) {
-    for (int s = 0; s < sp.S; ++s) list.push_back({mat, whole + tt, tt, s, sp.S});
-    if (sp.S > 1) fix.push_back({mat, whole + tt, tt, 0, sp.S});
+    for (int s = 0; s < sp.S; ++s) list.push_back(F32Tile::make(mat, whole + tt, s, sp.S));
+    if (sp.S > 1) fix.push_back(F32Tile::make(mat, whole + tt, 0, sp.S));
   }
 }
 
@@ -903,11 +914,12 @@ cudaError_t bf32_gemm_tc(bool trans, const BMat* T, const F32Tile* list, int n,
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  kern<<<std::min(n, sm_count()), FT_THREADS, smem, st>>>(list, n, T, src, dst, stages, wmax, err);
+  kern<<<std::min(n, sm_count()), FT_THREADS, smem, st>>>(list, n, T, src, dst, sm_count(), stages,
+                                                             wmax, err);
   count_launch();
   e = cudaGetLastError();
   if (e != cudaSuccess || nfix <= 0) return e;
-  k_bf32_fixup<<<dim3(nfix, F32_BM / 4), 256, 0, st>>>(fix, T, dst, trans);
+  k_bf32_fixup<<<dim3(nfix, F32_BM / 4), 256, 0, st>>>(fix, T, dst, trans, sm_count());
   count_launch();
   return cudaGetLastError();
 }

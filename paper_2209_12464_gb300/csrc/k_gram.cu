@@ -300,8 +300,11 @@ constexpr int packed_blocks(int dp) {
   for (int bi = 0; bi < dp / 4; ++bi) n += dp / 8 - bi / 2;
   return n;
 }
-template <int DP>
-__device__ __forceinline__ void gram_sym_packed(const float* __restrict__ X, int64_t ld,
+// SYM = false: the upper triangle of X^T W instead (R_B = P^T B^T, of which L
+// keeps only that triangle).
+template <int DP, bool SYM>
+__device__ __forceinline__ void gram_sym_packed(const float* __restrict__ X,
+                                                const float* __restrict__ W, int64_t ld,
                                                 int64_t M, int d, int64_t slab,
                                                 double* __restrict__ partial, int slab_id,
                                                 float* __restrict__ sbuf) {
@@ -310,6 +313,7 @@ __device__ __forceinline__ void gram_sym_packed(const float* __restrict__ X, int
   static_assert(NV * 4 * NTS == TK * DP, "chunk split");
   static_assert(packed_blocks(DP) <= NTS, "one block per thread");
   float(*Xs)[DP] = reinterpret_cast<float(*)[DP]>(sbuf);
+  float(*Ws)[DP] = SYM ? Xs : reinterpret_cast<float(*)[DP]>(sbuf + TK * DP);
   const int64_t r_begin = (int64_t)slab_id * slab;
   const int64_t r_end = min(M, r_begin + slab);
   const int t = threadIdx.x;
@@ -325,33 +329,40 @@ __device__ __forceinline__ void gram_sym_packed(const float* __restrict__ X, int
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-  auto load = [&](int64_t r0, float4 (&v)[NV]) {
+  auto load = [&](const float* S, int64_t r0, float4 (&v)[NV]) {
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
       const int e = (q * NTS + t) * 4;
       const int rr = e / DP, cc = e % DP;
       const int64_t r = r0 + rr;
-      v[q] = (r < r_end) ? *reinterpret_cast<const float4*>(X + r * ld + cc)
+      v[q] = (r < r_end) ? *reinterpret_cast<const float4*>(S + r * ld + cc)
                          : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
-  float4 vx[NV];
+  float4 vx[NV], vw[SYM ? 1 : NV];
   int64_t r0 = r_begin;
-  if (r0 < r_end) load(r0, vx);
+  if (r0 < r_end) {
+    load(X, r0, vx);
+    if constexpr (!SYM) load(W, r0, vw);
+  }
   for (; r0 < r_end; r0 += TK) {
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
       const int e = (q * NTS + t) * 4;
       *reinterpret_cast<float4*>(&Xs[e / DP][e % DP]) = vx[q];
+      if constexpr (!SYM) *reinterpret_cast<float4*>(&Ws[e / DP][e % DP]) = vw[q];
     }
     __syncthreads();
-    if (r0 + TK < r_end) load(r0 + TK, vx);  // next chunk while computing this one
+    if (r0 + TK < r_end) {  // next chunk while computing this one
+      load(X, r0 + TK, vx);
+      if constexpr (!SYM) load(W, r0 + TK, vw);
+    }
     if (active) {
 #pragma unroll 4
       for (int k = 0; k < TK; ++k) {
         const float4 a4 = *reinterpret_cast<const float4*>(&Xs[k][ra]);
-        const float4 b0 = *reinterpret_cast<const float4*>(&Xs[k][cb]);
-        const float4 b1 = *reinterpret_cast<const float4*>(&Xs[k][cb + 4]);
+        const float4 b0 = *reinterpret_cast<const float4*>(&Ws[k][cb]);
+        const float4 b1 = *reinterpret_cast<const float4*>(&Ws[k][cb + 4]);
         const float a[4] = {a4.x, a4.y, a4.z, a4.w};
         const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
@@ -378,10 +389,11 @@ __device__ __forceinline__ void gram_sym_packed(const float* __restrict__ X, int
 
 // Batched symmetric Grams of the items with dp <= 80: CTA t of the launch ->
 // (item, slab) through prefix (launch order appended, as k_bgram).
+template <bool SYM>
 __global__ void __launch_bounds__(NTS)
 k_bgram_sym(const BMat* __restrict__ Tb, const int* __restrict__ prefix, int count, int src,
-            int max_slabs) {
-  __shared__ __align__(16) float sbuf[TK * SMALL_MAX];
+            int src2, int max_slabs) {
+  __shared__ __align__(16) float sbuf[(SYM ? 1 : 2) * TK * SMALL_MAX];
   const int t = blockIdx.x;
   int lo = 0, hi = count;
   while (hi - lo > 1) {
@@ -393,13 +405,13 @@ k_bgram_sym(const BMat* __restrict__ Tb, const int* __restrict__ prefix, int cou
   const int64_t M = (src == B_Y) ? b.m : b.n;
   int64_t slab;
   gram_slabs(M, max_slabs, &slab);
-  const float* X = bbuf(b, src);
+  const float *X = bbuf(b, src), *W = bbuf(b, src2);
   switch (b.dp / 16) {
-    case 1: gram_sym_packed<16>(X, b.dp, M, b.d, slab, b.partial, local, sbuf); break;
-    case 2: gram_sym_packed<32>(X, b.dp, M, b.d, slab, b.partial, local, sbuf); break;
-    case 3: gram_sym_packed<48>(X, b.dp, M, b.d, slab, b.partial, local, sbuf); break;
-    case 4: gram_sym_packed<64>(X, b.dp, M, b.d, slab, b.partial, local, sbuf); break;
-    default: gram_sym_packed<80>(X, b.dp, M, b.d, slab, b.partial, local, sbuf); break;
+    case 1: gram_sym_packed<16, SYM>(X, W, b.dp, M, b.d, slab, b.partial, local, sbuf); break;
+    case 2: gram_sym_packed<32, SYM>(X, W, b.dp, M, b.d, slab, b.partial, local, sbuf); break;
+    case 3: gram_sym_packed<48, SYM>(X, W, b.dp, M, b.d, slab, b.partial, local, sbuf); break;
+    case 4: gram_sym_packed<64, SYM>(X, W, b.dp, M, b.d, slab, b.partial, local, sbuf); break;
+    default: gram_sym_packed<80, SYM>(X, W, b.dp, M, b.d, slab, b.partial, local, sbuf); break;
   }
 }
 
@@ -412,14 +424,20 @@ __global__ void k_bgram_reduce(const BMat* __restrict__ Tb, int src, int src2, i
   const int64_t M = (src == B_Y) ? b.m : b.n;
   int64_t slab;
   const int slabs = (int)gram_slabs(M, max_slabs, &slab);
-  const int i = (int)(idx / d), j = (int)(idx % d);
-  // symmetric partials hold one triangle: the upper one from the CUDA-core
-  // tiles, the lower one from the tensor-core kernel (orth_tc items)
-  const bool mirror = sym && (b.orth_tc ? j > i : j < i);
-  const int64_t so = mirror ? ((int64_t)j * d + i) : idx;
-  const double s = slab_sum(b.partial, slabs, (int64_t)d * d, so);
-  b.G[idx] = s;
-  b.Gf[idx] = (float)s;
+  const int i = (int)idx / d, j = (int)idx - i * d;
+  // one sum per entry of the upper triangle: a Gram is mirrored (the Cholesky
+  // reads Gf alone), of R_B = P^T B^T only that triangle is kept (L reads G
+  // alone).  Symmetric partials hold one triangle: the upper one from the
+  // CUDA-core tiles, the lower one from the tensor-core kernel (orth_tc items)
+  if (j < i) return;
+  const int64_t lo = (int64_t)j * d + i;
+  const double s = slab_sum(b.partial, slabs, (int64_t)d * d, sym && b.orth_tc ? lo : idx);
+  if (sym) {
+    b.Gf[idx] = (float)s;
+    b.Gf[lo] = (float)s;
+  } else {
+    b.G[idx] = s;
+  }
 }
 
 }  // namespace
@@ -437,10 +455,11 @@ int bgram_sym_ctas(int64_t M, int d, int max_slabs) {
   return gram_is_small((d + 15) / 16 * 16) ? (int)gram_slabs(M, max_slabs, &slab) : 0;
 }
 
-cudaError_t bgram_sym(const BMat* T, const int* prefix, int total, int count, int src,
+cudaError_t bgram_sym(const BMat* T, const int* prefix, int total, int count, int src, int src2,
                       int max_slabs, cudaStream_t st) {
   if (total <= 0) return cudaSuccess;
-  k_bgram_sym<<<total, NTS, 0, st>>>(T, prefix, count, src, max_slabs);
+  auto kern = src == src2 ? k_bgram_sym<true> : k_bgram_sym<false>;
+  kern<<<total, NTS, 0, st>>>(T, prefix, count, src, src2, max_slabs);
   count_launch();
   return cudaGetLastError();
 }
@@ -454,13 +473,11 @@ cudaError_t bgram_reduce(const BMat* T, int count, int src, int src2, int max_sl
 }
 
 cudaError_t bgram(const BMat* T, const int* prefix, int total, int count, int src, int src2,
-                  int max_slabs, int dmax, cudaStream_t st, bool reduce) {
+                  int max_slabs, cudaStream_t st) {
   if (total <= 0) return cudaSuccess;
   k_bgram<<<total, NT, 0, st>>>(T, prefix, count, src, src2, max_slabs);
   count_launch();
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || !reduce) return e;
-  return bgram_reduce(T, count, src, src2, max_slabs, dmax, st);
+  return cudaGetLastError();
 }
 
 cudaError_t gram_f32(const float* X, int64_t ldx, const float* W, int64_t ldw, int64_t M, int d1,

@@ -146,7 +146,7 @@ k_bgemm(const BMat* __restrict__ T, const int* __restrict__ prefix, int count, i
     if (prefix[mid] <= t) lo = mid; else hi = mid;
   }
   const BMat& b = T[prefix[count + 1 + lo]];  // the launch order's item lo
-  if (b.f32_tc[TRANS_A ? 1 : 0] && !range_redo(b.status->range)) return;
+  if ((b.flags & (TRANS_A ? BM_F32_ATY : BM_F32_AX)) && !range_redo(b.status->range)) return;
   const int local = t - prefix[lo];
   const int ntn = (b.d + BN - 1) / BN;
   const int64_t Mout = TRANS_A ? b.n : b.m, K = TRANS_A ? b.m : b.n;

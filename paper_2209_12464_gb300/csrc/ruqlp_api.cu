@@ -869,6 +869,7 @@ struct BatchPlan {
   std::vector<F32Tile> ft[2], ftfix[2];
   size_t off_ft[2], off_ftfix[2];
   int wmax_ft = 16;
+  bool any_tc = false;  // any BF16 tensor-core item
   // tensor-core CholeskyQR items (orth_tc): their list (for k_btrinv) and,
   // over Y (m rows) and over Z (n rows), the Gram units (one row slab each)
   // and the Q = Y R^{-1} units with their per-CTA ranges
@@ -913,8 +914,8 @@ ruqlp_status batch_launches(ruqlp_ctx* h, const BatchPlan& bp, int count, int q,
     for (int pass = 0; pass < passes; ++pass) {
       const int from = pass == 0 ? src : dst;
       const int mb = pass == passes - 1 ? make_bt : 0;
-      CK(bgram_sym(T, pre(gp), tot(gp), count, from, kMaxSplits, st));
-      CK(bgram(T, pre(gw), tot(gw), count, from, from, kMaxSplits, bp.dmax, st, false));
+      CK(bgram_sym(T, pre(gp), tot(gp), count, from, from, kMaxSplits, st));
+      CK(bgram(T, pre(gw), tot(gw), count, from, from, kMaxSplits, st));
       CK(bgram_tc(T, (const BoUnit*)dev(bo.o_gu), (const int*)dev(bo.o_goff), ng, from,
                   kMaxSplits, err, st));
       if (tot(gp) > 0 || tot(gw) > 0 || ng > 0) CK(bgram_reduce(T, count, from, from, kMaxSplits, bp.dmax, st));
@@ -954,7 +955,11 @@ ruqlp_status batch_launches(ruqlp_ctx* h, const BatchPlan& bp, int count, int q,
   }
   if ((s = prod(true, B_Y, B_Z, true)) != RUQLP_OK) return s;
   if ((s = orth_b(B_Z, B_P, 3, 0)) != RUQLP_OK) return s;
-  CK(bgram(T, pre(PF_GPZ), tot(PF_GPZ), count, B_P, B_Z, kMaxSplits, bp.dmax, st));
+  // R_B = P^T B^T: the narrow items' upper triangles (over the same slabs as
+  // their Grams), the others' tiles
+  CK(bgram_sym(T, pre(PF_GN), tot(PF_GN), count, B_P, B_Z, kMaxSplits, st));
+  CK(bgram(T, pre(PF_GPZ), tot(PF_GPZ), count, B_P, B_Z, kMaxSplits, st));
+  CK(bgram_reduce(T, count, B_P, B_Z, kMaxSplits, bp.dmax, st));
   CK(boutputs(T, count, bp.max_out, st));
   return RUQLP_OK;
 }
@@ -1029,12 +1034,13 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
     b.use_tc = (ct0 == Ty::BF16 && !h->bf16_simt && tc_supported(D.data, D.ld, dp)) ? 1 : 0;
     for (int x = 0; x < 2; ++x) {
       const int64_t rows = x ? n : m, K = x ? m : n;
-      b.f32_tc[x] = (ct0 == Ty::F32 && f32_tc_supported(K)) ? 1 : 0;
-      if (!b.f32_tc[x]) continue;
+      if (ct0 != Ty::F32 || !f32_tc_supported(K)) continue;
+      b.flags |= x ? BM_F32_ATY : BM_F32_AX;
       bp.wmax_ft = std::max(bp.wmax_ft, f32_columns(dp).w);
       f32_tiles(i, f32_split(rows, K, m, n, d, dp), bp.ft[x], bp.ftfix[x]);
     }
-    const bool img = h->f32_img && (b.f32_tc[0] || b.f32_tc[1]);
+    const bool img = h->f32_img && (b.flags & (BM_F32_AX | BM_F32_ATY));
+    bp.any_tc = bp.any_tc || b.use_tc;
     // option batch_orth_tc: BF16 items of width dp <= 80 run their
     // CholeskyQR passes on the tensor cores (a rule on the dtype, the
     // options and d only, so an item decides the same alone and in any
@@ -1082,7 +1088,7 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
     // longest contraction first, as the BF16 tile lists
     std::stable_sort(bp.ft[x].begin(), bp.ft[x].end(), [&](const F32Tile& a, const F32Tile& b) {
       auto cost = [&](const F32Tile& t) {
-        return (x ? A[t.mat].dense.m : A[t.mat].dense.n) / t.S;
+        return (x ? A[t.mat()].dense.m : A[t.mat()].dense.n) / t.S();
       };
       return cost(a) > cost(b);
     });
@@ -1146,7 +1152,7 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
     bp.off_bo_items = take(sizeof(int) * std::max<size_t>(bp.bo_items.size(), 1));
   }
   const size_t map3 = btc_map_bytes();  // all tensor maps of one matrix
-  bp.off_maps = take(map3 * count);
+  bp.off_maps = take(bp.any_tc ? map3 * count : 0);
   bp.meta_end = off;
   bp.off_status = take(sizeof(DevStatus) * count);
   bp.off_err = take(sizeof(int));
@@ -1176,9 +1182,10 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
     b.G = (double*)(base + oG[i]);
     b.Gf = (float*)(base + oGf[i]);
     b.tiles = (float*)(base + oT[i]);
-    b.Bt = b.use_tc ? (void*)(base + oB[i]) : nullptr;
+    b.Bt = b.use_tc || (h->f32_img && (b.flags & (BM_F32_AX | BM_F32_ATY)))
+               ? (void*)(base + oB[i])
+               : nullptr;
     b.Btl = b.use_tc ? (void*)(base + oB[i] + (size_t)b.dp * b.ldbt * 2) : nullptr;
-    b.Ximg = h->f32_img && (b.f32_tc[0] || b.f32_tc[1]) ? (void*)(base + oB[i]) : nullptr;
     b.St = b.orth_tc ? (void*)(base + oS[i]) : nullptr;
     b.omega = prm[i].omega;
     b.seed = prm[i].omega_seed;
@@ -1195,7 +1202,7 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
                           b.use_tc ? 0 : bgemm_tiles(b.n, b.d),
                           cc ? bgram_sym_ctas(b.m, b.d, kMaxSplits) : 0,
                           cc ? bgram_sym_ctas(b.n, b.d, kMaxSplits) : 0,
-                          bgram_tiles(b.n, b.d, false, kMaxSplits),
+                          cc && narrow ? 0 : bgram_tiles(b.n, b.d, false, kMaxSplits),
                           cc ? btrsm_blocks(b.m) : 0,
                           cc ? btrsm_blocks(b.n) : 0,
                           cc && !narrow ? bgram_tiles(b.m, b.d, true, kMaxSplits) : 0,
@@ -1230,7 +1237,7 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
     key.push_back(bp.table[i].n);
     key.push_back(bp.table[i].d);
     key.push_back(bp.table[i].use_tc);
-    key.push_back(bp.table[i].f32_tc[0] + 2 * bp.table[i].f32_tc[1]);
+    key.push_back(bp.table[i].flags);
     key.push_back(bp.table[i].orth_tc);
   }
   ruqlp_ctx::BatchEntry* g = nullptr;
@@ -1281,7 +1288,7 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
   }
   put(bp.off_tc_nn, bp.tc_nn.data(), sizeof(BTcTile) * bp.tc_nn.size());
   put(bp.off_tc_tn, bp.tc_tn.data(), sizeof(BTcTile) * bp.tc_tn.size());
-  put(bp.off_maps, g->maps.data(), g->maps.size());
+  if (bp.any_tc) put(bp.off_maps, g->maps.data(), g->maps.size());
   for (const auto& bo : bp.bo) {
     put(bo.o_gu, bo.gu.data(), sizeof(BoUnit) * bo.gu.size());
     put(bo.o_goff, bo.goff.data(), sizeof(int) * bo.goff.size());
