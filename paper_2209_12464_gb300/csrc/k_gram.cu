@@ -393,6 +393,8 @@ constexpr int packed_blocks(int dp) {
   for (int bi = 0; bi < dp / 4; ++bi) n += dp / 8 - bi / 2;
   return n;
 }
+// The chunks come through a cp.async ring (a batch of 64 FP32 matrices: 34 ->
+// 30 us a launch; 512 BF16 ones, which fill the chip, 91 either way).
 // SYM = false: the upper triangle of X^T W instead (R_B = P^T B^T, of which L
 // keeps only that triangle).
 template <int DP, bool SYM>
@@ -403,10 +405,11 @@ __device__ __forceinline__ void gram_sym_packed(const float* __restrict__ X,
                                                 float* __restrict__ sbuf) {
   constexpr int NBR = DP / 4, NBC = DP / 8;
   constexpr int NV = TK * DP / 4 / NTS;  // float4s per thread per 32-row chunk
+  constexpr int GS = SYM ? 4 : 2;        // chunks in the cp.async ring
   static_assert(NV * 4 * NTS == TK * DP, "chunk split");
   static_assert(packed_blocks(DP) <= NTS, "one block per thread");
-  float(*Xs)[DP] = reinterpret_cast<float(*)[DP]>(sbuf);
-  float(*Ws)[DP] = SYM ? Xs : reinterpret_cast<float(*)[DP]>(sbuf + TK * DP);
+  auto Xs = reinterpret_cast<float(*)[TK][DP]>(sbuf);
+  auto Ws = SYM ? Xs : reinterpret_cast<float(*)[TK][DP]>(sbuf + GS * TK * DP);
   const int64_t r_begin = (int64_t)slab_id * slab;
   const int64_t r_end = min(M, r_begin + slab);
   const int t = threadIdx.x;
@@ -422,40 +425,43 @@ __device__ __forceinline__ void gram_sym_packed(const float* __restrict__ X,
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-  auto load = [&](const float* S, int64_t r0, float4 (&v)[NV]) {
+  auto copy = [&](float (*D)[DP], const float* S, int64_t r0) {
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
       const int e = (q * NTS + t) * 4;
-      const int rr = e / DP, cc = e % DP;
-      const int64_t r = r0 + rr;
-      v[q] = (r < r_end) ? *reinterpret_cast<const float4*>(S + r * ld + cc)
-                         : make_float4(0.f, 0.f, 0.f, 0.f);
+      const int64_t r = r0 + e / DP;
+      const bool ok = r < r_end;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                       (uint32_t)__cvta_generic_to_shared(&D[e / DP][e % DP])),
+                   "l"(ok ? S + r * ld + e % DP : S), "r"(ok ? 16 : 0)
+                   : "memory");
     }
   };
-  float4 vx[NV], vw[SYM ? 1 : NV];
-  int64_t r0 = r_begin;
-  if (r0 < r_end) {
-    load(X, r0, vx);
-    if constexpr (!SYM) load(W, r0, vw);
-  }
-  for (; r0 < r_end; r0 += TK) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      const int e = (q * NTS + t) * 4;
-      *reinterpret_cast<float4*>(&Xs[e / DP][e % DP]) = vx[q];
-      if constexpr (!SYM) *reinterpret_cast<float4*>(&Ws[e / DP][e % DP]) = vw[q];
+  int64_t rl = r_begin;  // next chunk to fetch
+  int st_l = 0, st = 0;
+  auto fetch = [&]() {
+    if (rl < r_end) {
+      copy(Xs[st_l], X, rl);
+      if constexpr (!SYM) copy(Ws[st_l], W, rl);
     }
-    __syncthreads();
-    if (r0 + TK < r_end) {  // next chunk while computing this one
-      load(X, r0 + TK, vx);
-      if constexpr (!SYM) load(W, r0 + TK, vw);
-    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    rl += TK;
+    if (++st_l == GS) st_l = 0;
+  };
+  for (int i = 0; i < GS - 1; ++i) fetch();
+  for (int64_t r0 = r_begin; r0 < r_end; r0 += TK) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(GS - 2) : "memory");
+    __syncthreads();  // the chunk has landed, and its predecessor's slot is free
+    fetch();
+    const float(*Xc)[DP] = Xs[st];
+    const float(*Wc)[DP] = Ws[st];
+    if (++st == GS) st = 0;
     if (active) {
 #pragma unroll 4
       for (int k = 0; k < TK; ++k) {
-        const float4 a4 = *reinterpret_cast<const float4*>(&Xs[k][ra]);
-        const float4 b0 = *reinterpret_cast<const float4*>(&Ws[k][cb]);
-        const float4 b1 = *reinterpret_cast<const float4*>(&Ws[k][cb + 4]);
+        const float4 a4 = *reinterpret_cast<const float4*>(&Xc[k][ra]);
+        const float4 b0 = *reinterpret_cast<const float4*>(&Wc[k][cb]);
+        const float4 b1 = *reinterpret_cast<const float4*>(&Wc[k][cb + 4]);
         const float a[4] = {a4.x, a4.y, a4.z, a4.w};
         const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
@@ -464,7 +470,6 @@ __device__ __forceinline__ void gram_sym_packed(const float* __restrict__ X,
           for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
       }
     }
-    __syncthreads();
   }
   if (!active) return;
   double* P = partial + (int64_t)slab_id * d * d;
@@ -486,7 +491,7 @@ template <bool SYM>
 __global__ void __launch_bounds__(NTS)
 k_bgram_sym(const BMat* __restrict__ Tb, const int* __restrict__ prefix, int count, int src,
             int src2, int max_slabs) {
-  __shared__ __align__(16) float sbuf[(SYM ? 1 : 2) * TK * SMALL_MAX];
+  __shared__ __align__(16) float sbuf[4 * TK * SMALL_MAX];  // (two chunks of two operands: the same)
   const int t = blockIdx.x;
   int lo = 0, hi = count;
   while (hi - lo > 1) {
