@@ -135,8 +135,10 @@ typedef struct {
  * the FP64 path and FP32 (shifted CholeskyQR3) on the FP32/BF16 paths unless
  * the "orth_fp64" option is set.  compute must equal A's dtype.
  * BF16 inputs use the tensor cores when A's leading dimension is a multiple
- * of 8 elements and A is 16-byte aligned (sketches wider than 256 columns
- * run as column chunks, one pass over A each); otherwise CUDA cores.
+ * of 8 elements and A is 16-byte aligned (sketches wider than 384 columns, or
+ * than 256 under a memory budget, run as column chunks, one pass over A each);
+ * otherwise CUDA cores.  FP32 products over 128 rows or more take the tensor
+ * cores too, each value split exactly into three BF16 parts (FP32 accuracy).
  * omega: n x d row-major FP64 Gaussian test matrix (device memory for
  * ruqlp_decompose / ruqlp_submit; host memory for ruqlp_decompose_host), or
  * NULL: then the library generates it on the device from omega_seed with
@@ -383,12 +385,12 @@ int64_t ruqlp_launch_count(void);
 /* Tile tuner of the tensor-core products (the sketch / power / B^T passes
  * of Section III-D, the bulk of the O(mnd) work): the first product of each
  * shape (orientation, two-part operand, output rows, K, dp) outside stream
- * capture times every valid column split (1, 2, 4; each with the deepest
- * shared-memory ring that fits) twice with CUDA events and keeps the fastest
+ * capture times CTA pairs sharing the skinny operand's loads and every valid
+ * column split (1, 2, 4; each with the deepest shared-memory ring that fits) twice with CUDA events and keeps the fastest
  * for the process; that configuration computes the result, so results are
  * deterministic from then on.  ruqlp_tune_file(path) loads earlier choices
  * from a text file (one "tc_gemm trans two_part rows K dp split stages us"
- * line each) and appends every new choice to it; NULL or "" stops the
+ * line each; pairs: split 1, 64 added to the stages) and appends every new choice to it; NULL or "" stops the
  * mirroring.  Returns the number of entries loaded.  Process-wide (all
  * handles); thread-safe. */
 int ruqlp_tune_file(const char* path);

@@ -115,7 +115,9 @@ cudaError_t write_L(const double* R, int d, Ty tl, void* L, bool upper, cudaStre
 cudaError_t tc_gemm(bool trans, const void* A, int64_t lda, int64_t m, int64_t n, const void* Bt,
                     int64_t ldb, int dp, float* out, int64_t ldo, float* frag, int* err,
                     cudaStream_t st, const std::function<void(bool)>& mark = {},
-                    const void* Btl = nullptr, int force_ns = 0, int withhold = 0);
+                    const void* Btl = nullptr, int force_ns = 0, int withhold = 0, int cols = 0);
+// (cols: the columns of out that are stored, a multiple of 4; 0: all dp)
+bool tc_wide_fits(int64_t m, int64_t n, int dp);
 // Mirror the product tuner's choices in a text file (loaded now, appended
 // to as shapes are tuned); returns the entries loaded.
 int tune_file(const char* path);
@@ -327,14 +329,14 @@ __host__ __device__ inline uint32_t f32_img_off(int k, int col) {
 }
 F32Split f32_split(int64_t rows, int64_t K, int64_t m, int64_t n, int d, int dp);
 bool f32_tc_supported(int64_t K);
-// out (ld ldo, dp columns written) = A X or A^T X, A m x n FP32 (ld lda), X
+// out (ld ldo, the first ocols -- d or dp, a multiple of 4 -- written) = A X or A^T X, A m x n FP32 (ld lda), X
 // FP32 (ld ldx, d columns, the first xcols >= d -- a multiple of 4 --
 // readable); frag: the Gram partials' buffer.  Sets st->range
 // when an operand is outside the split's range: the product must then be
 // formed again on the CUDA cores (a launch gated by that word).
 cudaError_t f32_gemm_tc(bool trans, const float* A, int64_t lda, int64_t m, int64_t n,
                         const float* X, int64_t ldx, int xcols, int d, int dp, float* out,
-                        int64_t ldo, float* frag, void* img, DevStatus* st,
+                        int64_t ldo, int ocols, float* frag, void* img, DevStatus* st,
                         cudaStream_t stream);
 // out = A X with X given split (img, one column chunk: dp <= 224, K < 512 rows);
 // out may be A (lda = ldo): a tile's rows are read before they are written.

@@ -84,6 +84,7 @@ struct FtUnit {
   int d, xcols;          // columns; columns of X that may be read (a multiple of 4)
   int col0, w, xw, tile, kb0, kb1;  // xw: the chunk width (the image's stages)
   float* out;            // the tile's first row, first column
+  int ocols;             // columns of the chunk that are stored
   int64_t ldo;
   bool vec;              // A's rows start on 16 bytes
   DevStatus* st;
@@ -98,7 +99,7 @@ struct FtParams {
   float* out;
   int64_t ldo;
   float* frag;
-  int d, xcols, dp, vec;
+  int d, xcols, ocols, dp, vec;
   F32Split sp;
   DevStatus* st;  // null: no range notes
   int* err;
@@ -115,6 +116,9 @@ __device__ __forceinline__ void ft_columns(const F32Split& sp, int item, int dp,
 // slab of a tail item.
 struct FtSingle {
   const FtParams* p;
+  __device__ bool skip() const {
+    return p->st != nullptr && range_redo(*(volatile int32_t*)&p->st->range);
+  }
   __device__ int count() const {
     const F32Split& sp = p->sp;
     return sp.full_waves + ((int)blockIdx.x < sp.tail * sp.S ? 1 : 0);
@@ -145,9 +149,11 @@ struct FtSingle {
                 : p->img + (int64_t)(u.col0 / sp.w) * sp.KB * f32_xstage(sp.w);
     u.kb0 = (int)((int64_t)sp.KB * s / S);
     u.kb1 = (int)((int64_t)sp.KB * (s + 1) / S);
+    u.ocols = u.w;
     if (S == 1) {
       u.out = p->out + (int64_t)u.tile * F32_BM * p->ldo + u.col0;
       u.ldo = p->ldo;
+      u.ocols = min(u.w, p->ocols - u.col0);
     } else {
       u.out = p->frag + (int64_t)c * F32_BM * sp.w;
       u.ldo = sp.w;
@@ -169,6 +175,7 @@ struct FtBatch {
   const BMat* T;
   int src, dst, sms;
   bool trans;
+  __device__ bool skip() const { return false; }
   __device__ int tail_index(int64_t rows, int nch, int item) const {
     return tail_index_of(rows, nch, item, sms);
   }
@@ -196,6 +203,7 @@ struct FtBatch {
                 ? nullptr
                 : (const uint8_t*)b.Bt + (int64_t)(u.col0 / sp.w) * KB * f32_xstage(sp.w);
     const int s = e.s(), S = e.S();
+    u.ocols = u.w;
     u.kb0 = (int)((int64_t)KB * s / S);
     u.kb1 = (int)((int64_t)KB * (s + 1) / S);
     if (S == 1) {
@@ -368,7 +376,7 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
   auto tempty = [&](int a) { return bar + 8u * (2 * FT_NA + 2 * NX + 2 + a); };
   const uint32_t drain = bar + 8u * (2 * FT_NA + 2 * NX + 4);
   uint32_t* tmem_slot = (uint32_t*)(base_ptr + (drain + 8 - base));
-  __shared__ int s_abort;
+  __shared__ int s_abort, s_skip;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31, wg = warp >> 2;
   if (t == 0) {
     for (int i = 0; i < FT_NA; ++i) {
@@ -398,9 +406,13 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   volatile int* abort_flag = &s_abort;
-  const int nunits = w.count();
   pdl_launch();
   pdl_wait();
+  // an earlier product of this run already asked for the CUDA cores (one thread
+  // reads the word: other CTAs of this launch may be setting it)
+  if (t == 0) s_skip = w.skip() ? 1 : 0;
+  __syncthreads();
+  const int nunits = s_skip ? 0 : w.count();
 
   if (wg == 0) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(FT_REG_CTL));
@@ -670,7 +682,7 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
           const int rr = r * 8 + (lane >> 2), cc = (lane & 3) * 4;
-          if (rr < left)
+          if (rr < left && c * 16 + cc < u.ocols)
             *reinterpret_cast<float4*>(u.out + (int64_t)(g * 32 + rr) * u.ldo + c * 16 + cc) =
                 *reinterpret_cast<const float4*>(stg + rr * FT_SP + cc);
         }
@@ -738,7 +750,7 @@ __global__ void __launch_bounds__(256) k_f32_fixup(const __grid_constant__ FtPar
   pdl_wait();
   FtUnit u;
   ft_columns(p.sp, p.sp.full_waves * p.sp.P + (int)blockIdx.x, p.dp, u);
-  f32_fixup(p.frag, blockIdx.x, p.sp.S, p.sp.w, u.w, p.rows - (int64_t)u.tile * F32_BM,
+  f32_fixup(p.frag, blockIdx.x, p.sp.S, p.sp.w, min(u.w, p.ocols - u.col0), p.rows - (int64_t)u.tile * F32_BM,
             p.out + (int64_t)u.tile * F32_BM * p.ldo + u.col0, p.ldo);
 }
 
@@ -814,9 +826,9 @@ bool f32_tc_supported(int64_t K) { return K >= 128; }
 
 cudaError_t f32_gemm_tc(bool trans, const float* A, int64_t lda, int64_t m, int64_t n,
                         const float* X, int64_t ldx, int xcols, int d, int dp, float* out,
-                        int64_t ldo, float* frag, void* img, DevStatus* st,
+                        int64_t ldo, int ocols, float* frag, void* img, DevStatus* st,
                         cudaStream_t stream) {
-  if (xcols < d || xcols > ldx || (xcols & 3) || (ldx & 3) || ((uintptr_t)X & 15) || (ldo & 3) || ((uintptr_t)out & 15))
+  if (ocols < d || ocols > dp || (ocols & 3) || xcols < d || xcols > ldx || (xcols & 3) || (ldx & 3) || ((uintptr_t)X & 15) || (ldo & 3) || ((uintptr_t)out & 15))
     return cudaErrorInvalidValue;
   FtParams p{};
   p.A = A;
@@ -828,6 +840,7 @@ cudaError_t f32_gemm_tc(bool trans, const float* A, int64_t lda, int64_t m, int6
   p.img = (const uint8_t*)img;
   p.out = out;
   p.ldo = ldo;
+  p.ocols = ocols;
   p.frag = frag;
   p.d = d;
   p.xcols = xcols;
@@ -868,6 +881,7 @@ cudaError_t f32_mul_img(const float* A, int64_t lda, int64_t M, int K, int dp, c
   p.img = (const uint8_t*)img;
   p.out = out;
   p.ldo = ldo;
+  p.ocols = dp;
   p.d = K;
   p.dp = dp;
   p.vec = (lda & 3) == 0 && ((uintptr_t)A & 15) == 0;

@@ -51,8 +51,11 @@ constexpr int kBatchMaps = 4;              // tensor maps per batched matrix
 struct TcParams {
   int64_t Mout;   // output rows
   int64_t K;      // contraction length
-  int dp;         // output columns (multiple of 16, <= 256)
+  int dp;         // output columns (multiple of 16, <= 256; of 32, <= 384 when wide)
+  int cols;       // columns stored (a multiple of 4)
   int ns, dpi;    // column split: items of dpi = dp / ns columns (MMA N)
+  int pair;       // 1: CTA pairs (clusters of two) take two tiles and share the
+                  // skinny operand's loads; T, tail and U then count pair tiles
   int stages;
   float* out;
   int64_t ldo;
@@ -72,7 +75,7 @@ struct Item {
 __device__ __forceinline__ int64_t sk_start(int64_t c, int64_t U, int P) { return c * U / P; }
 
 __device__ __forceinline__ int item_count(const TcParams& p) {
-  const int P = gridDim.x, c = blockIdx.x;
+  const int P = gridDim.x >> p.pair, c = blockIdx.x >> p.pair;
   int n = p.full_waves;
   if (p.tail > 0) {
     const int64_t u0 = sk_start(c, p.U, P), u1 = sk_start(c + 1, p.U, P);
@@ -82,7 +85,7 @@ __device__ __forceinline__ int item_count(const TcParams& p) {
 }
 
 __device__ __forceinline__ Item get_item(const TcParams& p, int i) {
-  const int P = gridDim.x, c = blockIdx.x;
+  const int P = gridDim.x >> p.pair, c = blockIdx.x >> p.pair;
   if (i < p.full_waves) return {c + i * P, 0, p.KB, -1};
   const int64_t u0 = sk_start(c, p.U, P), u1 = sk_start(c + 1, p.U, P);
   const int base = p.full_waves * P;
@@ -101,6 +104,7 @@ struct TcItem {
   int tile, kb0, kb1, dp;  // 128-row tile, K blocks, output columns (MMA N)
   int bcol;                // first output column (row of the skinny operand Bt)
   float* out;
+  int cols;                // columns to store
   int64_t ldo, rows;
   bool a_split;  // K-major A loaded as two 64-row boxes (batched maps)
 };
@@ -114,10 +118,12 @@ struct WorkSingle {
   static constexpr bool kGlobalMaps = false;
   __device__ int count() const { return item_count(*p); }
   __device__ TcItem get(int i) const {
-    const Item it = get_item(*p, i);
+    Item it = get_item(*p, i);
+    if (p->pair) it.tile = 2 * it.tile + (blockIdx.x & 1);
     const int mt = it.tile / p->ns, h = it.tile - mt * p->ns;
-    TcItem r{mA, mB, mB2, mt, it.kb0, it.kb1, p->dpi, h * p->dpi, nullptr, 0, 0, false};
+    TcItem r{mA, mB, mB2, mt, it.kb0, it.kb1, p->dpi, h * p->dpi, nullptr, p->dpi, 0, 0, false};
     if (it.slot < 0) {
+      r.cols = min(p->dpi, p->cols - r.bcol);
       r.out = p->out + (int64_t)mt * BM * p->ldo + r.bcol;
       r.ldo = p->ldo;
       r.rows = p->Mout - (int64_t)mt * BM;
@@ -160,6 +166,7 @@ struct WorkBatch {
     r.dp = b.dp;
     r.bcol = 0;
     r.out = bbuf(b, dst) + (int64_t)w.tile * BM * b.dp;
+    r.cols = b.dp;
     r.ldo = b.dp;
     r.rows = Mout - (int64_t)w.tile * BM;
     r.a_split = true;
@@ -178,9 +185,17 @@ __device__ __forceinline__ void tmap_acquire(const CUtensorMap* m) {
 // so h + l carries about 16 significant bits of the FP32 value); each stage
 // holds both parts' tiles and every A tile is multiplied by both into the same
 // accumulator, D += A h + A l.
-template <bool TRANS, bool B2, class W>
+// PAIR: the CTAs of a cluster of two take two tiles with the same K blocks; each
+// loads its own A tiles and one half of the skinny operand's tile, multicast to
+// both, so that half crosses the L2 -> SM path once for two SMs.  A stage is
+// free when both CTAs' MMAs have read it (each commits to both empty barriers).
+// 20000 x 20000 at d = 220: 165 -> 158 us a launch (the skinny operand's traffic
+// is not what bounds it: 0.77 of measured HBM).
+template <bool TRANS, bool B2, bool PAIR, class W>
 __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
                                         int withhold = 0) {
+  // single one-part products may have items of more than 256 columns
+  constexpr bool kWide = !B2 && !PAIR && !W::kGlobalMaps;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -202,7 +217,7 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(full_bar(s), 1);
-      mbar_init(empty_bar(s), 1);
+      mbar_init(empty_bar(s), PAIR ? 2 : 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(tfull_bar(a), 1);
@@ -229,6 +244,7 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   volatile int* abort_flag = &s_abort;
+  if (PAIR) cluster_sync();  // the peer's barriers are initialised
   pdl_launch();
   pdl_wait();
 
@@ -274,8 +290,28 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
             tma_load_2d(sa + A_TILE_BYTES / 2, it.mA, full_bar(stage), it.tile * BM + 64,
                         kb * BK, pol_a);
           }
-          tma_load_2d(sb, it.mB, full_bar(stage), kb * BK, it.bcol, pol_b);
-          if (B2) tma_load_2d(sb + b_tile, it.mB2, full_bar(stage), kb * BK, it.bcol, pol_b);
+          if constexpr (PAIR) {
+            const int half = it.dp / 2, r = (int)(blockIdx.x & 1) * half;
+            tma_load_2d_mc(sb + r * BK * 2, it.mB, full_bar(stage), kb * BK, r, 3, pol_b);
+            if (B2)
+              tma_load_2d_mc(sb + b_tile + r * BK * 2, it.mB2, full_bar(stage), kb * BK, r, 3,
+                             pol_b);
+          } else if (kWide && it.dp > 256) {  // wide: two boxes of half the columns
+            const int half = it.dp / 2;
+            tma_load_2d(sb, it.mB, full_bar(stage), kb * BK, 0, pol_b);
+            tma_load_2d(sb + half * BK * 2, it.mB, full_bar(stage), kb * BK, half, pol_b);
+          } else {
+            tma_load_2d(sb, it.mB, full_bar(stage), kb * BK, it.bcol, pol_b);
+            if (B2) tma_load_2d(sb + b_tile, it.mB2, full_bar(stage), kb * BK, it.bcol, pol_b);
+          }
+          if (++stage == S) { stage = 0; phase ^= 1u; }
+        }
+      }
+      if (PAIR && ok) {
+        // every stage released by both CTAs: the peer's last commits have
+        // reached this CTA's barriers
+        for (int s = 0; s < S; ++s) {
+          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
       }
@@ -303,9 +339,12 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
       bool ok = true;
       for (int i = 0; i < nitems && ok; ++i) {
         const TcItem it = w.get(i);
-        const uint32_t idesc = idesc_bf16(it.dp, TRANS);
-        const int acc = i & 1;
-        const uint32_t use = (uint32_t)(i >> 1);
+        // wide items (more than 256 columns) take both accumulators, half of
+        // the columns each
+        const bool wide = kWide && it.dp > 256;
+        const uint32_t idesc = idesc_bf16(wide ? it.dp / 2 : it.dp, TRANS);
+        const int acc = wide ? 0 : i & 1;
+        const uint32_t use = (uint32_t)(wide ? i : i >> 1);
         if (!mbar_wait(tempty_bar(acc), (use & 1u) ^ 1u, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + (uint32_t)(acc * 256);
@@ -321,8 +360,12 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
             bd = sdesc(sb + kk * 32, 16, 1024);
             mma_bf16(tmem_d, ad, bd, idesc, (kb > it.kb0 || kk > 0) ? 1u : 0u);
             if (B2) mma_bf16(tmem_d, ad, sdesc(sb + b_tile + kk * 32, 16, 1024), idesc, 1u);
+            if (wide)
+              mma_bf16(tmem_d + 256, ad, sdesc(sb + it.dp / 2 * BK * 2 + kk * 32, 16, 1024), idesc,
+                       (kb > it.kb0 || kk > 0) ? 1u : 0u);
           }
-          mma_commit(empty_bar(stage));
+          if (PAIR) mma_commit_mc(empty_bar(stage), 3);
+          else mma_commit(empty_bar(stage));
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
@@ -341,8 +384,9 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
     bool ok = true;
     for (int i = 0; i < nitems && ok; ++i) {
       const TcItem it = w.get(i);
-      const int acc = i & 1;
-      const uint32_t use = (uint32_t)(i >> 1);
+      const bool wide = kWide && it.dp > 256;
+      const int acc = wide ? 0 : i & 1;
+      const uint32_t use = (uint32_t)(wide ? i : i >> 1);
       // the warp agrees on the outcome before its collective TMEM loads
       if (!__all_sync(0xffffffffu, mbar_wait(tfull_bar(acc), use & 1u, abort_flag))) {
         ok = false;
@@ -354,11 +398,13 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
       float* dst = it.out + (int64_t)row * it.ldo;
       for (int c = 0; c < it.dp; c += 16) {
         float v[16];
-        tmem_ld16(taddr + c, v);
+        tmem_ld16(taddr + (wide && c >= it.dp / 2 ? 256 + c - it.dp / 2 : c), v);
         if (valid) {
           float4* d4 = reinterpret_cast<float4*>(dst + c);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) d4[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+          for (int j = 0; j < 4; ++j)
+            if (W::kGlobalMaps || c + 4 * j < it.cols)  // (a batch stores whole chunks)
+              d4[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
         }
       }
       tc_fence_before();
@@ -374,14 +420,16 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base)
                  : "memory");
   }
+  // neither CTA leaves while the other's copies or commits may still reach it
+  if (PAIR) cluster_sync();
 }
 
-template <bool TRANS, bool B2>
+template <bool TRANS, bool B2, bool PAIR>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
           const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ TcParams p) {
   const WorkSingle w{&tmA, &tmB, &tmB2, &p};
-  tc_body<TRANS, B2>(w, p.err, p.stages, p.dpi, p.withhold);
+  tc_body<TRANS, B2, PAIR>(w, p.err, p.stages, p.dpi, p.withhold);
 }
 
 template <bool TRANS, bool B2>
@@ -389,7 +437,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 k_btc_gemm(const BTcTile* __restrict__ list, int n, const BMat* __restrict__ T,
            const CUtensorMap* __restrict__ maps, int dst, int stages, int dpmax, int* err) {
   const WorkBatch w{list, n, T, maps, dst, TRANS};
-  tc_body<TRANS, B2>(w, err, stages, dpmax);
+  tc_body<TRANS, B2, false>(w, err, stages, dpmax);
 }
 
 // Sum the stream-K fragments of each tail tile in CTA order into the output.
@@ -401,7 +449,8 @@ __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
   __shared__ int s_cnt[8];
   pdl_launch();
   pdl_wait();
-  const int tt = blockIdx.x;  // tail tile index
+  // tail tile index (with pairs: member `mem` of pair tile tt; P counts pairs)
+  const int tt = blockIdx.x >> p.pair, mem = p.pair ? (int)(blockIdx.x & 1) : 0;
   const int64_t KB = p.KB;
   const int64_t lo = tt * KB, hi = lo + KB;
   // the contributors are consecutive CTAs starting near lo P / U (at most
@@ -426,16 +475,17 @@ __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
     if (k < w) pos += s_cnt[k];
     n += s_cnt[k];
   }
-  if (f) s_src[pos] = cc * 2 + slot;
+  if (f) s_src[pos] = ((cc << p.pair) + mem) * 2 + slot;
   __syncthreads();
   // block (tt, y): rows 4 y .. 4 y + 3 of the tile, a thread per 4 columns
-  const int tile = p.full_waves * P + tt;
+  const int tile = ((p.full_waves * P + tt) << p.pair) + mem;
   const int mt = tile / p.ns, col0 = (tile - mt * p.ns) * p.dpi;
-  const int q4 = p.dpi / 4;
-  const int r = blockIdx.y * 4 + threadIdx.x / 64, c4 = threadIdx.x % 64;
+  const int q4 = p.dpi / 4, qs = min(p.dpi, p.cols - col0) / 4;  // stored
+  const int r = blockIdx.y * 4 + threadIdx.x / 64;
   const int64_t gr = (int64_t)mt * BM + r;
-  if (gr >= p.Mout || c4 >= q4) return;
+  if (gr >= p.Mout) return;
   const float4* frag = reinterpret_cast<const float4*>(p.frag);
+  for (int c4 = threadIdx.x % 64; c4 < qs; c4 += 64) {
   // sixteen 16-byte loads in flight, summed in contributor order
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int i = 0; i < n; i += 16) {
@@ -453,33 +503,57 @@ __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
       }
   }
   *reinterpret_cast<float4*>(p.out + gr * p.ldo + col0 + 4 * c4) = s;
+  }
 }
 
 // dst[c][r] = bf16(src[r][c]) for c < cols, 0 for cols <= c < dp (r < rows);
 // lo (optional): the low part, bf16(src[r][c] - dst[c][r]).
+// A block takes 128 rows x 32 columns (16 loads in flight per thread) and writes
+// four rows' values of a column at a time (20000 x 220: 10.8 us with 32 x 32
+// blocks and single values).
+constexpr int TR_R = 128;
 template <typename TS>
-__global__ void k_transpose_bf16(const TS* __restrict__ src, int64_t lds, int64_t rows, int cols,
-                                 int dp, __nv_bfloat16* __restrict__ dst, int64_t ldd,
-                                 __nv_bfloat16* __restrict__ lo) {
-  __shared__ float t[32][33];
-  const int64_t r0 = (int64_t)blockIdx.x * 32;
+__global__ void __launch_bounds__(256)
+k_transpose_bf16(const TS* __restrict__ src, int64_t lds, int64_t rows, int cols, int dp,
+                 __nv_bfloat16* __restrict__ dst, int64_t ldd, __nv_bfloat16* __restrict__ lo) {
+  __shared__ float t[32][TR_R + 4];
+  const int64_t r0 = (int64_t)blockIdx.x * TR_R;
   const int c0 = blockIdx.y * 32;
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int64_t r = r0 + i;
-    const int c = c0 + threadIdx.x;
-    float v = 0.f;
-    if (r < rows && c < cols) v = (float)src[r * lds + c];
-    t[i][threadIdx.x] = v;
+  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+  float v[TR_R / 8];
+#pragma unroll
+  for (int q = 0; q < TR_R / 8; ++q) {
+    const int64_t r = r0 + ty + 8 * q;
+    v[q] = (r < rows && c0 + tx < cols) ? (float)src[r * lds + c0 + tx] : 0.f;
   }
+#pragma unroll
+  for (int q = 0; q < TR_R / 8; ++q) t[tx][ty + 8 * q] = v[q];
   __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int c = c0 + i;
-    const int64_t r = r0 + threadIdx.x;
-    if (c < dp && r < rows) {
-      const float v = t[threadIdx.x][i];
-      const __nv_bfloat16 h = __float2bfloat16_rn(v);
-      dst[(int64_t)c * ldd + r] = h;
-      if (lo != nullptr) lo[(int64_t)c * ldd + r] = __float2bfloat16_rn(v - __bfloat162float(h));
+  // (dst rows start on 16 bytes, their pitch a multiple of 8)
+  const int64_t r = r0 + 4 * tx;
+  for (int i = ty; i < 32 && c0 + i < dp; i += 8) {
+    if (r >= rows) break;
+    const float4 x = *reinterpret_cast<const float4*>(&t[i][4 * tx]);
+    const float f[4] = {x.x, x.y, x.z, x.w};
+    __nv_bfloat16 h[4], l[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      h[j] = __float2bfloat16_rn(f[j]);
+      l[j] = __float2bfloat16_rn(f[j] - __bfloat162float(h[j]));
+    }
+    const int64_t o = (int64_t)(c0 + i) * ldd + r;
+    if (r + 4 <= rows) {
+      auto pack = [](const __nv_bfloat16 (&a)[4]) {
+        return make_uint2(__bfloat16_as_ushort(a[0]) | (uint32_t)__bfloat16_as_ushort(a[1]) << 16,
+                          __bfloat16_as_ushort(a[2]) | (uint32_t)__bfloat16_as_ushort(a[3]) << 16);
+      };
+      *reinterpret_cast<uint2*>(dst + o) = pack(h);
+      if (lo != nullptr) *reinterpret_cast<uint2*>(lo + o) = pack(l);
+    } else {
+      for (int j = 0; j < 4 && r + j < rows; ++j) {
+        dst[o + j] = h[j];
+        if (lo != nullptr) lo[o + j] = l[j];
+      }
     }
   }
 }
@@ -825,6 +899,16 @@ bool tc_supported(const void* A, int64_t lda, int dp) {
          encode_fn() != nullptr;
 }
 
+// Sketches of 257 .. 384 columns in one pass over A (their columns in two halves,
+// multiples of 16 each) when A exceeds the 126 MB L2, so that a second pass would
+// come from HBM again: a stage is 16 KB of A and up to 48 KB of the skinny
+// operand, at least three deep.  16384 x 8192 transposed at d = 272: the call
+// 186 us in two passes of 144 columns, 136 us in one.
+static bool tc_wide_dp(int dp) { return dp > 256 && dp <= 384 && dp % 32 == 0; }
+bool tc_wide_fits(int64_t m, int64_t n, int dp) {
+  return tc_wide_dp(dp) && m * n * 2 > (int64_t)1 << 27;
+}
+
 size_t tc_frag_bytes(int dp) { return (size_t)sm_count() * 2 * BM * dp * sizeof(float); }
 
 // Rows per CTA (a multiple of the 64-row chunk) and the number of CTAs, every
@@ -905,7 +989,7 @@ namespace {
 
 // Launch configuration of one product: column split and ring depth.
 struct TcCfg {
-  int ns = 1, stages = 0;
+  int ns = 1, stages = 0, pair = 0;
 };
 
 size_t tc_stage_bytes(int dp, int ns, bool b2) {
@@ -924,8 +1008,10 @@ void tune_save_line(const std::array<int64_t, 5>& key, const TcCfg& c, double us
   if (g_tune_path.empty()) return;
   FILE* f = fopen(g_tune_path.c_str(), "a");
   if (!f) return;
+  // (pairs: split 1, 64 added to the stages)
   fprintf(f, "tc_gemm %lld %lld %lld %lld %lld %d %d %.3f\n", (long long)key[0], (long long)key[1],
-          (long long)key[2], (long long)key[3], (long long)key[4], c.ns, c.stages, us);
+          (long long)key[2], (long long)key[3], (long long)key[4], c.ns,
+          c.pair ? c.stages + 64 : c.stages, us);
   fclose(f);
 }
 
@@ -933,7 +1019,7 @@ struct TcOperands {
   bool trans, b2;
   const void *A, *Bt, *Btl;
   int64_t lda, m, n, ldb, ldo;
-  int dp;
+  int dp, cols;
   float *out, *frag;
   int* err;
 };
@@ -946,10 +1032,11 @@ cudaError_t tc_launch(const TcOperands& o, const TcCfg& c, cudaStream_t st,
   CUtensorMap mA, mB, mB2;
   if (!make_map(&mA, o.A, (uint64_t)o.n, (uint64_t)o.m, (uint64_t)o.lda, 64, o.trans ? 64 : BM))
     return cudaErrorInvalidValue;
-  if (!make_map(&mB, o.Bt, (uint64_t)K, (uint64_t)o.dp, (uint64_t)o.ldb, 64, (uint32_t)dpi))
+  const uint32_t brows = (uint32_t)(dpi > 256 ? dpi / 2 : dpi >> c.pair);
+  if (!make_map(&mB, o.Bt, (uint64_t)K, (uint64_t)o.dp, (uint64_t)o.ldb, 64, brows))
     return cudaErrorInvalidValue;
   if (o.b2) {
-    if (!make_map(&mB2, o.Btl, (uint64_t)K, (uint64_t)o.dp, (uint64_t)o.ldb, 64, (uint32_t)dpi))
+    if (!make_map(&mB2, o.Btl, (uint64_t)K, (uint64_t)o.dp, (uint64_t)o.ldb, 64, brows))
       return cudaErrorInvalidValue;
   } else {
     mB2 = mB;  // unused
@@ -960,13 +1047,16 @@ cudaError_t tc_launch(const TcOperands& o, const TcCfg& c, cudaStream_t st,
   p.dp = o.dp;
   p.ns = c.ns;
   p.dpi = dpi;
+  p.cols = o.cols;
   p.out = o.out;
   p.ldo = o.ldo;
   p.frag = o.frag;
   p.err = o.err;
-  p.T = ceil_div(Mout, BM) * c.ns;
+  p.pair = c.pair;
+  p.T = c.pair ? ceil_div(Mout, 2 * BM) : ceil_div(Mout, BM) * c.ns;
   p.KB = ceil_div(K, BK);
-  int P = sm_count();  // never more CTAs than the fragment buffer has slots for
+  // CTAs (or pairs): never more than the fragment buffer has slots for
+  int P = sm_count() >> c.pair;
   if ((int64_t)p.T * p.KB < P) P = p.T * p.KB;
   p.full_waves = p.T / P;
   p.tail = p.T - p.full_waves * P;
@@ -974,17 +1064,20 @@ cudaError_t tc_launch(const TcOperands& o, const TcCfg& c, cudaStream_t st,
   p.stages = c.stages;
   p.withhold = withhold;
   const size_t smem = tc_smem(c.stages, tc_stage_bytes(o.dp, c.ns, o.b2));
-  auto kern = o.trans ? (o.b2 ? k_tc_gemm<true, true> : k_tc_gemm<true, false>)
-                      : (o.b2 ? k_tc_gemm<false, true> : k_tc_gemm<false, false>);
+  auto kern = c.pair ? (o.trans ? (o.b2 ? k_tc_gemm<true, true, true> : k_tc_gemm<true, false, true>)
+                                : (o.b2 ? k_tc_gemm<false, true, true> : k_tc_gemm<false, false, true>))
+                     : (o.trans ? (o.b2 ? k_tc_gemm<true, true, false> : k_tc_gemm<true, false, false>)
+                                : (o.b2 ? k_tc_gemm<false, true, false> : k_tc_gemm<false, false, false>));
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (mark) mark(true);
-  e = launch_pdl(kern, dim3(P), dim3(NTHREADS), smem, st, mA, mB, mB2, p);
+  e = c.pair ? launch_pdl_cluster(kern, dim3(2 * P), dim3(NTHREADS), smem, 2, st, mA, mB, mB2, p)
+             : launch_pdl(kern, dim3(P), dim3(NTHREADS), smem, st, mA, mB, mB2, p);
   if (mark) mark(false);
   count_launch();
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess || p.tail == 0) return e;
-  e = launch_pdl(k_tc_fixup, dim3(p.tail, BM / 4), dim3(256), 0, st, p, P);
+  e = launch_pdl(k_tc_fixup, dim3(p.tail << c.pair, BM / 4), dim3(256), 0, st, p, P);
   count_launch();
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
@@ -1004,12 +1097,16 @@ int tune_file(const char* path) {
   double us;
   while (fscanf(f, "%31s %lld %lld %lld %lld %lld %d %d %lf", tag, &k0, &k1, &k2, &k3, &k4, &ns,
                 &stages, &us) == 9) {
-    if (strcmp(tag, "tc_gemm") != 0 || !tc_ns_valid((int)k4, ns) || stages < 2 ||
+    const bool pair = stages > 64;
+    if (pair) stages -= 64;
+    if (strcmp(tag, "tc_gemm") != 0 || (pair && ns != 1) || !tc_ns_valid((int)k4, ns) ||
+        stages < 2 ||
         tc_smem(stages, tc_stage_bytes((int)k4, ns, k1 != 0)) > 226 * 1024)
       continue;
     TcCfg c;
     c.ns = ns;
     c.stages = stages;
+    c.pair = pair;
     g_tune[{k0, k1, k2, k3, k4}] = c;
     ++n;
   }
@@ -1018,26 +1115,31 @@ int tune_file(const char* path) {
 }
 
 // Products of one shape run with the configuration measured fastest the
-// first time that shape is seen (outside stream capture): every valid
-// column split ns in {1, 2, 4} with the deepest ring that fits, each timed
+// first time that shape is seen (outside stream capture): CTA pairs and every
+// valid column split ns in {1, 2, 4} with the deepest ring that fits, each timed
 // twice with CUDA events on the stream (the better time counts); the chosen
 // configuration then computes the result, so repeated calls are bitwise
 // equal.  force_ns > 0 skips the tuner.
 cudaError_t tc_gemm(bool trans, const void* A, int64_t lda, int64_t m, int64_t n, const void* Bt,
                     int64_t ldb, int dp, float* out, int64_t ldo, float* frag, int* err,
                     cudaStream_t st, const std::function<void(bool)>& mark, const void* Btl,
-                    int force_ns, int withhold) {
-  if (dp < 16 || dp > 256 || dp % 16 != 0) return cudaErrorInvalidValue;
+                    int force_ns, int withhold, int cols) {
+  const bool wide = dp > 256;
+  if (dp < 16 || dp % 16 != 0 || (wide && (!tc_wide_dp(dp) || Btl != nullptr)))
+    return cudaErrorInvalidValue;
+  if (cols <= 0) cols = dp;
+  if (cols % 4 != 0 || cols > dp) return cudaErrorInvalidValue;
   if (lda % 8 != 0 || ldb % 8 != 0 || ((uintptr_t)A & 15) || ((uintptr_t)Bt & 15) || ldo % 4 != 0 ||
       ((uintptr_t)out & 15) || ((uintptr_t)Btl & 15))
     return cudaErrorInvalidValue;
-  TcOperands o{trans, Btl != nullptr, A, Bt, Btl, lda, m, n, ldb, ldo, dp, out, frag, err};
+  TcOperands o{trans, Btl != nullptr, A, Bt, Btl, lda, m, n, ldb, ldo, dp, cols, out, frag, err};
   auto cfg_of = [&](int ns) {
     TcCfg c;
     c.ns = ns;
     c.stages = tc_stages(tc_stage_bytes(dp, ns, o.b2));
     return c;
   };
+  if (wide) return tc_launch(o, cfg_of(1), st, mark, withhold);
   if (force_ns > 0) {
     if (!tc_ns_valid(dp, force_ns)) return cudaErrorInvalidValue;
     const TcCfg c = cfg_of(force_ns);
@@ -1061,10 +1163,14 @@ cudaError_t tc_gemm(bool trans, const void* A, int64_t lda, int64_t m, int64_t n
   }
   TcCfg best = cfg_of(1);
   float best_ms = 1e30f;
-  for (int ns : {1, 2, 4}) {
+  for (int cand : {1, 0, 2, 4}) {  // 0: CTA pairs
+    const int ns = std::max(cand, 1);
     if (!tc_ns_valid(dp, ns)) continue;
-    const TcCfg c = cfg_of(ns);
-    if (c.stages < 2) continue;
+    TcCfg c = cfg_of(ns);
+    c.pair = cand == 0;
+    // (pairs from 16 tiles on: below, one tile more or less changes a CTA's K
+    // range, and with it the truncation of the tensor core's sums)
+    if (c.stages < 2 || (c.pair && (sm_count() < 2 || ceil_div(Mout, BM) < 16))) continue;
     float t = 1e30f;
     for (int rep = 0; rep < 2; ++rep) {
       cudaEventRecord(e0, st);
@@ -1136,7 +1242,8 @@ cudaError_t btc_gemm(bool trans, const BMat* T, int count, const BTcTile* list, 
 
 cudaError_t transpose_to_bf16(Ty ts, const void* src, int64_t lds, int64_t rows, int cols, int dp,
                               void* dst, int64_t ldd, cudaStream_t st, void* lo) {
-  dim3 grid(ceil_div(rows, 32), ceil_div(dp, 32)), block(32, 8);
+  if (ldd % 4 || ((uintptr_t)dst & 7) || ((uintptr_t)lo & 7)) return cudaErrorInvalidValue;
+  dim3 grid(ceil_div(rows, TR_R), ceil_div(dp, 32)), block(32, 8);
   if (ts == Ty::F64)
     k_transpose_bf16<double><<<grid, block, 0, st>>>((const double*)src, lds, rows, cols, dp,
                                                      (__nv_bfloat16*)dst, ldd,

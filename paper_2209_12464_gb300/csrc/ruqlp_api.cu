@@ -130,7 +130,8 @@ inline int64_t round8(int64_t x) { return (x + 7) / 8 * 8; }
 
 // nnz >= 0: A is CSR with nnz nonzeros of val_bytes each (CSC copy kept too).
 // finish: room for Algorithm 1 step 5 (an m x dp buffer for Q P~).
-// img: room for the split skinny operand of an FP32 product (L.Bt).
+// img: room for the split skinny operand of an FP32 product (L.Bt) and for the
+// fragments of a one-pass BF16 product of 257 .. 384 columns.
 // tsqr: room for the Householder TSQR orth() (the rank-deficiency fallback).
 Layout layout_of(int64_t m, int64_t n, int d, Ty ct, int64_t nnz = -1, size_t val_bytes = 0,
                  int finish = 0, bool gen_omega = false, int64_t lr_r = 0, bool tsqr = false,
@@ -169,7 +170,8 @@ Layout layout_of(int64_t m, int64_t n, int d, Ty ct, int64_t nnz = -1, size_t va
     const size_t one = (size_t)dp * round8(m > n ? m : n) * 2;
     L.Bt = take(2 * one);
     L.Btl = L.Bt + one;
-    L.frag = take(tc_frag_bytes(dp <= 256 ? dp : 256));  // per column chunk
+    const int dpw = (dp + 31) / 32 * 32;
+    L.frag = take(tc_frag_bytes(dp <= 256 ? dp : img && tc_wide_fits(m, n, dpw) ? dpw : 256));  // per chunk
   }
   if (ct == Ty::F32 && nnz < 0 && img && f32_tc_supported(std::max(m, n)))
     L.Bt = take(f32_img_bytes(std::max(m, n), dp));
@@ -297,6 +299,8 @@ struct Job {
   bool use_tc;  // BF16 products on the tensor cores (k_tc.cu)
   bool f32_tc[2] = {false, false};  // FP32 A X, A^T Y on the tensor cores (k_f32tc.cu)
   int x_cols = 0;       // readable columns of a caller's skinny operand (0: an arena buffer)
+  int64_t out_ld = 0;   // a product straight into a caller's buffer: its leading
+                        // dimension, d columns stored (0: an arena buffer, ld dp)
   // CSR input (work type FP32): A's arrays and the CSC copy in the arena
   bool csr = false;
   const int32_t* rowptr = nullptr;
@@ -431,6 +435,7 @@ ruqlp_status product(ruqlp_ctx* h, const Layout& Lo, const Job& J, bool trans, T
   char* base = (char*)h->arena;
   const int64_t K = trans ? J.m : J.n;
   const int64_t Mout = trans ? J.n : J.m;
+  const int64_t ldo = J.out_ld ? J.out_ld : J.dp;
   if (J.csr) {
     if (xt != Ty::F32) return fail(h, RUQLP_ERR_INVALID, "internal: CSR operand type");
     if (!trans)
@@ -469,16 +474,20 @@ ruqlp_status product(ruqlp_ctx* h, const Layout& Lo, const Job& J, bool trans, T
     void* Bt = base + Lo.Bt;
     void* Btl = split2 ? base + Lo.Btl : nullptr;
     const int64_t ldb = round8(K);
-    const int nch = (J.dp + 255) / 256;
-    const int w = round16((J.dp + nch - 1) / nch);
+    // (up to 384 in one when a second pass would read A from HBM again and the
+    // workspace has room for the fragments)
+    const int dpw = (J.dp + 31) / 32 * 32;
+    const bool wide = !split2 && h->f32_img && h->tc_nsplit <= 1 && tc_wide_fits(J.m, J.n, dpw);
+    const int nch = wide ? 1 : (J.dp + 255) / 256;
+    const int w = wide ? dpw : round16((J.dp + nch - 1) / nch);
     const size_t xes = ty_size(xt);
     for (int c0 = 0; c0 < J.dp; c0 += w) {
-      const int wc = std::min(w, J.dp - c0);
+      const int wc = wide ? w : std::min(w, J.dp - c0);
       const int cols = std::max(0, std::min(J.d - c0, wc));
       if (!(bt_ready && nch == 1))  // else the last solve of orth() wrote it
         CK(transpose_to_bf16(xt, (const char*)Xin + (size_t)c0 * xes, ldx, K, cols, wc, Bt, ldb,
                              st, Btl));
-      CK(tc_gemm(trans, J.A, J.lda, J.m, J.n, Bt, ldb, wc, (float*)out + c0, J.dp,
+      CK(tc_gemm(trans, J.A, J.lda, J.m, J.n, Bt, ldb, wc, (float*)out + c0, ldo,
                  (float*)(base + Lo.frag), &h->status->timeout, st,
                  h->profile ? [&](bool begin) {
                    static thread_local cudaEvent_t a;
@@ -489,7 +498,8 @@ ruqlp_status product(ruqlp_ctx* h, const Layout& Lo, const Job& J, bool trans, T
                      h->spans.push_back(
                          {trans ? (split2 ? PROF_TC_ATX2 : PROF_TC_ATX) : PROF_TC_AX, a, b});
                    }
-                 } : std::function<void(bool)>(), Btl, h->tc_nsplit, h->test_withhold));
+                 } : std::function<void(bool)>(), Btl, h->tc_nsplit, h->test_withhold,
+                 std::min(wc, (J.out_ld ? J.d : J.dp) - c0)));
     }
     return RUQLP_OK;
   }
@@ -499,8 +509,8 @@ ruqlp_status product(ruqlp_ctx* h, const Layout& Lo, const Job& J, bool trans, T
   const int32_t* redo = nullptr;
   if (J.f32_tc[trans]) {
     CK(f32_gemm_tc(trans, (const float*)J.A, J.lda, J.m, J.n, (const float*)Xin, ldx,
-                   J.x_cols ? J.x_cols : J.dp, J.d, J.dp, (float*)out, J.dp,
-                   (float*)(base + Lo.partial), Lo.Bt ? base + Lo.Bt : nullptr, h->status, st));
+                   J.x_cols ? J.x_cols : J.dp, J.d, J.dp, (float*)out, ldo,
+                   J.out_ld ? J.d : J.dp, (float*)(base + Lo.partial), Lo.Bt ? base + Lo.Bt : nullptr, h->status, st));
     redo = &h->status->range;
   }
   if (J.ct == Ty::BF16 && split2) {
@@ -521,10 +531,10 @@ ruqlp_status product(ruqlp_ctx* h, const Layout& Lo, const Job& J, bool trans, T
     ldx = J.d;
   }
   if (!trans)
-    CK(simt_gemm_nn(J.ct, xt, J.wt, mul, J.A, J.lda, Xin, ldx, out, J.dp, Mout, K, J.d, st,
+    CK(simt_gemm_nn(J.ct, xt, J.wt, mul, J.A, J.lda, Xin, ldx, out, ldo, Mout, K, J.d, st,
                     redo));
   else
-    CK(simt_gemm_tn(J.ct, xt, J.wt, mul, J.A, J.lda, Xin, ldx, out, J.dp, Mout, K, J.d, 1,
+    CK(simt_gemm_tn(J.ct, xt, J.wt, mul, J.A, J.lda, Xin, ldx, out, ldo, Mout, K, J.d, 1,
                     nullptr, nullptr, st, redo));
   return RUQLP_OK;
 }
@@ -1491,9 +1501,10 @@ ruqlp_status ruqlp_reserve(ruqlp_handle h, int64_t m, int64_t n, int d, ruqlp_dt
   if (!h) return RUQLP_ERR_INVALID;
   const size_t b = ruqlp_workspace_bytes(m, n, d, compute, nnz);
   if (b == 0) return fail(h, RUQLP_ERR_INVALID, "invalid sizes for ruqlp_reserve");
-  return ensure_arena(h, nnz < 0 && compute == RUQLP_F32 && h->f32_img
-                             ? layout_of(m, n, d, Ty::F32, -1, 0, 0, false, 0, false, true).total
-                             : b);
+  Ty ct = Ty::F32;
+  ty_of(compute, &ct);
+  return ensure_arena(h, nnz < 0 ? layout_of(m, n, d, ct, -1, 0, 0, false, 0, false, h->f32_img).total
+                                 : b);
 }
 
 ruqlp_status ruqlp_decompose(ruqlp_handle h, const ruqlp_matrix* A, const ruqlp_params* prm,
@@ -1706,9 +1717,22 @@ ruqlp_status ruqlp_sketch(ruqlp_handle h, const ruqlp_matrix* A, int trans, cons
     Xuse = Xa;
     ldxu = J.dp;
   }
-  s = product(h, Lo, J, trans != 0, J.wt, Xuse, ldxu, stage);
+  // straight into Y where its rows take the kernel's stores (the tensor-core
+  // kernels write 16 bytes at a time) and it does not overlap an operand
+  const bool tc = J.use_tc || f32_tc;
+  const size_t wes = ty_size(J.wt);
+  auto apart = [&](const void* p, int64_t rows, int64_t ld, int64_t cols, size_t es) {
+    const uintptr_t a0 = (uintptr_t)p, a1 = a0 + ((size_t)(rows - 1) * ld + cols) * es;
+    const uintptr_t y0 = (uintptr_t)Y, y1 = y0 + ((size_t)(Mout - 1) * ldy + d) * wes;
+    return a1 <= y0 || y1 <= a0;
+  };
+  const bool direct = !J.csr && (!tc || (d % 4 == 0 && ldy % 4 == 0 && ((uintptr_t)Y & 15) == 0)) &&
+                      apart(X, trans ? m : n, ldx, d, wes) &&
+                      apart(J.A, m, J.lda, n, ty_size(J.ct));
+  if (direct) J.out_ld = ldy;
+  s = product(h, Lo, J, trans != 0, J.wt, Xuse, ldxu, direct ? Y : stage);
   if (s != RUQLP_OK) return s;
-  CK(copy_cast_2d(J.wt, stage, J.dp, J.wt, Y, ldy, Mout, d, h->stream));
+  if (!direct) CK(copy_cast_2d(J.wt, stage, J.dp, J.wt, Y, ldy, Mout, d, h->stream));
   ruqlp_outputs dummy{};
   return finish(h, &dummy);
 }

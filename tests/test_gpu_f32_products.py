@@ -75,3 +75,26 @@ def test_special_values_and_range(handles, trans):
     Y = h.sketch(B, X, trans)
     _check(Y, B, X, trans)
     assert bool((Y[4] == 0).all())
+
+
+@pytest.mark.parametrize("m,n,d", [(4100, 1024, 220), (2049, 520, 16), (5000, 4096, 224),
+                                   (16392, 4104, 257), (4100, 16400, 272), (8200, 8207, 384),
+                                   (640, 808, 272), (500, 1200, 385)])
+@pytest.mark.parametrize("trans", [False, True])
+def test_bf16_products_pairs_and_wide(handles, m, n, d, trans):
+    """BF16 products with the tuner free (CTA pairs among its choices) and of more
+    than 256 columns in one pass.  Every addition of a K-long accumulation may be
+    truncated by the tensor core: |error| <= (K / 16 + 160) 2^-23 sum |a x|."""
+    h = handles[0]
+    g = torch.Generator(device="cuda")
+    g.manual_seed(m + n + d)
+    n8 = (n + 7) // 8 * 8
+    A = torch.randn(m, n8, generator=g, device="cuda").bfloat16()[:, :n]
+    X = torch.randn(m if trans else n, d, generator=g, device="cuda")
+    Y = h.sketch(A, X, trans)
+    R, S = _ref(A, X.bfloat16(), trans)
+    assert bool(((Y.double() - R).abs() <= (X.shape[0] / 16 + 160) * 2.0 ** -23 * S).all())
+    assert torch.equal(Y, h.sketch(A, X, trans))
+    # a handle under a budget takes wide sketches in column chunks
+    Z = handles[1].sketch(A, X, trans)
+    assert bool(((Z.double() - R).abs() <= (X.shape[0] / 16 + 160) * 2.0 ** -23 * S).all())
