@@ -191,11 +191,11 @@ __device__ __forceinline__ void tmap_acquire(const CUtensorMap* m) {
 // free when both CTAs' MMAs have read it (each commits to both empty barriers).
 // 20000 x 20000 at d = 220: 165 -> 158 us a launch (the skinny operand's traffic
 // is not what bounds it: 0.77 of measured HBM).
-template <bool TRANS, bool B2, bool PAIR, class W>
+template <bool TRANS, bool B2, bool PAIR, bool WIDE, class W>
 __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
                                         int withhold = 0) {
-  // single one-part products may have items of more than 256 columns
-  constexpr bool kWide = !B2 && !PAIR && !W::kGlobalMaps;
+  // WIDE: items of more than 256 columns (one-part, not batched)
+  static_assert(!WIDE || (!B2 && !PAIR && !W::kGlobalMaps));
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -296,7 +296,7 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
             if (B2)
               tma_load_2d_mc(sb + b_tile + r * BK * 2, it.mB2, full_bar(stage), kb * BK, r, 3,
                              pol_b);
-          } else if (kWide && it.dp > 256) {  // wide: two boxes of half the columns
+          } else if constexpr (WIDE) {  // two boxes of half the columns
             const int half = it.dp / 2;
             tma_load_2d(sb, it.mB, full_bar(stage), kb * BK, 0, pol_b);
             tma_load_2d(sb + half * BK * 2, it.mB, full_bar(stage), kb * BK, half, pol_b);
@@ -341,7 +341,7 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
         const TcItem it = w.get(i);
         // wide items (more than 256 columns) take both accumulators, half of
         // the columns each
-        const bool wide = kWide && it.dp > 256;
+        constexpr bool wide = WIDE;
         const uint32_t idesc = idesc_bf16(wide ? it.dp / 2 : it.dp, TRANS);
         const int acc = wide ? 0 : i & 1;
         const uint32_t use = (uint32_t)(wide ? i : i >> 1);
@@ -384,7 +384,7 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
     bool ok = true;
     for (int i = 0; i < nitems && ok; ++i) {
       const TcItem it = w.get(i);
-      const bool wide = kWide && it.dp > 256;
+      constexpr bool wide = WIDE;
       const int acc = wide ? 0 : i & 1;
       const uint32_t use = (uint32_t)(wide ? i : i >> 1);
       // the warp agrees on the outcome before its collective TMEM loads
@@ -396,14 +396,28 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
       const uint32_t taddr = tmem_base + (uint32_t)(acc * 256) + ((uint32_t)(g * 32) << 16);
       const bool valid = row < it.rows;
       float* dst = it.out + (int64_t)row * it.ldo;
-      for (int c = 0; c < it.dp; c += 16) {
+      // whole chunks without a condition per store, so that the compiler keeps
+      // several chunks in flight (with one: a 9668 x 4912 product at d = 126 6 us
+      // slower); the last one may store 4, 8 or 12 columns
+      const int half = wide ? it.dp / 2 : it.dp;  // from here on, the second accumulator
+      const int whole = W::kGlobalMaps ? it.dp : it.cols & ~15;
+      for (int c = 0; c < whole; c += 16) {
         float v[16];
-        tmem_ld16(taddr + (wide && c >= it.dp / 2 ? 256 + c - it.dp / 2 : c), v);
+        tmem_ld16(taddr + c + (WIDE && c >= half ? 256 - half : 0), v);
         if (valid) {
           float4* d4 = reinterpret_cast<float4*>(dst + c);
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (W::kGlobalMaps || c + 4 * j < it.cols)  // (a batch stores whole chunks)
+          for (int j = 0; j < 4; ++j) d4[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        }
+      }
+      if (!W::kGlobalMaps && whole < it.cols) {
+        float v[16];
+        tmem_ld16(taddr + whole + (WIDE && whole >= half ? 256 - half : 0), v);
+        if (valid) {
+          float4* d4 = reinterpret_cast<float4*>(dst + whole);
+#pragma unroll
+          for (int j = 0; j < 3; ++j)
+            if (whole + 4 * j < it.cols)
               d4[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
         }
       }
@@ -424,12 +438,12 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
   if (PAIR) cluster_sync();
 }
 
-template <bool TRANS, bool B2, bool PAIR>
+template <bool TRANS, bool B2, bool PAIR, bool WIDE>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
           const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ TcParams p) {
   const WorkSingle w{&tmA, &tmB, &tmB2, &p};
-  tc_body<TRANS, B2, PAIR>(w, p.err, p.stages, p.dpi, p.withhold);
+  tc_body<TRANS, B2, PAIR, WIDE>(w, p.err, p.stages, p.dpi, p.withhold);
 }
 
 template <bool TRANS, bool B2>
@@ -437,20 +451,21 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 k_btc_gemm(const BTcTile* __restrict__ list, int n, const BMat* __restrict__ T,
            const CUtensorMap* __restrict__ maps, int dst, int stages, int dpmax, int* err) {
   const WorkBatch w{list, n, T, maps, dst, TRANS};
-  tc_body<TRANS, B2, false>(w, err, stages, dpmax);
+  tc_body<TRANS, B2, false, false>(w, err, stages, dpmax);
 }
 
 // Sum the stream-K fragments of each tail tile in CTA order into the output.
 // One block per (tail tile, 4 rows), one thread per 4 columns (16-byte loads,
 // up to 16 contributors in flight), after the block lists the tile's
 // contributing CTAs and fragment slots.
+template <bool PAIR, bool WIDE>
 __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
   __shared__ int s_src[256];
   __shared__ int s_cnt[8];
   pdl_launch();
   pdl_wait();
   // tail tile index (with pairs: member `mem` of pair tile tt; P counts pairs)
-  const int tt = blockIdx.x >> p.pair, mem = p.pair ? (int)(blockIdx.x & 1) : 0;
+  const int tt = blockIdx.x >> (int)PAIR, mem = PAIR ? (int)(blockIdx.x & 1) : 0;
   const int64_t KB = p.KB;
   const int64_t lo = tt * KB, hi = lo + KB;
   // the contributors are consecutive CTAs starting near lo P / U (at most
@@ -475,35 +490,36 @@ __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
     if (k < w) pos += s_cnt[k];
     n += s_cnt[k];
   }
-  if (f) s_src[pos] = ((cc << p.pair) + mem) * 2 + slot;
+  if (f) s_src[pos] = ((cc << (int)PAIR) + mem) * 2 + slot;
   __syncthreads();
   // block (tt, y): rows 4 y .. 4 y + 3 of the tile, a thread per 4 columns
-  const int tile = ((p.full_waves * P + tt) << p.pair) + mem;
+  const int tile = ((p.full_waves * P + tt) << (int)PAIR) + mem;
   const int mt = tile / p.ns, col0 = (tile - mt * p.ns) * p.dpi;
   const int q4 = p.dpi / 4, qs = min(p.dpi, p.cols - col0) / 4;  // stored
   const int r = blockIdx.y * 4 + threadIdx.x / 64;
   const int64_t gr = (int64_t)mt * BM + r;
-  if (gr >= p.Mout) return;
+  int c4 = threadIdx.x % 64;
+  if (gr >= p.Mout || c4 >= qs) return;
   const float4* frag = reinterpret_cast<const float4*>(p.frag);
-  for (int c4 = threadIdx.x % 64; c4 < qs; c4 += 64) {
-  // sixteen 16-byte loads in flight, summed in contributor order
-  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int i = 0; i < n; i += 16) {
-    float4 v[16];
-#pragma unroll
-    for (int u = 0; u < 16; ++u)
-      if (i + u < n) v[u] = frag[((int64_t)s_src[i + u] * BM + r) * q4 + c4];
-#pragma unroll
-    for (int u = 0; u < 16; ++u)
-      if (i + u < n) {
-        s.x += v[u].x;
-        s.y += v[u].y;
-        s.z += v[u].z;
-        s.w += v[u].w;
-      }
-  }
-  *reinterpret_cast<float4*>(p.out + gr * p.ldo + col0 + 4 * c4) = s;
-  }
+  do {  // (one column group per thread, two when wide)
+    // sixteen 16-byte loads in flight, summed in contributor order
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < n; i += 16) {
+      float4 v[16];
+  #pragma unroll
+      for (int u = 0; u < 16; ++u)
+        if (i + u < n) v[u] = frag[((int64_t)s_src[i + u] * BM + r) * q4 + c4];
+  #pragma unroll
+      for (int u = 0; u < 16; ++u)
+        if (i + u < n) {
+          s.x += v[u].x;
+          s.y += v[u].y;
+          s.z += v[u].z;
+          s.w += v[u].w;
+        }
+    }
+    *reinterpret_cast<float4*>(p.out + gr * p.ldo + col0 + 4 * c4) = s;
+  } while (WIDE && (c4 += 64) < qs);
 }
 
 // dst[c][r] = bf16(src[r][c]) for c < cols, 0 for cols <= c < dp (r < rows);
@@ -1064,10 +1080,13 @@ cudaError_t tc_launch(const TcOperands& o, const TcCfg& c, cudaStream_t st,
   p.stages = c.stages;
   p.withhold = withhold;
   const size_t smem = tc_smem(c.stages, tc_stage_bytes(o.dp, c.ns, o.b2));
-  auto kern = c.pair ? (o.trans ? (o.b2 ? k_tc_gemm<true, true, true> : k_tc_gemm<true, false, true>)
-                                : (o.b2 ? k_tc_gemm<false, true, true> : k_tc_gemm<false, false, true>))
-                     : (o.trans ? (o.b2 ? k_tc_gemm<true, true, false> : k_tc_gemm<true, false, false>)
-                                : (o.b2 ? k_tc_gemm<false, true, false> : k_tc_gemm<false, false, false>));
+  auto pick = [&](auto tr) {
+    constexpr bool TR = decltype(tr)::value;
+    if (dpi > 256) return k_tc_gemm<TR, false, false, true>;
+    if (c.pair) return o.b2 ? k_tc_gemm<TR, true, true, false> : k_tc_gemm<TR, false, true, false>;
+    return o.b2 ? k_tc_gemm<TR, true, false, false> : k_tc_gemm<TR, false, false, false>;
+  };
+  auto kern = o.trans ? pick(std::true_type{}) : pick(std::false_type{});
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (mark) mark(true);
@@ -1077,7 +1096,7 @@ cudaError_t tc_launch(const TcOperands& o, const TcCfg& c, cudaStream_t st,
   count_launch();
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess || p.tail == 0) return e;
-  e = launch_pdl(k_tc_fixup, dim3(p.tail << c.pair, BM / 4), dim3(256), 0, st, p, P);
+  e = launch_pdl(dpi > 256 ? k_tc_fixup<false, true> : c.pair ? k_tc_fixup<true, false> : k_tc_fixup<false, false>, dim3(p.tail << c.pair, BM / 4), dim3(256), 0, st, p, P);
   count_launch();
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
@@ -1115,8 +1134,8 @@ int tune_file(const char* path) {
 }
 
 // Products of one shape run with the configuration measured fastest the
-// first time that shape is seen (outside stream capture): CTA pairs and every
-// valid column split ns in {1, 2, 4} with the deepest ring that fits, each timed
+// first time that shape is seen (outside stream capture): every valid column
+// split ns in {1, 2, 4} with the deepest ring that fits, and CTA pairs, each timed
 // twice with CUDA events on the stream (the better time counts); the chosen
 // configuration then computes the result, so repeated calls are bitwise
 // equal.  force_ns > 0 skips the tuner.
@@ -1163,14 +1182,18 @@ cudaError_t tc_gemm(bool trans, const void* A, int64_t lda, int64_t m, int64_t n
   }
   TcCfg best = cfg_of(1);
   float best_ms = 1e30f;
-  for (int cand : {1, 0, 2, 4}) {  // 0: CTA pairs
+  for (int cand : {1, 2, 4, 0}) {  // 0: CTA pairs
     const int ns = std::max(cand, 1);
     if (!tc_ns_valid(dp, ns)) continue;
     TcCfg c = cfg_of(ns);
     c.pair = cand == 0;
     // (pairs from 16 tiles on: below, one tile more or less changes a CTA's K
-    // range, and with it the truncation of the tensor core's sums)
-    if (c.stages < 2 || (c.pair && (sm_count() < 2 || ceil_div(Mout, BM) < 16))) continue;
+    // range, and with it the truncation of the tensor core's sums;
+    // and where A exceeds the 126 MB L2: 9668 x 4912 at d = 126, 95 MB, measured 81 us
+    // in pairs against 68 with ns = 2 once the operands alternate)
+    if (c.stages < 2 || (c.pair && (sm_count() < 2 || ceil_div(Mout, BM) < 16 ||
+                                    m * n * 2 <= (int64_t)1 << 27)))
+      continue;
     float t = 1e30f;
     for (int rep = 0; rep < 2; ++rep) {
       cudaEventRecord(e0, st);

@@ -79,7 +79,7 @@ def test_special_values_and_range(handles, trans):
 
 @pytest.mark.parametrize("m,n,d", [(4100, 1024, 220), (2049, 520, 16), (5000, 4096, 224),
                                    (16392, 4104, 257), (4100, 16400, 272), (8200, 8207, 384),
-                                   (640, 808, 272), (500, 1200, 385)])
+                                   (640, 808, 272), (500, 1200, 385), (20000, 4096, 220)])
 @pytest.mark.parametrize("trans", [False, True])
 def test_bf16_products_pairs_and_wide(handles, m, n, d, trans):
     """BF16 products with the tuner free (CTA pairs among its choices) and of more
