@@ -178,37 +178,44 @@ k_trsm(const T* __restrict__ Y, int64_t ldy, const T* __restrict__ R, T* __restr
   }
 }
 
-// Four columns per thread, with vector loads and stores where the rows of both
-// sides start on them (vec), and 32-bit index arithmetic below 2^31 groups
-// (20000 x 220 FP32: 12.9 us with one element and a 64-bit division per thread).
+// Rows whose starts take 4-wide loads and stores on both sides (vec): four
+// columns per thread; else one element per thread (four, consecutive or a block
+// apart, measured 3 to 10 us slower on small copies).  32-bit index arithmetic
+// below 2^31 items.  20000 x 220 FP32: 12.9 us with one element and a 64-bit division
+// per thread, 5.3 with vec.
 template <typename T> struct alignas(4 * sizeof(T)) Quad { T v[4]; };
+__device__ __forceinline__ void split_index(int64_t idx, int64_t total, int per, int64_t& i, int& j) {
+  if (total < (int64_t)1 << 31) {
+    const uint32_t q = (uint32_t)idx / (uint32_t)per;
+    i = q;
+    j = (int)((uint32_t)idx - q * (uint32_t)per);
+  } else {
+    i = idx / per;
+    j = (int)(idx - i * per);
+  }
+}
 template <typename TS, typename TD>
-__global__ void k_copy_cast(const TS* __restrict__ src, int64_t lds, TD* __restrict__ dst,
-                            int64_t ldd, int64_t rows, int cols, bool vec) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int g = (cols + 3) / 4;
+__global__ void __launch_bounds__(256)
+k_copy_cast(const TS* __restrict__ src, int64_t lds, TD* __restrict__ dst, int64_t ldd,
+            int64_t rows, int cols, bool vec) {
   int64_t i;
   int j;
-  if (rows * g < (int64_t)1 << 31) {
-    const uint32_t q = (uint32_t)idx / (uint32_t)g;
-    i = q;
-    j = (int)((uint32_t)idx - q * (uint32_t)g) * 4;
-  } else {
-    i = idx / g;
-    j = (int)(idx - i * g) * 4;
-  }
-  if (i >= rows) return;
-  const TS* s = src + i * lds + j;
-  TD* o = dst + i * ldd + j;
-  if (vec && j + 4 <= cols) {
-    const Quad<TS> x = *reinterpret_cast<const Quad<TS>*>(s);
+  if (vec) {
+    const int g = cols / 4;
+    const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (idx >= rows * g) return;
+    split_index(idx, rows * g, g, i, j);
+    const Quad<TS> x = *reinterpret_cast<const Quad<TS>*>(src + i * lds + 4 * j);
     Quad<TD> y;
 #pragma unroll
     for (int u = 0; u < 4; ++u) y.v[u] = Cvt<TD>::from(x.v[u]);
-    *reinterpret_cast<Quad<TD>*>(o) = y;
-  } else {
-    for (int u = 0; u < 4 && j + u < cols; ++u) o[u] = Cvt<TD>::from(s[u]);
+    *reinterpret_cast<Quad<TD>*>(dst + i * ldd + 4 * j) = y;
+    return;
   }
+  const int64_t tot = rows * cols, idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (idx >= tot) return;
+  split_index(idx, tot, cols, i, j);
+  dst[i * ldd + j] = Cvt<TD>::from(src[i * lds + j]);
 }
 
 // dst = h + bf16(v - h), h = bf16(v): v rounded to the sum of its two BF16
@@ -327,9 +334,9 @@ cudaError_t round2_bf16_2d(Ty ts, const void* src, int64_t lds, float* dst, int6
 cudaError_t copy_cast_2d(Ty ts, const void* src, int64_t lds, Ty td, void* dst, int64_t ldd,
                          int64_t rows, int64_t cols, cudaStream_t st) {
   if (rows <= 0 || cols <= 0) return cudaSuccess;
-  const int grid = ceil_div(rows * ((cols + 3) / 4), 256);
   const size_t as = 4 * ty_size(ts), ad = 4 * ty_size(td);
-  const bool vec = lds % 4 == 0 && ldd % 4 == 0 && (uintptr_t)src % as == 0 && (uintptr_t)dst % ad == 0;
+  const bool vec = cols % 4 == 0 && lds % 4 == 0 && ldd % 4 == 0 && (uintptr_t)src % as == 0 && (uintptr_t)dst % ad == 0;
+  const int grid = ceil_div(rows * cols, vec ? 1024 : 256);
 #define RUQLP_CC(TS_, TD_, CS, CD)                                                           \
   if (ts == TS_ && td == TD_) {                                                              \
     k_copy_cast<CS, CD><<<grid, 256, 0, st>>>((const CS*)src, lds, (CD*)dst, ldd, rows, (int)cols, vec); \
