@@ -458,14 +458,13 @@ k_btc_gemm(const BTcTile* __restrict__ list, int n, const BMat* __restrict__ T,
 // One block per (tail tile, 4 rows), one thread per 4 columns (16-byte loads,
 // up to 16 contributors in flight), after the block lists the tile's
 // contributing CTAs and fragment slots.
-template <bool PAIR, bool WIDE>
 __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
   __shared__ int s_src[256];
   __shared__ int s_cnt[8];
   pdl_launch();
   pdl_wait();
   // tail tile index (with pairs: member `mem` of pair tile tt; P counts pairs)
-  const int tt = blockIdx.x >> (int)PAIR, mem = PAIR ? (int)(blockIdx.x & 1) : 0;
+  const int tt = blockIdx.x >> p.pair, mem = p.pair ? (int)(blockIdx.x & 1) : 0;
   const int64_t KB = p.KB;
   const int64_t lo = tt * KB, hi = lo + KB;
   // the contributors are consecutive CTAs starting near lo P / U (at most
@@ -490,36 +489,35 @@ __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
     if (k < w) pos += s_cnt[k];
     n += s_cnt[k];
   }
-  if (f) s_src[pos] = ((cc << (int)PAIR) + mem) * 2 + slot;
+  if (f) s_src[pos] = ((cc << p.pair) + mem) * 2 + slot;
   __syncthreads();
   // block (tt, y): rows 4 y .. 4 y + 3 of the tile, a thread per 4 columns
-  const int tile = ((p.full_waves * P + tt) << (int)PAIR) + mem;
+  const int tile = ((p.full_waves * P + tt) << p.pair) + mem;
   const int mt = tile / p.ns, col0 = (tile - mt * p.ns) * p.dpi;
   const int q4 = p.dpi / 4, qs = min(p.dpi, p.cols - col0) / 4;  // stored
   const int r = blockIdx.y * 4 + threadIdx.x / 64;
   const int64_t gr = (int64_t)mt * BM + r;
-  int c4 = threadIdx.x % 64;
-  if (gr >= p.Mout || c4 >= qs) return;
+  if (gr >= p.Mout) return;
   const float4* frag = reinterpret_cast<const float4*>(p.frag);
-  do {  // (one column group per thread, two when wide)
-    // sixteen 16-byte loads in flight, summed in contributor order
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int i = 0; i < n; i += 16) {
-      float4 v[16];
-  #pragma unroll
-      for (int u = 0; u < 16; ++u)
-        if (i + u < n) v[u] = frag[((int64_t)s_src[i + u] * BM + r) * q4 + c4];
-  #pragma unroll
-      for (int u = 0; u < 16; ++u)
-        if (i + u < n) {
-          s.x += v[u].x;
-          s.y += v[u].y;
-          s.z += v[u].z;
-          s.w += v[u].w;
-        }
-    }
-    *reinterpret_cast<float4*>(p.out + gr * p.ldo + col0 + 4 * c4) = s;
-  } while (WIDE && (c4 += 64) < qs);
+  for (int c4 = threadIdx.x % 64; c4 < qs; c4 += 64) {
+  // sixteen 16-byte loads in flight, summed in contributor order
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int i = 0; i < n; i += 16) {
+    float4 v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (i + u < n) v[u] = frag[((int64_t)s_src[i + u] * BM + r) * q4 + c4];
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (i + u < n) {
+        s.x += v[u].x;
+        s.y += v[u].y;
+        s.z += v[u].z;
+        s.w += v[u].w;
+      }
+  }
+  *reinterpret_cast<float4*>(p.out + gr * p.ldo + col0 + 4 * c4) = s;
+  }
 }
 
 // dst[c][r] = bf16(src[r][c]) for c < cols, 0 for cols <= c < dp (r < rows);
@@ -1096,7 +1094,7 @@ cudaError_t tc_launch(const TcOperands& o, const TcCfg& c, cudaStream_t st,
   count_launch();
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess || p.tail == 0) return e;
-  e = launch_pdl(dpi > 256 ? k_tc_fixup<false, true> : c.pair ? k_tc_fixup<true, false> : k_tc_fixup<false, false>, dim3(p.tail << c.pair, BM / 4), dim3(256), 0, st, p, P);
+  e = launch_pdl(k_tc_fixup, dim3(p.tail << c.pair, BM / 4), dim3(256), 0, st, p, P);
   count_launch();
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
