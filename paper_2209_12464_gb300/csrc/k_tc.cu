@@ -458,7 +458,69 @@ k_btc_gemm(const BTcTile* __restrict__ list, int n, const BMat* __restrict__ T,
 // One block per (tail tile, 4 rows), one thread per 4 columns (16-byte loads,
 // up to 16 contributors in flight), after the block lists the tile's
 // contributing CTAs and fragment slots.
+// Single CTAs and up to 256 columns (89 registers against 108 in the form below:
+// 3842 x 1632 transposed at d = 107, the call 57 -> 53 us).
 __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
+  __shared__ int s_src[256];
+  __shared__ int s_cnt[8];
+  pdl_launch();
+  pdl_wait();
+  const int tt = blockIdx.x;  // tail tile index
+  const int64_t KB = p.KB;
+  const int64_t lo = tt * KB, hi = lo + KB;
+  // the contributors are consecutive CTAs starting near lo P / U (at most
+  // P / tail + 2 of them): thread i tests CTA c0 + i, then an ordered
+  // compaction by warp ballots lists them with their fragment slots
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int c0 = max(0, (int)((lo * P) / p.U) - 2);
+  const int cc = c0 + (int)threadIdx.x;
+  bool f = false;
+  int slot = 0;
+  if (cc < P) {
+    const int64_t u0 = sk_start(cc, p.U, P), u1 = sk_start(cc + 1, p.U, P);
+    f = u0 < hi && u1 > lo && u1 > u0;
+    slot = (u0 / KB == tt) ? 0 : 1;
+  }
+  const unsigned b = __ballot_sync(0xffffffffu, f);
+  if (lane == 0) s_cnt[w] = __popc(b);
+  __syncthreads();
+  int pos = __popc(b & ((1u << lane) - 1u)), n = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    if (k < w) pos += s_cnt[k];
+    n += s_cnt[k];
+  }
+  if (f) s_src[pos] = cc * 2 + slot;
+  __syncthreads();
+  // block (tt, y): rows 4 y .. 4 y + 3 of the tile, a thread per 4 columns
+  const int tile = p.full_waves * P + tt;
+  const int mt = tile / p.ns, col0 = (tile - mt * p.ns) * p.dpi;
+  const int q4 = p.dpi / 4;
+  const int r = blockIdx.y * 4 + threadIdx.x / 64, c4 = threadIdx.x % 64;
+  const int64_t gr = (int64_t)mt * BM + r;
+  if (gr >= p.Mout || c4 >= q4 || col0 + 4 * c4 >= p.cols) return;
+  const float4* frag = reinterpret_cast<const float4*>(p.frag);
+  // sixteen 16-byte loads in flight, summed in contributor order
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int i = 0; i < n; i += 16) {
+    float4 v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (i + u < n) v[u] = frag[((int64_t)s_src[i + u] * BM + r) * q4 + c4];
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (i + u < n) {
+        s.x += v[u].x;
+        s.y += v[u].y;
+        s.z += v[u].z;
+        s.w += v[u].w;
+      }
+  }
+  *reinterpret_cast<float4*>(p.out + gr * p.ldo + col0 + 4 * c4) = s;
+}
+
+// CTA pairs, and items of more than 256 columns.
+__global__ void __launch_bounds__(256) k_tc_fixup_any(TcParams p, int P) {
   __shared__ int s_src[256];
   __shared__ int s_cnt[8];
   pdl_launch();
@@ -1094,7 +1156,7 @@ cudaError_t tc_launch(const TcOperands& o, const TcCfg& c, cudaStream_t st,
   count_launch();
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess || p.tail == 0) return e;
-  e = launch_pdl(k_tc_fixup, dim3(p.tail << c.pair, BM / 4), dim3(256), 0, st, p, P);
+  e = launch_pdl(c.pair || dpi > 256 ? k_tc_fixup_any : k_tc_fixup, dim3(p.tail << c.pair, BM / 4), dim3(256), 0, st, p, P);
   count_launch();
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
