@@ -386,14 +386,14 @@ int64_t ruqlp_launch_count(void);
  * of Section III-D, the bulk of the O(mnd) work): the first product of each
  * shape (orientation, two-part operand, output rows, K, dp) outside stream
  * capture times every valid column split (1, 2, 4; each with the deepest
- * shared-memory ring that fits) and, when A exceeds the L2, CTA pairs sharing
- * the skinny operand's loads, twice with CUDA events and keeps the fastest
+ * shared-memory ring that fits) twice with CUDA events and keeps the fastest
  * for the process; that configuration computes the result, so results are
  * deterministic from then on.  ruqlp_tune_file(path) loads earlier choices
  * from a text file (one "tc_gemm trans two_part rows K dp split stages us"
- * line each; pairs: split 1, 64 added to the stages) and appends every new
- * choice to it; NULL or "" stops the mirroring.  Returns the number of entries loaded.  Process-wide (all
- * handles); thread-safe. */
+ * line each) and appends every new choice to it; NULL or "" stops the
+ * mirroring.  Lines that name no configuration of this library are skipped.
+ * Returns the number of entries loaded.  Process-wide (all handles);
+ * thread-safe. */
 int ruqlp_tune_file(const char* path);
 
 /* With the "profile" option on: number of spans and their summed device time

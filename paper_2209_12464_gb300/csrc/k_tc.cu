@@ -54,8 +54,6 @@ struct TcParams {
   int dp;         // output columns (multiple of 16, <= 256; of 32, <= 384 when wide)
   int cols;       // columns stored (a multiple of 4)
   int ns, dpi;    // column split: items of dpi = dp / ns columns (MMA N)
-  int pair;       // 1: CTA pairs (clusters of two) take two tiles and share the
-                  // skinny operand's loads; T, tail and U then count pair tiles
   int stages;
   float* out;
   int64_t ldo;
@@ -75,7 +73,7 @@ struct Item {
 __device__ __forceinline__ int64_t sk_start(int64_t c, int64_t U, int P) { return c * U / P; }
 
 __device__ __forceinline__ int item_count(const TcParams& p) {
-  const int P = gridDim.x >> p.pair, c = blockIdx.x >> p.pair;
+  const int P = gridDim.x, c = blockIdx.x;
   int n = p.full_waves;
   if (p.tail > 0) {
     const int64_t u0 = sk_start(c, p.U, P), u1 = sk_start(c + 1, p.U, P);
@@ -85,7 +83,7 @@ __device__ __forceinline__ int item_count(const TcParams& p) {
 }
 
 __device__ __forceinline__ Item get_item(const TcParams& p, int i) {
-  const int P = gridDim.x >> p.pair, c = blockIdx.x >> p.pair;
+  const int P = gridDim.x, c = blockIdx.x;
   if (i < p.full_waves) return {c + i * P, 0, p.KB, -1};
   const int64_t u0 = sk_start(c, p.U, P), u1 = sk_start(c + 1, p.U, P);
   const int base = p.full_waves * P;
@@ -118,8 +116,7 @@ struct WorkSingle {
   static constexpr bool kGlobalMaps = false;
   __device__ int count() const { return item_count(*p); }
   __device__ TcItem get(int i) const {
-    Item it = get_item(*p, i);
-    if (p->pair) it.tile = 2 * it.tile + (blockIdx.x & 1);
+    const Item it = get_item(*p, i);
     const int mt = it.tile / p->ns, h = it.tile - mt * p->ns;
     TcItem r{mA, mB, mB2, mt, it.kb0, it.kb1, p->dpi, h * p->dpi, nullptr, p->dpi, 0, 0, false};
     if (it.slot < 0) {
@@ -185,17 +182,11 @@ __device__ __forceinline__ void tmap_acquire(const CUtensorMap* m) {
 // so h + l carries about 16 significant bits of the FP32 value); each stage
 // holds both parts' tiles and every A tile is multiplied by both into the same
 // accumulator, D += A h + A l.
-// PAIR: the CTAs of a cluster of two take two tiles with the same K blocks; each
-// loads its own A tiles and one half of the skinny operand's tile, multicast to
-// both, so that half crosses the L2 -> SM path once for two SMs.  A stage is
-// free when both CTAs' MMAs have read it (each commits to both empty barriers).
-// 20000 x 20000 at d = 220: 165 -> 158 us a launch (the skinny operand's traffic
-// is not what bounds it: 0.77 of measured HBM).
-template <bool TRANS, bool B2, bool PAIR, bool WIDE, class W>
+template <bool TRANS, bool B2, bool WIDE, class W>
 __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
                                         int withhold = 0) {
   // WIDE: items of more than 256 columns (one-part, not batched)
-  static_assert(!WIDE || (!B2 && !PAIR && !W::kGlobalMaps));
+  static_assert(!WIDE || (!B2 && !W::kGlobalMaps));
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -217,7 +208,7 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(full_bar(s), 1);
-      mbar_init(empty_bar(s), PAIR ? 2 : 1);
+      mbar_init(empty_bar(s), 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(tfull_bar(a), 1);
@@ -244,7 +235,6 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   volatile int* abort_flag = &s_abort;
-  if (PAIR) cluster_sync();  // the peer's barriers are initialised
   pdl_launch();
   pdl_wait();
 
@@ -290,13 +280,7 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
             tma_load_2d(sa + A_TILE_BYTES / 2, it.mA, full_bar(stage), it.tile * BM + 64,
                         kb * BK, pol_a);
           }
-          if constexpr (PAIR) {
-            const int half = it.dp / 2, r = (int)(blockIdx.x & 1) * half;
-            tma_load_2d_mc(sb + r * BK * 2, it.mB, full_bar(stage), kb * BK, r, 3, pol_b);
-            if (B2)
-              tma_load_2d_mc(sb + b_tile + r * BK * 2, it.mB2, full_bar(stage), kb * BK, r, 3,
-                             pol_b);
-          } else if constexpr (WIDE) {  // two boxes of half the columns
+          if constexpr (WIDE) {  // two boxes of half the columns
             const int half = it.dp / 2;
             tma_load_2d(sb, it.mB, full_bar(stage), kb * BK, 0, pol_b);
             tma_load_2d(sb + half * BK * 2, it.mB, full_bar(stage), kb * BK, half, pol_b);
@@ -304,14 +288,6 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
             tma_load_2d(sb, it.mB, full_bar(stage), kb * BK, it.bcol, pol_b);
             if (B2) tma_load_2d(sb + b_tile, it.mB2, full_bar(stage), kb * BK, it.bcol, pol_b);
           }
-          if (++stage == S) { stage = 0; phase ^= 1u; }
-        }
-      }
-      if (PAIR && ok) {
-        // every stage released by both CTAs: the peer's last commits have
-        // reached this CTA's barriers
-        for (int s = 0; s < S; ++s) {
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
       }
@@ -364,8 +340,7 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
               mma_bf16(tmem_d + 256, ad, sdesc(sb + it.dp / 2 * BK * 2 + kk * 32, 16, 1024), idesc,
                        (kb > it.kb0 || kk > 0) ? 1u : 0u);
           }
-          if (PAIR) mma_commit_mc(empty_bar(stage), 3);
-          else mma_commit(empty_bar(stage));
+          mma_commit(empty_bar(stage));
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
@@ -434,16 +409,14 @@ __device__ __forceinline__ void tc_body(const W& w, int* err, int S, int dpmax,
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base)
                  : "memory");
   }
-  // neither CTA leaves while the other's copies or commits may still reach it
-  if (PAIR) cluster_sync();
 }
 
-template <bool TRANS, bool B2, bool PAIR, bool WIDE>
+template <bool TRANS, bool B2, bool WIDE>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
           const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ TcParams p) {
   const WorkSingle w{&tmA, &tmB, &tmB2, &p};
-  tc_body<TRANS, B2, PAIR, WIDE>(w, p.err, p.stages, p.dpi, p.withhold);
+  tc_body<TRANS, B2, WIDE>(w, p.err, p.stages, p.dpi, p.withhold);
 }
 
 template <bool TRANS, bool B2>
@@ -451,15 +424,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 k_btc_gemm(const BTcTile* __restrict__ list, int n, const BMat* __restrict__ T,
            const CUtensorMap* __restrict__ maps, int dst, int stages, int dpmax, int* err) {
   const WorkBatch w{list, n, T, maps, dst, TRANS};
-  tc_body<TRANS, B2, false, false>(w, err, stages, dpmax);
+  tc_body<TRANS, B2, false>(w, err, stages, dpmax);
 }
 
 // Sum the stream-K fragments of each tail tile in CTA order into the output.
 // One block per (tail tile, 4 rows), one thread per 4 columns (16-byte loads,
 // up to 16 contributors in flight), after the block lists the tile's
-// contributing CTAs and fragment slots.
-// Single CTAs and up to 256 columns (89 registers against 108 in the form below:
-// 3842 x 1632 transposed at d = 107, the call 57 -> 53 us).
+// contributing CTAs and fragment slots.  WIDE (more than 256 columns): a thread
+// takes further columns too; without that loop the others need 90 registers
+// instead of 108 (3842 x 1632 transposed at d = 107, the call 57 -> 53 us).
+template <bool WIDE>
 __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
   __shared__ int s_src[256];
   __shared__ int s_cnt[8];
@@ -495,90 +469,30 @@ __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
   // block (tt, y): rows 4 y .. 4 y + 3 of the tile, a thread per 4 columns
   const int tile = p.full_waves * P + tt;
   const int mt = tile / p.ns, col0 = (tile - mt * p.ns) * p.dpi;
-  const int q4 = p.dpi / 4;
-  const int r = blockIdx.y * 4 + threadIdx.x / 64, c4 = threadIdx.x % 64;
-  const int64_t gr = (int64_t)mt * BM + r;
-  if (gr >= p.Mout || c4 >= q4 || col0 + 4 * c4 >= p.cols) return;
-  const float4* frag = reinterpret_cast<const float4*>(p.frag);
-  // sixteen 16-byte loads in flight, summed in contributor order
-  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int i = 0; i < n; i += 16) {
-    float4 v[16];
-#pragma unroll
-    for (int u = 0; u < 16; ++u)
-      if (i + u < n) v[u] = frag[((int64_t)s_src[i + u] * BM + r) * q4 + c4];
-#pragma unroll
-    for (int u = 0; u < 16; ++u)
-      if (i + u < n) {
-        s.x += v[u].x;
-        s.y += v[u].y;
-        s.z += v[u].z;
-        s.w += v[u].w;
-      }
-  }
-  *reinterpret_cast<float4*>(p.out + gr * p.ldo + col0 + 4 * c4) = s;
-}
-
-// CTA pairs, and items of more than 256 columns.
-__global__ void __launch_bounds__(256) k_tc_fixup_any(TcParams p, int P) {
-  __shared__ int s_src[256];
-  __shared__ int s_cnt[8];
-  pdl_launch();
-  pdl_wait();
-  // tail tile index (with pairs: member `mem` of pair tile tt; P counts pairs)
-  const int tt = blockIdx.x >> p.pair, mem = p.pair ? (int)(blockIdx.x & 1) : 0;
-  const int64_t KB = p.KB;
-  const int64_t lo = tt * KB, hi = lo + KB;
-  // the contributors are consecutive CTAs starting near lo P / U (at most
-  // P / tail + 2 of them): thread i tests CTA c0 + i, then an ordered
-  // compaction by warp ballots lists them with their fragment slots
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int c0 = max(0, (int)((lo * P) / p.U) - 2);
-  const int cc = c0 + (int)threadIdx.x;
-  bool f = false;
-  int slot = 0;
-  if (cc < P) {
-    const int64_t u0 = sk_start(cc, p.U, P), u1 = sk_start(cc + 1, p.U, P);
-    f = u0 < hi && u1 > lo && u1 > u0;
-    slot = (u0 / KB == tt) ? 0 : 1;
-  }
-  const unsigned b = __ballot_sync(0xffffffffu, f);
-  if (lane == 0) s_cnt[w] = __popc(b);
-  __syncthreads();
-  int pos = __popc(b & ((1u << lane) - 1u)), n = 0;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    if (k < w) pos += s_cnt[k];
-    n += s_cnt[k];
-  }
-  if (f) s_src[pos] = ((cc << p.pair) + mem) * 2 + slot;
-  __syncthreads();
-  // block (tt, y): rows 4 y .. 4 y + 3 of the tile, a thread per 4 columns
-  const int tile = ((p.full_waves * P + tt) << p.pair) + mem;
-  const int mt = tile / p.ns, col0 = (tile - mt * p.ns) * p.dpi;
   const int q4 = p.dpi / 4, qs = min(p.dpi, p.cols - col0) / 4;  // stored
   const int r = blockIdx.y * 4 + threadIdx.x / 64;
   const int64_t gr = (int64_t)mt * BM + r;
   if (gr >= p.Mout) return;
   const float4* frag = reinterpret_cast<const float4*>(p.frag);
   for (int c4 = threadIdx.x % 64; c4 < qs; c4 += 64) {
-  // sixteen 16-byte loads in flight, summed in contributor order
-  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int i = 0; i < n; i += 16) {
-    float4 v[16];
+    // sixteen 16-byte loads in flight, summed in contributor order
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < n; i += 16) {
+      float4 v[16];
 #pragma unroll
-    for (int u = 0; u < 16; ++u)
-      if (i + u < n) v[u] = frag[((int64_t)s_src[i + u] * BM + r) * q4 + c4];
+      for (int u = 0; u < 16; ++u)
+        if (i + u < n) v[u] = frag[((int64_t)s_src[i + u] * BM + r) * q4 + c4];
 #pragma unroll
-    for (int u = 0; u < 16; ++u)
-      if (i + u < n) {
-        s.x += v[u].x;
-        s.y += v[u].y;
-        s.z += v[u].z;
-        s.w += v[u].w;
-      }
-  }
-  *reinterpret_cast<float4*>(p.out + gr * p.ldo + col0 + 4 * c4) = s;
+      for (int u = 0; u < 16; ++u)
+        if (i + u < n) {
+          s.x += v[u].x;
+          s.y += v[u].y;
+          s.z += v[u].z;
+          s.w += v[u].w;
+        }
+    }
+    *reinterpret_cast<float4*>(p.out + gr * p.ldo + col0 + 4 * c4) = s;
+    if (!WIDE) break;
   }
 }
 
@@ -1065,7 +979,7 @@ namespace {
 
 // Launch configuration of one product: column split and ring depth.
 struct TcCfg {
-  int ns = 1, stages = 0, pair = 0;
+  int ns = 1, stages = 0;
 };
 
 size_t tc_stage_bytes(int dp, int ns, bool b2) {
@@ -1084,10 +998,8 @@ void tune_save_line(const std::array<int64_t, 5>& key, const TcCfg& c, double us
   if (g_tune_path.empty()) return;
   FILE* f = fopen(g_tune_path.c_str(), "a");
   if (!f) return;
-  // (pairs: split 1, 64 added to the stages)
   fprintf(f, "tc_gemm %lld %lld %lld %lld %lld %d %d %.3f\n", (long long)key[0], (long long)key[1],
-          (long long)key[2], (long long)key[3], (long long)key[4], c.ns,
-          c.pair ? c.stages + 64 : c.stages, us);
+          (long long)key[2], (long long)key[3], (long long)key[4], c.ns, c.stages, us);
   fclose(f);
 }
 
@@ -1108,7 +1020,7 @@ cudaError_t tc_launch(const TcOperands& o, const TcCfg& c, cudaStream_t st,
   CUtensorMap mA, mB, mB2;
   if (!make_map(&mA, o.A, (uint64_t)o.n, (uint64_t)o.m, (uint64_t)o.lda, 64, o.trans ? 64 : BM))
     return cudaErrorInvalidValue;
-  const uint32_t brows = (uint32_t)(dpi > 256 ? dpi / 2 : dpi >> c.pair);
+  const uint32_t brows = (uint32_t)(dpi > 256 ? dpi / 2 : dpi);  // of a box
   if (!make_map(&mB, o.Bt, (uint64_t)K, (uint64_t)o.dp, (uint64_t)o.ldb, 64, brows))
     return cudaErrorInvalidValue;
   if (o.b2) {
@@ -1128,11 +1040,9 @@ cudaError_t tc_launch(const TcOperands& o, const TcCfg& c, cudaStream_t st,
   p.ldo = o.ldo;
   p.frag = o.frag;
   p.err = o.err;
-  p.pair = c.pair;
-  p.T = c.pair ? ceil_div(Mout, 2 * BM) : ceil_div(Mout, BM) * c.ns;
+  p.T = ceil_div(Mout, BM) * c.ns;
   p.KB = ceil_div(K, BK);
-  // CTAs (or pairs): never more than the fragment buffer has slots for
-  int P = sm_count() >> c.pair;
+  int P = sm_count();  // never more CTAs than the fragment buffer has slots for
   if ((int64_t)p.T * p.KB < P) P = p.T * p.KB;
   p.full_waves = p.T / P;
   p.tail = p.T - p.full_waves * P;
@@ -1142,21 +1052,20 @@ cudaError_t tc_launch(const TcOperands& o, const TcCfg& c, cudaStream_t st,
   const size_t smem = tc_smem(c.stages, tc_stage_bytes(o.dp, c.ns, o.b2));
   auto pick = [&](auto tr) {
     constexpr bool TR = decltype(tr)::value;
-    if (dpi > 256) return k_tc_gemm<TR, false, false, true>;
-    if (c.pair) return o.b2 ? k_tc_gemm<TR, true, true, false> : k_tc_gemm<TR, false, true, false>;
-    return o.b2 ? k_tc_gemm<TR, true, false, false> : k_tc_gemm<TR, false, false, false>;
+    if (dpi > 256) return k_tc_gemm<TR, false, true>;
+    return o.b2 ? k_tc_gemm<TR, true, false> : k_tc_gemm<TR, false, false>;
   };
   auto kern = o.trans ? pick(std::true_type{}) : pick(std::false_type{});
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (mark) mark(true);
-  e = c.pair ? launch_pdl_cluster(kern, dim3(2 * P), dim3(NTHREADS), smem, 2, st, mA, mB, mB2, p)
-             : launch_pdl(kern, dim3(P), dim3(NTHREADS), smem, st, mA, mB, mB2, p);
+  e = launch_pdl(kern, dim3(P), dim3(NTHREADS), smem, st, mA, mB, mB2, p);
   if (mark) mark(false);
   count_launch();
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess || p.tail == 0) return e;
-  e = launch_pdl(c.pair || dpi > 256 ? k_tc_fixup_any : k_tc_fixup, dim3(p.tail << c.pair, BM / 4), dim3(256), 0, st, p, P);
+  e = launch_pdl(dpi > 256 ? k_tc_fixup<true> : k_tc_fixup<false>, dim3(p.tail, BM / 4),
+                 dim3(256), 0, st, p, P);
   count_launch();
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
@@ -1176,16 +1085,12 @@ int tune_file(const char* path) {
   double us;
   while (fscanf(f, "%31s %lld %lld %lld %lld %lld %d %d %lf", tag, &k0, &k1, &k2, &k3, &k4, &ns,
                 &stages, &us) == 9) {
-    const bool pair = stages > 64;
-    if (pair) stages -= 64;
-    if (strcmp(tag, "tc_gemm") != 0 || (pair && ns != 1) || !tc_ns_valid((int)k4, ns) ||
-        stages < 2 ||
+    if (strcmp(tag, "tc_gemm") != 0 || !tc_ns_valid((int)k4, ns) || stages < 2 ||
         tc_smem(stages, tc_stage_bytes((int)k4, ns, k1 != 0)) > 226 * 1024)
       continue;
     TcCfg c;
     c.ns = ns;
     c.stages = stages;
-    c.pair = pair;
     g_tune[{k0, k1, k2, k3, k4}] = c;
     ++n;
   }
@@ -1194,8 +1099,8 @@ int tune_file(const char* path) {
 }
 
 // Products of one shape run with the configuration measured fastest the
-// first time that shape is seen (outside stream capture): every valid column
-// split ns in {1, 2, 4} with the deepest ring that fits, and CTA pairs, each timed
+// first time that shape is seen (outside stream capture): every valid
+// column split ns in {1, 2, 4} with the deepest ring that fits, each timed
 // twice with CUDA events on the stream (the better time counts); the chosen
 // configuration then computes the result, so repeated calls are bitwise
 // equal.  force_ns > 0 skips the tuner.
@@ -1242,18 +1147,10 @@ cudaError_t tc_gemm(bool trans, const void* A, int64_t lda, int64_t m, int64_t n
   }
   TcCfg best = cfg_of(1);
   float best_ms = 1e30f;
-  for (int cand : {1, 2, 4, 0}) {  // 0: CTA pairs
-    const int ns = std::max(cand, 1);
+  for (int ns : {1, 2, 4}) {
     if (!tc_ns_valid(dp, ns)) continue;
-    TcCfg c = cfg_of(ns);
-    c.pair = cand == 0;
-    // (pairs from 16 tiles on: below, one tile more or less changes a CTA's K
-    // range, and with it the truncation of the tensor core's sums;
-    // and where A exceeds the 126 MB L2: 9668 x 4912 at d = 126, 95 MB, measured 81 us
-    // in pairs against 68 with ns = 2 once the operands alternate)
-    if (c.stages < 2 || (c.pair && (sm_count() < 2 || ceil_div(Mout, BM) < 16 ||
-                                    m * n * 2 <= (int64_t)1 << 27)))
-      continue;
+    const TcCfg c = cfg_of(ns);
+    if (c.stages < 2) continue;
     float t = 1e30f;
     for (int rep = 0; rep < 2; ++rep) {
       cudaEventRecord(e0, st);
