@@ -135,9 +135,9 @@ typedef struct {
  * the FP64 path and FP32 (shifted CholeskyQR3) on the FP32/BF16 paths unless
  * the "orth_fp64" option is set.  compute must equal A's dtype.
  * BF16 inputs use the tensor cores when A's leading dimension is a multiple
- * of 8 elements and A is 16-byte aligned (sketches wider than 384 columns, or
- * than 256 under a memory budget, run as column chunks, one pass over A each);
- * otherwise CUDA cores.  FP32 products over 128 rows or more take the tensor
+ * of 8 elements and A is 16-byte aligned (sketches wider than 256 columns
+ * run as column chunks, one pass over A each; up to 384 in one pass when A
+ * exceeds 128 MB); otherwise CUDA cores.  FP32 products over 128 rows or more take the tensor
  * cores too, each value split exactly into three BF16 parts (FP32 accuracy).
  * omega: n x d row-major FP64 Gaussian test matrix (device memory for
  * ruqlp_decompose / ruqlp_submit; host memory for ruqlp_decompose_host), or

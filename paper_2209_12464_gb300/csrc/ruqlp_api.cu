@@ -122,7 +122,7 @@ constexpr int kMaxSplits = 64;
 
 // Workspace layout for one problem.
 struct Layout {
-  size_t X, Y, Z, P, partial, G, Gf, R, Rw, St, Bt, Btl, frag, colptr, rowidx, cvals, cscratch, T, Om,
+  size_t X, Y, Z, P, partial, G, Gf, R, Rw, St, Bt, Btl, frag, frag_end, colptr, rowidx, cvals, cscratch, T, Om,
       lrT1, lrT2, lrTmp, lrPart, svdW, svdV, svdS, svdOrd, svdTmp, svdU, svdVs, Ts, total;
 };
 
@@ -130,8 +130,7 @@ inline int64_t round8(int64_t x) { return (x + 7) / 8 * 8; }
 
 // nnz >= 0: A is CSR with nnz nonzeros of val_bytes each (CSC copy kept too).
 // finish: room for Algorithm 1 step 5 (an m x dp buffer for Q P~).
-// img: room for the split skinny operand of an FP32 product (L.Bt) and for the
-// fragments of a one-pass BF16 product of 257 .. 384 columns.
+// img: room for the split skinny operand of an FP32 product (L.Bt).
 // tsqr: room for the Householder TSQR orth() (the rank-deficiency fallback).
 Layout layout_of(int64_t m, int64_t n, int d, Ty ct, int64_t nnz = -1, size_t val_bytes = 0,
                  int finish = 0, bool gen_omega = false, int64_t lr_r = 0, bool tsqr = false,
@@ -151,8 +150,11 @@ Layout layout_of(int64_t m, int64_t n, int d, Ty ct, int64_t nnz = -1, size_t va
   L.P = take((size_t)n * dp * wes);
   // Gram scratch: FP64 slab partials (SIMT Gram) or FP32 slab sums of the
   // tensor-core Gram (one per SM, at most 160)
-  L.partial = take(std::max((size_t)d * d * std::max<size_t>(kMaxSplits * sizeof(double), 160 * sizeof(float)),
-                             gram_tc_part_bytes(d)));
+  const size_t part = std::max(
+      (size_t)d * d * std::max<size_t>(kMaxSplits * sizeof(double), 160 * sizeof(float)),
+      gram_tc_part_bytes(d));
+  const bool bf16 = ct == Ty::BF16 && nnz < 0;
+  if (!bf16) L.partial = take(part);
   L.G = take((size_t)d * d * sizeof(double));
   L.Gf = take((size_t)d * d * sizeof(float));
   L.R = take((size_t)d * d * sizeof(double));
@@ -163,15 +165,19 @@ Layout layout_of(int64_t m, int64_t n, int d, Ty ct, int64_t nnz = -1, size_t va
   }
   // S = R^{-1} as three BF16 parts for the tensor-core Q = Y S
   if (work_ty(ct) == Ty::F32 && dp <= 256) L.St = take(qmul_st_bytes(d));
-  if (ct == Ty::BF16 && nnz < 0) {
+  if (bf16) {
     // the transposed BF16 skinny operand, then its low BF16 part (the
     // two-part B^T = A^T Q); the CUDA-core kernel's rounded FP32 operand
     // (K x d) fits the two together
     const size_t one = (size_t)dp * round8(m > n ? m : n) * 2;
     L.Bt = take(2 * one);
     L.Btl = L.Bt + one;
-    const int dpw = (dp + 31) / 32 * 32;
-    L.frag = take(tc_frag_bytes(dp <= 256 ? dp : img && tc_wide_fits(m, n, dpw) ? dpw : 256));  // per chunk
+    // the product's fragments (per column chunk) after the Gram scratch: no
+    // Gram runs during a product, so a one-pass product of 257 .. 384 columns
+    // has both for its fragments ([partial, frag_end))
+    L.partial = take(part);
+    L.frag = take(tc_frag_bytes(std::min(dp, 256)));
+    L.frag_end = off;
   }
   if (ct == Ty::F32 && nnz < 0 && img && f32_tc_supported(std::max(m, n)))
     L.Bt = take(f32_img_bytes(std::max(m, n), dp));
@@ -474,10 +480,11 @@ ruqlp_status product(ruqlp_ctx* h, const Layout& Lo, const Job& J, bool trans, T
     void* Bt = base + Lo.Bt;
     void* Btl = split2 ? base + Lo.Btl : nullptr;
     const int64_t ldb = round8(K);
-    // (up to 384 in one when a second pass would read A from HBM again and the
-    // workspace has room for the fragments)
+    // (up to 384 in one when a second pass would read A from HBM again: a rule
+    // on the shape alone, so that every handle has the same result)
     const int dpw = (J.dp + 31) / 32 * 32;
-    const bool wide = !split2 && h->f32_img && h->tc_nsplit <= 1 && tc_wide_fits(J.m, J.n, dpw);
+    const bool wide = !split2 && h->tc_nsplit <= 1 && tc_wide_fits(J.m, J.n, dpw) &&
+                      tc_frag_bytes(dpw) <= Lo.frag_end - Lo.partial;
     const int nch = wide ? 1 : (J.dp + 255) / 256;
     const int w = wide ? dpw : round16((J.dp + nch - 1) / nch);
     const size_t xes = ty_size(xt);
@@ -488,7 +495,7 @@ ruqlp_status product(ruqlp_ctx* h, const Layout& Lo, const Job& J, bool trans, T
         CK(transpose_to_bf16(xt, (const char*)Xin + (size_t)c0 * xes, ldx, K, cols, wc, Bt, ldb,
                              st, Btl));
       CK(tc_gemm(trans, J.A, J.lda, J.m, J.n, Bt, ldb, wc, (float*)out + c0, ldo,
-                 (float*)(base + Lo.frag), &h->status->timeout, st,
+                 (float*)(base + (wide ? Lo.partial : Lo.frag)), &h->status->timeout, st,
                  h->profile ? [&](bool begin) {
                    static thread_local cudaEvent_t a;
                    if (begin) { a = ev_get(h); cudaEventRecord(a, st); }
