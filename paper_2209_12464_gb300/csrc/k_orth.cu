@@ -88,8 +88,18 @@ k_chol(const double* __restrict__ G, int d, double shift_rel, int force_shift,
             }
           }
         }
-        const TF inv = TF(1) / piv;
-        for (int j = k + 1 + lane; j < d; j += 32) s_t[j] = W[uidx<PACKED>(k, j, d)] * inv;
+        // (a pivot whose reciprocal could overflow, from a sketch near the
+        // square root of the type's least number, is scaled by a power of two)
+        constexpr TF TINY = sizeof(TF) == 8 ? TF(0x1p-900) : TF(0x1p-100f);
+        constexpr TF UP = sizeof(TF) == 8 ? TF(0x1p600) : TF(0x1p60f);
+        if (piv < TINY) {
+          const TF inv = TF(1) / (piv * UP);
+          for (int j = k + 1 + lane; j < d; j += 32)
+            s_t[j] = (W[uidx<PACKED>(k, j, d)] * UP) * inv;
+        } else {
+          const TF inv = TF(1) / piv;
+          for (int j = k + 1 + lane; j < d; j += 32) s_t[j] = W[uidx<PACKED>(k, j, d)] * inv;
+        }
       }
       __syncthreads();
       if (s_bad) break;
