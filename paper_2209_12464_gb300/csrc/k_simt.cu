@@ -159,8 +159,12 @@ k_bgemm(const BMat* __restrict__ T, const int* __restrict__ prefix, int count, i
 }
 
 // FP64 products of one matrix with tiles fitted to the shape.  A CTA computes a
-// BM x BN tile (BN any multiple of NI), each thread MI x NI of it, an FMA chain
-// over K per entry.
+// BM x BN tile (BN any multiple of NI), each thread MI x NI of it: per entry FMA
+// chains of BL rows of K, whose sums are added in turn.  (Measured against chains of
+// 16, the 64 x 64 tiles' order: one chain over all of a slab has 1.2 to 1.6 times
+// the rounding error in products of K <= 300, 1.1 at 8192, 1.2 to 1.5 in Grams;
+// with these chains 1.00 at K <= 64, 0.7 at 544, 0.39 at 4096, 0.65 to 0.99 in
+// Grams.  Chains of 32 halve the additions, 3 instead of 6 % of the FP64 work.)
 // Products (PART = false): a cluster of S CTAs shares a tile; CTA s sums K slab
 // s, and the slab sums are added in slab order through distributed shared
 // memory.  Partial sums (PART = true, C = A^T B of a few columns): CTA (pair,
@@ -192,7 +196,7 @@ __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
-template <bool TRANS_A, typename T, int MI, int NI, bool PART>
+template <bool TRANS_A, typename T, int MI, int NI, bool PART, int BL>
 __global__ void __launch_bounds__(512)
 k_fit(const T* __restrict__ A, int64_t lda, const T* __restrict__ B, int64_t ldb,
       double* __restrict__ C, int64_t ldc, int64_t M, int64_t K, int64_t N, FitShape f,
@@ -255,15 +259,27 @@ k_fit(const T* __restrict__ A, int64_t lda, const T* __restrict__ B, int64_t ldb
                                                       : 0.0;
     __syncthreads();
     if (live) {
-#pragma unroll 16
-      for (int kk = 0; kk < BK; ++kk) {
-        double a[MI], b[NI];
-        fit_ld(As + kk * pa + ty * MI, a);
-        fit_ld(Bs + kk * pb + tx * NI, b);
+#pragma unroll 1
+      for (int kb = 0; kb < BK; kb += BL) {
+        double part[MI][NI];
 #pragma unroll
         for (int i = 0; i < MI; ++i)
 #pragma unroll
-          for (int j = 0; j < NI; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+          for (int j = 0; j < NI; ++j) part[i][j] = 0.0;
+#pragma unroll 16
+        for (int kk = kb; kk < kb + BL; ++kk) {
+          double a[MI], b[NI];
+          fit_ld(As + kk * pa + ty * MI, a);
+          fit_ld(Bs + kk * pb + tx * NI, b);
+#pragma unroll
+          for (int i = 0; i < MI; ++i)
+#pragma unroll
+            for (int j = 0; j < NI; ++j) part[i][j] = fma(a[i], b[j], part[i][j]);
+        }
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+          for (int j = 0; j < NI; ++j) acc[i][j] += part[i][j];
       }
     }
     __syncthreads();
@@ -327,6 +343,13 @@ void fit_columns(int64_t N, int ni, int widest, FitShape& f) {
   f.bn = ceil_div(ceil_div(N, f.nch), ni) * ni;
 }
 
+// Chain length over K rows.  In units of a product's rounding error squared, K
+// rows in chains of L and S slabs add K L / 2 + K^2 / (2 L S) + K S / 2 (the
+// chains, their sums, the slab sums; eight slabs at a time in a Gram: K S / 16):
+// 32 is no worse than the 64 x 64 tiles' 16 (with one slab, or a Gram's few)
+// from about 544 rows on in a product, 2048 in a Gram.
+int fit_chain(int64_t K, bool gram) { return K >= (gram ? 2048 : 544) ? 32 : 16; }
+
 int fit_threads(const FitShape& f, int mi, int ni) {
   return ceil_div((f.bm / mi) * (f.bn / ni), 32) * 32;
 }
@@ -334,8 +357,8 @@ int fit_threads(const FitShape& f, int mi, int ni) {
 // A product: the tile rows and the K split are taken that leave the fullest SM
 // the least work, the CTAs (ceil(M / bm) nch S of bm bn K / S multiply-adds)
 // being dealt evenly.  8192 x 4096 at d = 72: 9.49 ms in 64 x 64 tiles of all K
-// (128 padded columns), 4.26 ms in 64 x 36 tiles and 8 slabs (1.13 TFLOP/s of
-// the 1.19 the FP64 units do); 1000 x 800 at d = 30: 990 us (16 CTAs) to 76 us.
+// (128 padded columns), 4.41 ms in 64 x 36 tiles and 8 slabs (1.10 TFLOP/s of
+// the 1.19 the FP64 units do, and the additions of the chains); 1000 x 800 at d = 30: 990 us (16 CTAs) to 76 us.
 template <bool TRANS_A>
 cudaError_t fit_launch(const double* A, int64_t lda, const double* B, int64_t ldb, double* C,
                        int64_t ldc, int64_t M, int64_t K, int64_t N, const int32_t* gate,
@@ -366,7 +389,8 @@ cudaError_t fit_launch(const double* A, int64_t lda, const double* B, int64_t ld
   }
   f.kslab = ((K + f.S - 1) / f.S + FIT_BK - 1) / FIT_BK * FIT_BK;
   const size_t sm = fit_smem_bytes(f, f.S > 1);
-  auto kern = k_fit<TRANS_A, double, MI, NI, false>;
+  auto kern = fit_chain(K, false) == 32 ? k_fit<TRANS_A, double, MI, NI, false, 32>
+                                        : k_fit<TRANS_A, double, MI, NI, false, 16>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -385,8 +409,9 @@ cudaError_t fit_launch(const double* A, int64_t lda, const double* B, int64_t ld
 }
 
 // C[i][j] = sum_z P[z][i][j] in z order (deterministic), cast to TC.
-// sym: only the entries with j >= i were formed.
-template <typename TC>
+// sym: only the entries with j >= i were formed.  TREE: eight slabs are added in
+// pairs first (FP64 Grams, whose error many slabs added in turn would carry).
+template <typename TC, bool TREE = false>
 __global__ void k_reduce_partials(const double* __restrict__ P, int splits, int64_t M, int64_t N,
                                   TC* __restrict__ C, int64_t ldc,
                                   const int32_t* __restrict__ gate, bool sym = false) {
@@ -397,6 +422,14 @@ __global__ void k_reduce_partials(const double* __restrict__ P, int splits, int6
   if (sym && j < i) idx = j * N + i;
   double s = 0.0;  // split order, eight independent loads in flight
   int z = 0;
+  if constexpr (TREE) {
+    for (; z < splits; z += 8) {
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = z + u < splits ? P[(int64_t)(z + u) * M * N + idx] : 0.0;
+      s += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+    }
+  }
   for (; z + 8 <= splits; z += 8) {
     double v[8];
 #pragma unroll
@@ -425,14 +458,15 @@ cudaError_t fit_partial(const void* A, int64_t lda, const void* B, int64_t ldb, 
   f.S = (int)((K + f.kslab - 1) / f.kslab);
   const size_t sm = fit_smem_bytes(f, false);
   const int pairs = f.sym ? f.nch * (f.nch + 1) / 2 : f.nchm * f.nch;
-  k_fit<true, T, 2, 2, true>
-      <<<dim3(pairs, f.S), fit_threads(f, 2, 2), sm, st>>>((const T*)A, lda, (const T*)B, ldb,
+  auto kern = fit_chain(K, true) == 32 ? k_fit<true, T, 2, 2, true, 32>
+                                       : k_fit<true, T, 2, 2, true, 16>;
+  kern<<<dim3(pairs, f.S), fit_threads(f, 2, 2), sm, st>>>((const T*)A, lda, (const T*)B, ldb,
                                                            partial, N, M, K, N, f, gate);
   count_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_reduce_partials<TC><<<ceil_div(M * N, 256), 256, 0, st>>>(partial, f.S, M, N, (TC*)C, ldc, gate,
-                                                              f.sym);
+  k_reduce_partials<TC, true><<<ceil_div(M * N, 256), 256, 0, st>>>(partial, f.S, M, N, (TC*)C, ldc,
+                                                                    gate, f.sym);
   count_launch();
   return cudaGetLastError();
 }
