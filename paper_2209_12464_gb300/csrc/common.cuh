@@ -25,12 +25,16 @@ struct DevStatus {
 };
 
 // What the FP32 tensor-core products met (k_f32tc.cu): an operand outside the
-// range of their split; an operand below 2^-50; a result below 2^-70.  The
-// product is formed again on the CUDA cores for the first, and for the other
-// two together.
-constexpr int32_t RANGE_OFF = 1, RANGE_SMALL = 2, RANGE_TINY = 4;
+// range of their split; a nonzero operand below 2^-50; a nonzero result below
+// 2^-70; a result of exactly zero.  The product is formed again on the CUDA cores
+// for the first, and for the second and third together; for the second and fourth
+// together, those of its tiles whose zeros may be products that underflowed.
+constexpr int32_t RANGE_OFF = 1, RANGE_SMALL = 2, RANGE_TINY = 4, RANGE_ZERO = 8;
 __device__ __forceinline__ bool range_redo(int32_t r) {
   return (r & RANGE_OFF) || (r & (RANGE_SMALL | RANGE_TINY)) == (RANGE_SMALL | RANGE_TINY);
+}
+__device__ __forceinline__ bool range_zeros(int32_t r) {
+  return (r & (RANGE_SMALL | RANGE_ZERO)) == (RANGE_SMALL | RANGE_ZERO);
 }
 
 template <typename T> __device__ __forceinline__ float to_f32(T v);

@@ -18,7 +18,8 @@ enum class Mul : int {
 
 // C[M x N] = A[M x K] B[K x N]; all row-major with the given leading dims.
 // A non-null `redo` (DevStatus::range) makes the launch a no-op unless its
-// bits ask for the product to be formed again (range_redo).
+// bits ask for the product to be formed again (range_redo), or for a look at the
+// zeros among the results that C holds (range_zeros).
 cudaError_t simt_gemm_nn(Ty ta, Ty tb, Ty tc, Mul mul, const void* A, int64_t lda,
                          const void* B, int64_t ldb, void* C, int64_t ldc, int64_t M,
                          int64_t K, int64_t N, cudaStream_t st, const int32_t* redo = nullptr);

@@ -36,10 +36,15 @@
 // Range: the split is exact for 2^-110 <= |x| < 2^127, and FP32 products and
 // sums behave as on the CUDA cores while nothing comes near FP32's limits.
 // The converters note values that are not finite, at least 2^60 or (nonzero)
-// below 2^-100, and values below 2^-50; the epilogue notes results below
-// 2^-70.  The first, or both others together, make the CUDA-core kernel that
-// follows form the product again (DevStatus::range; set-only bits, read after
-// the launch, so the choice is deterministic).
+// below 2^-100, and nonzero values below 2^-50; the epilogue notes nonzero
+// results below 2^-70 and zeros.  The first, or the second and third together,
+// make the CUDA-core kernel that follows form the product again; the second and
+// the zeros together make it look at the zeros, whose row of A and column of X
+// say whether products may have underflowed there, and form the tiles again in
+// which they may (DevStatus::range; set-only bits, read after the launch, so the
+// choice is deterministic).  A zero row of A costs nothing that way: 8192 x 8192
+// with one and an element of 2^-60 elsewhere, d = 200: 4059 us for the call when
+// a zero counted as a tiny result, 470 now (295 without; the CUDA cores alone 3785).
 //
 // Bound: shared memory at wide sketches (the six products read 132 KB of
 // operands per 32-deep block at 224 columns, and the parts are written there
@@ -670,7 +675,8 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
       // whole 64-byte row segments (a lane storing its own row takes 32 of the
       // L1's cycles per instruction: 3600 clocks a tile at 112 columns)
       const int left = (int)min((int64_t)F32_BM, u.rows - (int64_t)u.tile * F32_BM) - g * 32;
-      float least = 1.f;
+      uint32_t lo = 0xFFFFFFFFu;  // (Range::key)
+      bool zero = false;
 #pragma unroll
       for (int c = 0; c < FT_NC; ++c) {
         if (c * 16 >= u.w) break;
@@ -689,9 +695,13 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < 16; ++j)
-          if (u.col0 + c * 16 + j < u.d) least = fminf(least, fabsf(acc[c][j]));
+          if (u.col0 + c * 16 + j < u.d) {
+            lo = min(lo, Range::key(acc[c][j]));
+            zero |= acc[c][j] == 0.f;
+          }
       }
-      if (lane < left && least < 8.470329e-22f) note(u.st, RANGE_TINY);  // 2^-70
+      if (lane < left && lo < 2u * 0x1C800000u - 1u) note(u.st, RANGE_TINY);  // 2^-70
+      if (lane < left && zero) note(u.st, RANGE_ZERO);
     }
     if (!ok) *abort_flag = 1;
   }

@@ -120,13 +120,85 @@ __device__ __forceinline__ void gemm_tile(const TA* __restrict__ A, int64_t lda,
   }
 }
 
+// Whether a zero of the tile (bx, by) of C = A B (A^T B), formed by the
+// tensor-core product, may stand for products that underflowed: both its row of A
+// and its column of B hold a nonzero value, and one of them one below 2^-50.
+// (Zero rows and columns, and sums that cancel among larger values, are exact.)
+template <bool TRANS_A>
+__device__ __forceinline__ bool zeros_suspect(const float* __restrict__ A, int64_t lda,
+                                           const float* __restrict__ B, int64_t ldb,
+                                           const float* __restrict__ C, int64_t ldc, int64_t M,
+                                           int64_t K, int64_t N, int bx, int by) {
+  constexpr int ZERO = 1, NONZERO = 2, SMALL = 4;
+  __shared__ int s_row[BM], s_col[BN];  // bits: a zero result; operands met
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int64_t m0 = (int64_t)bx * BM, n0 = (int64_t)by * BN;
+  auto kind = [](float x) {
+    const uint32_t u = __float_as_uint(x) << 1;
+    return u == 0u ? 0 : u < 2u * 0x26800000u ? NONZERO | SMALL : NONZERO;
+  };
+  auto is_zero = [&](int e) {
+    const int64_t i = m0 + e / BN, j = n0 + e % BN;
+    return i < M && j < N && C[i * ldc + j] == 0.f;
+  };
+  for (int e = t; e < BM + BN; e += NT) (e < BM ? s_row[e] : s_col[e - BM]) = 0;
+  __syncthreads();
+  bool any = false;
+  for (int e = t; e < BM * BN; e += NT)
+    if (is_zero(e)) {
+      any = true;
+      atomicOr(&s_row[e / BN], ZERO);
+      atomicOr(&s_col[e % BN], ZERO);
+    }
+  if (!__syncthreads_or(any)) return false;
+  // thread t: column t % 64 of a K x 64 panel, rows t / 64, + 4, ...
+  auto panel = [&](const float* P, int64_t ld, int64_t c0, int64_t width, int* s) {
+    const int c = t % 64;
+    if (c0 + c >= width || !(s[c] & ZERO)) return;
+    int f = 0;
+#pragma unroll 8
+    for (int64_t k = t / 64; k < K; k += NT / 64) f |= kind(P[k * ld + c0 + c]);
+    atomicOr(&s[c], f);
+  };
+  panel(B, ldb, n0, N, s_col);
+  if (TRANS_A) {
+    panel(A, lda, m0, M, s_row);
+  } else {
+    for (int r = warp; r < BM; r += NT / 32) {
+      if (!(s_row[r] & ZERO)) continue;
+      int f = 0;
+#pragma unroll 8
+      for (int64_t k = lane; k < K; k += 32) f |= kind(A[(m0 + r) * lda + k]);
+      atomicOr(&s_row[r], f);
+    }
+  }
+  __syncthreads();
+  any = false;
+  for (int e = t; e < BM * BN; e += NT) {
+    const int r = s_row[e / BN], c = s_col[e % BN];
+    any |= (r & c & NONZERO) && ((r | c) & SMALL) && is_zero(e);
+  }
+  return __syncthreads_or(any);
+}
+
+// (80 registers in FP32: left to itself the compiler takes 74 beside the zeros' check,
+// and the product 4 % longer)
 template <bool TRANS_A, typename TA, typename TB, typename TC, Mul MODE, bool PARTIAL>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, MODE == Mul::F32 ? 3 : 1)
 k_gemm(const TA* __restrict__ A, int64_t lda, const TB* __restrict__ B, int64_t ldb,
        TC* __restrict__ C, int64_t ldc, int64_t M, int64_t K, int64_t N, int64_t kslab,
        const int32_t* __restrict__ gate, const int32_t* __restrict__ redo) {
   if (gate != nullptr && *gate == 0) return;
-  if (redo != nullptr && !range_redo(*redo)) return;
+  if (redo != nullptr && !range_redo(*redo)) {
+    if constexpr (std::is_same_v<TA, float> && std::is_same_v<TB, float> &&
+                  std::is_same_v<TC, float> && !PARTIAL) {
+      if (!range_zeros(*redo) || !zeros_suspect<TRANS_A>(A, lda, B, ldb, C, ldc, M, K, N,
+                                                         blockIdx.x, blockIdx.y))
+        return;
+    } else {
+      return;
+    }
+  }
   gemm_tile<TRANS_A, TA, TB, TC, MODE, PARTIAL>(A, lda, B, ldb, C, ldc, M, K, N, kslab,
                                                 blockIdx.x, blockIdx.y, blockIdx.z);
 }
@@ -136,7 +208,7 @@ k_gemm(const TA* __restrict__ A, int64_t lda, const TB* __restrict__ B, int64_t 
 //   TRANS_A = false: buf[dst] (m x d) = A buf[src] (n x d)
 //   TRANS_A = true:  buf[dst] (n x d) = A^T buf[src] (m x d)
 template <bool TRANS_A, typename TA, typename TB, int SPLIT2 = 0>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, 3)
 k_bgemm(const BMat* __restrict__ T, const int* __restrict__ prefix, int count, int src, int dst) {
   // FP32 items on the tensor cores come here only to be formed again
   const int t = blockIdx.x;
@@ -146,10 +218,16 @@ k_bgemm(const BMat* __restrict__ T, const int* __restrict__ prefix, int count, i
     if (prefix[mid] <= t) lo = mid; else hi = mid;
   }
   const BMat& b = T[prefix[count + 1 + lo]];  // the launch order's item lo
-  if ((b.flags & (TRANS_A ? BM_F32_ATY : BM_F32_AX)) && !range_redo(b.status->range)) return;
   const int local = t - prefix[lo];
   const int ntn = (b.d + BN - 1) / BN;
   const int64_t Mout = TRANS_A ? b.n : b.m, K = TRANS_A ? b.m : b.n;
+  if constexpr (std::is_same_v<TA, float> && std::is_same_v<TB, float>) {
+    if ((b.flags & (TRANS_A ? BM_F32_ATY : BM_F32_AX)) && !range_redo(b.status->range) &&
+        (!range_zeros(b.status->range) ||
+         !zeros_suspect<TRANS_A>((const float*)b.A, b.lda, bbuf(b, src), b.dp, bbuf(b, dst), b.dp,
+                                 Mout, K, b.d, local / ntn, local % ntn)))
+      return;
+  }
   // with BF16 A the skinny operand is rounded to BF16 (or to its two-part
   // BF16 sum) as it is staged, the product the single-matrix BF16 path computes
   constexpr int RB = std::is_same<TA, __nv_bfloat16>::value ? (SPLIT2 ? 2 : 1) : 0;
