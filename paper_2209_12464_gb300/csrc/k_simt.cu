@@ -182,15 +182,15 @@ __device__ __forceinline__ bool zeros_suspect(const float* __restrict__ A, int64
 }
 
 // (80 registers in FP32: left to itself the compiler takes 74 beside the zeros' check,
-// and the product 4 % longer)
+// and the product 4 % longer; 0: the other types keep the compiler's choice)
 template <bool TRANS_A, typename TA, typename TB, typename TC, Mul MODE, bool PARTIAL>
-__global__ void __launch_bounds__(NT, MODE == Mul::F32 ? 3 : 1)
+__global__ void __launch_bounds__(NT, MODE == Mul::F32 ? 3 : 0)
 k_gemm(const TA* __restrict__ A, int64_t lda, const TB* __restrict__ B, int64_t ldb,
        TC* __restrict__ C, int64_t ldc, int64_t M, int64_t K, int64_t N, int64_t kslab,
        const int32_t* __restrict__ gate, const int32_t* __restrict__ redo) {
   if (gate != nullptr && *gate == 0) return;
   if (redo != nullptr && !range_redo(*redo)) {
-    if constexpr (std::is_same_v<TA, float> && std::is_same_v<TB, float> &&
+    if constexpr (MODE == Mul::F32 && std::is_same_v<TA, float> && std::is_same_v<TB, float> &&
                   std::is_same_v<TC, float> && !PARTIAL) {
       if (!range_zeros(*redo) || !zeros_suspect<TRANS_A>(A, lda, B, ldb, C, ldc, M, K, N,
                                                          blockIdx.x, blockIdx.y))
