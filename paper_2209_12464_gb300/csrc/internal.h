@@ -157,6 +157,8 @@ struct BMat {
   int64_t lda, m, n;
   int d, dp, ot;
   int flags;  // BM_* bits
+  int64_t f32_k[2];  // contraction lengths of A X, A^T Y on the tensor cores; 0 once a
+                     // product of the item has been left to the CUDA cores whole
   float* X;  // n x dp
   float* Y;  // m x dp
   float* Z;  // n x dp
@@ -202,7 +204,7 @@ __host__ __device__ inline int64_t gram_slabs(int64_t M, int max_slabs, int64_t*
 }
 int bgemm_tiles(int64_t rows, int d);
 // split2 (BF16 A): the skinny operand is rounded to the sum of its two BF16
-// parts (the two-part B^T = A^T Q), else to BF16.
+// parts (the two-part B^T = A^T Q), else to BF16. 
 cudaError_t bgemm(bool trans, Ty ta, Ty tb, const BMat* T, const int* prefix, int total, int count,
                   int src, int dst, cudaStream_t st, bool split2 = false);
 int bgram_tiles(int64_t M, int d, bool sym, int max_slabs);

@@ -1186,6 +1186,8 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
     b.lda = D.ld;
     b.m = D.m;
     b.n = D.n;
+    b.f32_k[0] = D.n;
+    b.f32_k[1] = D.m;
     b.d = dd[i];
     b.dp = round16(dd[i]);
     Ty ot;
