@@ -122,6 +122,9 @@ __device__ __forceinline__ void ft_columns(const F32Split& sp, int item, int dp,
 struct FtSingle {
   const FtParams* p;
   static constexpr bool kEmpty = false;  // units without K blocks
+  // A product that an operand outside the split's range sends to the CUDA cores is
+  // given up where one is met, and by the other CTAs when they see the note.
+  static constexpr bool kGiveUp = true;
   __device__ bool skip() const {
     return p->st != nullptr && range_redo(*(volatile int32_t*)&p->st->range);
   }
@@ -186,6 +189,7 @@ struct FtBatch {
   int src, dst, sms;
   bool trans;
   static constexpr bool kEmpty = true;
+  static constexpr bool kGiveUp = false;  // (the CTA's next item may be another matrix)
   __device__ bool skip() const { return false; }
   __device__ int tail_index(int64_t rows, int nch, int item) const {
     return tail_index_of(rows, nch, item, sms);
@@ -272,9 +276,12 @@ struct Range {
     lo = min(lo, min(key(v.x), key(v.y)));
     lo = min(lo, min(key(v.z), key(v.w)));
   }
-  __device__ __forceinline__ void tell(DevStatus* st) const {
-    if (!(hi < 1.152921504606846976e18f) || lo < 2u * 0x0D800000u - 1u) note(st, RANGE_OFF);
+  // (returns whether a value outside the split's range was noted)
+  __device__ __forceinline__ bool tell(DevStatus* st) const {
+    const bool off = !(hi < 1.152921504606846976e18f) || lo < 2u * 0x0D800000u - 1u;
+    if (off) note(st, RANGE_OFF);
     if (lo < 2u * 0x26800000u - 1u) note(st, RANGE_SMALL);
+    return off && st != nullptr;
   }
 };
 
@@ -417,6 +424,12 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   volatile int* abort_flag = &s_abort;
+  // why the CTA's roles stop early: a wait ran out (the error word is set), or the
+  // product is given up
+  constexpr int TIMED_OUT = 1, GIVE_UP = 2;
+  auto leave = [&]() {
+    if (*abort_flag == 0) *abort_flag = TIMED_OUT;
+  };
   pdl_launch();
   pdl_wait();
   // an earlier product of this run already asked for the CUDA cores (one thread
@@ -470,7 +483,7 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
           if (++sx == NX) { sx = 0; phx ^= 1u; }
         }
       }
-      if (!ok) { *abort_flag = 1; atomicExch(err, 1); }
+      if (!ok) leave();
       // every MMA has completed before TMEM is freed
       mma_commit(drain);
       volatile int never = 0;
@@ -480,12 +493,19 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
       bool ok = true;
       int sx = 0, issued = 0;
       uint32_t ph = 1;
+      int32_t seen = 0;  // the run's range word as of the block before (not waited for)
       for (int i = 0; i < nunits && ok; ++i) {
         const FtUnit u = w.get(i);
         const uint32_t bytes = f32_xstage(u.xw);
         const uint32_t part = bytes / 3;
         const uint8_t* src = u.img + (int64_t)u.kb0 * bytes;
         for (int kb = u.kb0; kb < u.kb1; ++kb) {
+          if (W::kGiveUp && (seen & RANGE_OFF)) {
+            *abort_flag = GIVE_UP;
+            ok = false;
+            break;
+          }
+          if (W::kGiveUp && u.st != nullptr) seen = *(volatile int32_t*)&u.st->range;
           if (!mbar_wait_inl(ex(sx), ph, abort_flag)) {
             ok = false;
             break;
@@ -504,7 +524,7 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
         }
       }
       if (!ok) {
-        *abort_flag = 1;
+        leave();
         // the copies already issued land before the CTA gives up its shared memory
         for (; issued > 0; --issued) {
           if (sx == 0) { sx = NX; ph ^= 1u; }
@@ -617,7 +637,12 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
         __syncwarp();
         if (lane == 0) mbar_arrive(fa(sa));
         fetch_a(slot);
-        rg.tell(u.st);
+        const bool off = rg.tell(u.st);
+        if (W::kGiveUp && __any_sync(0xffffffffu, off)) {
+          *abort_flag = GIVE_UP;
+          ok = false;
+          break;
+        }
         slot = (slot + 1) % FT_AHEAD;
         if (++sa == FT_NA) { sa = 0; pha ^= 1u; }
         if (!IMG) {
@@ -646,7 +671,7 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
       }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (!ok) *abort_flag = 1;
+    if (!ok) leave();
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(FT_REG_EPI));
     // ---------------- epilogue ----------------
@@ -715,10 +740,10 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
       if (lane < left && lo < 2u * 0x1C800000u - 1u) note(u.st, RANGE_TINY);  // 2^-70
       if (lane < left && zero) note(u.st, RANGE_ZERO);
     }
-    if (!ok) *abort_flag = 1;
+    if (!ok) leave();
   }
   __syncthreads();
-  if (t == 0 && *abort_flag) atomicExch(err, 1);
+  if (t == 0 && *abort_flag == TIMED_OUT) atomicExch(err, 1);
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base)

@@ -51,10 +51,8 @@ __device__ __forceinline__ bool mbar_wait_inl(uint32_t bar, uint32_t parity,
   const uint64_t t0 = gtimer();
   for (uint32_t it = 1;; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 63) == 0) {
-      if (*abort_flag) return false;
-      if (gtimer() - t0 > WAIT_NS) return false;
-    }
+    if (*abort_flag) return false;  // (64 tries last some 240 us)
+    if ((it & 63) == 0 && gtimer() - t0 > WAIT_NS) return false;
   }
 }
 __device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {

@@ -109,3 +109,23 @@ def test_batch_items_equal_the_single_matrices(h, q):
         for (Q, L, P), w in zip(b.outs, want):
             for x, y in zip((Q, L, P), w[:3]):
                 assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("m,n,d,i,j", [(20000, 1100, 96, 19999, 3), (20000, 1100, 96, 0, 1099),
+                                       (700, 9000, 224, 300, 4500)])
+@pytest.mark.parametrize("trans", [False, True])
+def test_one_element_outside_the_range(h, m, n, d, i, j, trans):
+    """The tensor-core product is given up in the middle: the whole result is the
+    CUDA cores', and the next product runs as ever."""
+    g = _gen(m + i)
+    A = torch.randn(m, n, generator=g, device="cuda")
+    X = torch.randn(m if trans else n, d, generator=g, device="cuda")
+    want = h.sketch(A, X, trans)
+    B = A.clone()
+    B[i, j] = 2.0 ** 61
+    Y = h.sketch(B, X, trans)
+    Bt = B.double().T if trans else B.double()
+    S = Bt.abs() @ X.double().abs()
+    assert bool(((Y.double() - Bt @ X.double()).abs() <= X.shape[0] * 2.0 ** -24 * S).all())
+    assert torch.equal(Y, h.sketch(B, X, trans))
+    assert torch.equal(want, h.sketch(A, X, trans))
