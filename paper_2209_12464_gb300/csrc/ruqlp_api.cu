@@ -1714,6 +1714,13 @@ ruqlp_status ruqlp_sketch(ruqlp_handle h, const ruqlp_matrix* A, int trans, cons
   void* stage = (char*)h->arena + (trans ? Lo.Z : Lo.Y);
   const void* Xuse = X;
   int64_t ldxu = ldx;
+  // an FP32 tensor-core product of rows that are not on 16 bytes copies them first
+  // (X in, Y out), the CUDA-core one does not: that one for a short contraction and
+  // few rows of result (20000 x 144, d = 1 .. 13: 53 to 57 us there, 58 to 60 on the
+  // tensor cores; K = 176 63 to 66 against 61; 100000 x 128 102 to 112 against 75)
+  if ((d % 4 || ldx % 4 || ldy % 4 || ((uintptr_t)X | (uintptr_t)Y) & 15) &&
+      (trans ? m : n) < 176 && Mout < 40000)
+    J.f32_tc[trans != 0] = false;
   // the SpMM's 128-bit gathers and the FP32 tensor-core product's 128-bit loads
   // need aligned rows
   const bool f32_tc = J.f32_tc[trans != 0];

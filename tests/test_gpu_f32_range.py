@@ -129,3 +129,19 @@ def test_one_element_outside_the_range(h, m, n, d, i, j, trans):
     assert bool(((Y.double() - Bt @ X.double()).abs() <= X.shape[0] * 2.0 ** -24 * S).all())
     assert torch.equal(Y, h.sketch(B, X, trans))
     assert torch.equal(want, h.sketch(A, X, trans))
+
+
+@pytest.mark.parametrize("m,K", [(300, 128), (300, 175), (300, 176), (39999, 175), (40000, 175)])
+@pytest.mark.parametrize("d", [1, 7, 40])
+@pytest.mark.parametrize("trans", [False, True])
+def test_short_contractions_of_unaligned_rows(h, m, K, d, trans):
+    """On both sides of the line between the CUDA cores and the tensor cores for
+    operands whose rows are not on 16 bytes, with X a slice of a wider matrix."""
+    g = _gen(m + K + d)
+    A = torch.randn(K, m, generator=g, device="cuda") if trans else torch.randn(m, K, generator=g,
+                                                                                device="cuda")
+    X = torch.randn(K, d + 1, generator=g, device="cuda")[:, 1:]
+    Y = h.sketch(A, X, trans)
+    Ad = (A.T if trans else A).double()
+    S = Ad.abs() @ X.double().abs()
+    assert bool(((Y.double() - Ad @ X.double()).abs() <= (58 + K) * 2.0 ** -24 * S).all())
