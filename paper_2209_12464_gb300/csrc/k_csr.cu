@@ -26,6 +26,9 @@ template <> __device__ __forceinline__ float val_f32<__nv_bfloat16>(__nv_bfloat1
   return __bfloat162float(v);
 }
 
+// (Up to 2^31 - 1 entries are accepted, and the last index plus a stride passes the
+// end of int32: loops over a row's entries are unsigned, or end at a multiple of the
+// stride.  64-bit indices take 5 to 10 % more on rows of a few entries.)
 // flag bit 1: rowptr not a valid prefix (rowptr[0] != 0, decreasing, or
 // rowptr[m] != nnz); bit 2: column index out of range or not strictly
 // increasing inside a row.  The valid columns are counted on the way (counts,
@@ -49,8 +52,8 @@ __global__ void k_csr_validate(const int32_t* __restrict__ rowptr, const int32_t
   }
   bool bad = false;
   int32_t before = -1;  // the last index of the chunk before
-  for (int32_t e0 = a; e0 < b; e0 += 32) {
-    const bool in = e0 + lane < b;
+  for (uint32_t e0 = a; e0 < (uint32_t)b; e0 += 32) {
+    const bool in = e0 + lane < (uint32_t)b;
     const int32_t c = in ? colidx[e0 + lane] : 0x7fffffff;
     int32_t prev = __shfl_up_sync(0xffffffffu, c, 1);
     if (lane == 0) prev = before;
@@ -129,7 +132,7 @@ __global__ void k_csc_scatter(const int32_t* __restrict__ rowptr, const int32_t*
   const int lane = threadIdx.x & 31;
   if (warp >= m) return;
   const int32_t a = rowptr[warp], b = rowptr[warp + 1];
-  for (int32_t e = a + lane; e < b; e += 32) {
+  for (uint32_t e = a + lane; e < (uint32_t)b; e += 32) {
     const int32_t pos = atomicAdd(&cursor[colidx[e]], 1);
     rowidx[pos] = (int32_t)warp;
     cvals[pos] = vals[e];
@@ -256,14 +259,14 @@ k_spmm(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx, const T
   const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (r >= rows) return;
-  const int32_t a = ptr[r], b = ptr[r + 1];
+  const int32_t a = ptr[r], b = ptr[r + 1], b4 = a + ((b - a) & ~3);
   const int nchunk = (d + 127) / 128;  // 128 columns per warp sweep (4 per lane)
   for (int ch = 0; ch < nchunk; ++ch) {
     const int c = ch * 128 + lane * 4;
     const bool on = c < d;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     int32_t e = a;
-    for (; e + 4 <= b; e += 4) {  // four independent gathers in flight
+    for (; e < b4; e += 4) {  // four independent gathers in flight
       int32_t col[4];
       float v[4];
 #pragma unroll
