@@ -67,7 +67,9 @@ __global__ void k_csr_validate(const int32_t* __restrict__ rowptr, const int32_t
 }
 
 // Exclusive scan of counts[0..n) into ptr[0..n]: block sums of 1024 counts,
-// then every block adds the sums before it and scans its own.
+// then every block adds the sums before it and scans its own.  A single block (n <=
+// 1024) needs no sums, and writes the scatter's cursors itself (300 x 200 with 6000
+// nonzeros: 76 to 79 us a call with the general form's three steps, 68 to 73 so).
 constexpr int SCAN_BLOCK = 1024;
 __device__ __forceinline__ int32_t block_sum(int32_t v, int32_t* red) {  // 256 threads
 #pragma unroll
@@ -92,8 +94,9 @@ __global__ void __launch_bounds__(256) k_scan_sums(const int32_t* __restrict__ c
   if (threadIdx.x == 0) sums[blockIdx.x] = v;
 }
 __global__ void __launch_bounds__(256) k_scan(const int32_t* __restrict__ counts,
-                                              const int32_t* __restrict__ sums, int64_t n,
-                                              int32_t* __restrict__ ptr) {
+                                              const int32_t* sums, int64_t n,
+                                              int32_t* __restrict__ ptr,
+                                              int32_t* cursor) {
   __shared__ int32_t red[8];
   int32_t v = 0;
   for (int i = threadIdx.x; i < (int)blockIdx.x; i += 256) v += sums[i];
@@ -118,7 +121,10 @@ __global__ void __launch_bounds__(256) k_scan(const int32_t* __restrict__ counts
   for (int k = 0; k < w; ++k) run += red[k];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    if (i0 + q < n) ptr[i0 + q] = run;
+    if (i0 + q < n) {
+      ptr[i0 + q] = run;
+      if (cursor != nullptr) cursor[i0 + q] = run;
+    }
     run += c[q];
     if (i0 + q + 1 == n) ptr[n] = run;
   }
@@ -335,12 +341,15 @@ cudaError_t csr_transpose(Ty tv, const int32_t* rowptr, const int32_t* colidx, c
   int32_t* counts = scratch;        // n, from csr_validate
   int32_t* cursor = scratch + n;    // n
   const int nblk = ceil_div(n, SCAN_BLOCK);
-  k_scan_sums<<<nblk, 256, 0, st>>>(counts, n, cursor);
-  count_launch();
-  k_scan<<<nblk, 256, 0, st>>>(counts, cursor, n, colptr);
+  const bool one = nblk == 1;
+  if (!one) {
+    k_scan_sums<<<nblk, 256, 0, st>>>(counts, n, cursor);
+    count_launch();
+  }
+  k_scan<<<nblk, 256, 0, st>>>(counts, cursor, n, colptr, one ? cursor : nullptr);
   count_launch();
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && !one)
     e = cudaMemcpyAsync(cursor, colptr, (size_t)n * sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
   if (e != cudaSuccess) return e;
   const int gw = ceil_div(m * 32, 256);
