@@ -122,15 +122,16 @@ k_chol(const double* __restrict__ G, int d, double shift_rel, int force_shift,
   // R (full FP64, zero lower part) and its working-type copy; in global mode
   // with TF = double the upper part of R already holds the factor
   if (!PACKED && sizeof(TF) != sizeof(double)) {
-    // float factor stored in R's memory: widen in place from the end
-    if (tid == 0) {
-      for (int64_t e = (int64_t)d * d - 1; e >= 0; --e) {
-        const int i = (int)(e / d), j = (int)(e % d);
-        const double v = (j >= i) ? (double)W[e] : 0.0;
-        R[e] = v;
-      }
+    // float factor stored in R's memory: widen in place, row by row from the end (d
+    // <= 512 threads read a row before any of them writes over it; the doubles of row
+    // i lie over floats of row i and later ones only).  d = 384: one thread going
+    // through all entries took most of the factorisation's 22 ms.
+    for (int i = d - 1; i >= 0; --i) {
+      const double v = tid < d && tid >= i ? (double)W[(int64_t)i * d + tid] : 0.0;
+      __syncthreads();
+      if (tid < d) R[(int64_t)i * d + tid] = v;
+      __syncthreads();
     }
-    __syncthreads();
     for (int i = warp; i < d; i += nwarps)
       for (int j = lane; j < d; j += 32) Rw[(int64_t)i * d + j] = (TW)R[(int64_t)i * d + j];
   } else {
@@ -160,7 +161,10 @@ k_trsm(const T* __restrict__ Y, int64_t ldy, const T* __restrict__ R, T* __restr
   if (gate != nullptr && *gate == 0) return;
   extern __shared__ unsigned char smem_raw[];
   T* S = reinterpret_cast<T*>(smem_raw);
-  __shared__ T s_inv[512];  // 1 / R_jj (d <= 512)
+  // 1 / R_jj (FP64: a division per column and thread would take longer; FP32 keeps the
+  // shared memory for a third CTA, 100000 x 300: 4.8 -> 6.3 ms a launch with two)
+  constexpr bool INV = sizeof(T) == 8;
+  __shared__ T s_inv[INV ? 512 : 1];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t r0 = (int64_t)blockIdx.x * rows;
   const int nr = (int)min((int64_t)rows, M - r0);
@@ -168,10 +172,11 @@ k_trsm(const T* __restrict__ Y, int64_t ldy, const T* __restrict__ R, T* __restr
     const int r = e / d, c = e % d;
     S[(int64_t)r * d + c] = Y[(r0 + r) * ldy + c];
   }
-  for (int j = tid; j < d; j += blockDim.x) s_inv[j] = T(1) / R[(int64_t)j * d + j];
+  if (INV)
+    for (int j = tid; j < d; j += blockDim.x) s_inv[j] = T(1) / R[(int64_t)j * d + j];
   __syncthreads();
   for (int j = 0; j < d; ++j) {
-    const T inv = s_inv[j];
+    const T inv = INV ? s_inv[j] : T(1) / R[(int64_t)j * d + j];
     for (int r = warp; r < nr; r += 8) {
       T* srow = S + (int64_t)r * d;
       const T xj = srow[j] * inv;
