@@ -213,6 +213,8 @@ ruqlp_status ruqlp_set_option(ruqlp_handle h, const char* name, int64_t value);
  *   call returns RUQLP_ERR_TIMEOUT after the CTA has drained its copies and
  *   freed its tensor memory; the handle stays usable.  Exercises the timeout
  *   path without faulting or hanging the GPU.
+ * (continued) "test_arena_limit": test hook, off (0) by default.  Workspaces of
+ *   more bytes fail as if the device had no room for them.
  * (continued) "tc_nsplit": column split of the tensor-core products: 0
  *   (default) = chosen per product shape by the library's tuner (below);
  *   1, 2, 4 = that split (each 128-row tile of the output taken as that many
@@ -234,8 +236,8 @@ ruqlp_status ruqlp_reserve(ruqlp_handle h, int64_t m, int64_t n, int d,
 
 /* Workspace bytes a problem needs (0 on invalid sizes); nnz as for
  * ruqlp_reserve.  (On a handle without a memory budget, dense FP32 problems
- * also keep the skinny operand of a product split for the tensor cores: about
- * 6 max(m, n) d bytes more.) */
+ * also keep the skinny operand of a product split for the tensor cores, about
+ * 6 max(m, n) d bytes more, where that can be had.) */
 size_t ruqlp_workspace_bytes(int64_t m, int64_t n, int d, ruqlp_dtype compute,
                              int64_t nnz);
 

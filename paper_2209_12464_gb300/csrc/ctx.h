@@ -33,8 +33,11 @@ struct ruqlp_ctx {
   int batch_orth_tc = 0;  // 1: batched BF16 items with dp <= 80 take the tensor-core passes
   int orth_tsqr = 0;    // 1: every orth() is a Householder TSQR
   // room for the split skinny operand of FP32 products (k_f32tc.cu): handles
-  // under a memory budget do without it (same results)
+  // under a memory budget do without it, and workspaces from img_limit on, which
+  // could not be had with it (same results)
   bool f32_img = true;
+  size_t img_limit = ~(size_t)0;
+  size_t test_arena_limit = 0;  // test hook: workspaces above it cannot be had
   int tc_nsplit = 0;    // tensor-core products: column split (0 = tuned per shape)
   int test_withhold = 0;  // test hook: the next tensor-core products run out a wait
   bool tsqr_now = false;  // this run takes the TSQR orth() (fallback rerun)

@@ -221,12 +221,32 @@ ruqlp_status ensure_arena(ruqlp_ctx* h, size_t bytes) {
     h->arena = nullptr;
     h->arena_bytes = 0;
   }
+  if (h->test_arena_limit && bytes > h->test_arena_limit)
+    return fail(h, RUQLP_ERR_CUDA, "test hook: no workspace of %zu bytes", bytes);
   CK(cudaMalloc(&h->arena, bytes));
   h->arena_bytes = bytes;
   for (auto& g : h->batches)
     if (g.exec) cudaGraphExecDestroy(g.exec);
   h->batches.clear();
   return RUQLP_OK;
+}
+
+// A workspace of bytes(true) with the split skinny operand of FP32 products, or else of
+// bytes(false): a problem that fits without that operand still runs.
+template <class F>
+ruqlp_status ensure_arena_img(ruqlp_ctx* h, F bytes, bool* img) {
+  const size_t with = h->f32_img ? bytes(true) : 0, without = bytes(false);
+  *img = with > without;
+  if (*img) {
+    if (with < h->img_limit) {
+      if (ensure_arena(h, with) == RUQLP_OK) return RUQLP_OK;
+      cudaGetLastError();  // not the next launch's error
+      h->err.clear();
+      h->img_limit = with;
+    }
+    *img = false;
+  }
+  return ensure_arena(h, without);
 }
 
 ruqlp_status validate_params(ruqlp_ctx* h, int64_t m, int64_t n, Ty at, const ruqlp_params* prm,
@@ -304,6 +324,7 @@ struct Job {
   int finish_paper;  // 0 none, 1 qr(L) (Algorithm 1 step 5), 2 SVD of L (Remark 1)
   bool use_tc;  // BF16 products on the tensor cores (k_tc.cu)
   bool f32_tc[2] = {false, false};  // FP32 A X, A^T Y on the tensor cores (k_f32tc.cu)
+  int img = -1;         // the workspace holds the split skinny operand (-1: not decided)
   int x_cols = 0;       // readable columns of a caller's skinny operand (0: an arena buffer)
   int64_t out_ld = 0;   // a product straight into a caller's buffer: its leading
                         // dimension, d columns stored (0: an arena buffer, ld dp)
@@ -612,12 +633,17 @@ ruqlp_status run_dense(ruqlp_ctx* h, const Job& J0) {
   Job J = J0;
   const bool gen = J.omega == nullptr;
   const bool ts = h->tsqr_now || h->orth_tsqr;
-  const Layout Lo = J.csr ? layout_of(J.m, J.n, J.d, J.ct, J.nnz, ty_size(J.tv), J.finish_paper,
-                                      gen, J.lr_r, ts)
-                          : layout_of(J.m, J.n, J.d, J.ct, -1, 0, J.finish_paper, gen, 0, ts,
-                                      h->f32_img);
-  ruqlp_status s = ensure_arena(h, Lo.total);
+  auto layout = [&](bool img) {
+    return J.csr ? layout_of(J.m, J.n, J.d, J.ct, J.nnz, ty_size(J.tv), J.finish_paper, gen,
+                             J.lr_r, ts)
+                 : layout_of(J.m, J.n, J.d, J.ct, -1, 0, J.finish_paper, gen, 0, ts, img);
+  };
+  bool img = J.img == 1;
+  ruqlp_status s = J.img >= 0
+                       ? ensure_arena(h, layout(img).total)
+                       : ensure_arena_img(h, [&](bool i) { return layout(i).total; }, &img);
   if (s != RUQLP_OK) return s;
+  const Layout Lo = layout(img);
   CK(status_reset(h->status, h->stream));
   if (gen) {  // a1: Omega from the counter-based generator, on the device
     double* Om = (double*)((char*)h->arena + Lo.Om);
@@ -887,6 +913,7 @@ struct BatchPlan {
   size_t off_ft[2], off_ftfix[2];
   int wmax_ft = 16;
   bool any_tc = false;  // any BF16 tensor-core item
+  bool img = false;     // FP32 items have their split skinny operands in Bt
   // tensor-core CholeskyQR items (orth_tc): their list (for k_btrinv) and,
   // over Y (m rows) and over Z (n rows), the Gram units (one row slab each)
   // and the Q = Y R^{-1} units with their per-CTA ranges
@@ -950,7 +977,7 @@ ruqlp_status batch_launches(ruqlp_ctx* h, const BatchPlan& bp, int count, int q,
     const int pf = trans ? PF_TN : PF_NN;
     CK(bf32_gemm_tc(trans, T, (const F32Tile*)(base + bp.off_ft[trans]), (int)bp.ft[trans].size(),
                     (const F32Tile*)(base + bp.off_ftfix[trans]), (int)bp.ftfix[trans].size(),
-                    src, dst, bp.wmax_ft, count, h->f32_img, err, st));
+                    src, dst, bp.wmax_ft, count, bp.img, err, st));
     CK(bgemm(trans, ct, Ty::F32, T, pre(pf), tot(pf), count, src, dst, st, split2));
     const auto& list = trans ? bp.tc_tn : bp.tc_nn;
     if (!list.empty()) {  // Bt (and Btl) were written by the step that produced buf[src]
@@ -1002,8 +1029,12 @@ void tc_list(const std::vector<BMat>& table, bool trans, std::vector<BTcTile>& o
 
 namespace ruqlp {
 
-ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const ruqlp_params* prm,
-                         const ruqlp_outputs* out, bool graphs_ok, BatchRun* run) {
+// want_img: room for the items' split skinny operands; no_room is set (and nothing
+// launched) when the workspace could not be had with it.
+static ruqlp_status batch_begin_img(ruqlp_ctx* h, int count, const ruqlp_matrix* A,
+                                    const ruqlp_params* prm, const ruqlp_outputs* out,
+                                    bool graphs_ok, BatchRun* run, bool want_img,
+                                    bool* no_room) {
   if (count < 1 || !A || !prm || !out) return fail(h, RUQLP_ERR_INVALID, "empty or NULL batch");
   Ty ct0 = Ty::F32;
   int q0 = 0;
@@ -1056,7 +1087,8 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
       bp.wmax_ft = std::max(bp.wmax_ft, f32_columns(dp).w);
       f32_tiles(i, f32_split(rows, K, m, n, d, dp), bp.ft[x], bp.ftfix[x]);
     }
-    const bool img = h->f32_img && (b.flags & (BM_F32_AX | BM_F32_ATY));
+    const bool img = want_img && (b.flags & (BM_F32_AX | BM_F32_ATY));
+    bp.img = bp.img || img;
     bp.any_tc = bp.any_tc || b.use_tc;
     // option batch_orth_tc: BF16 items of width dp <= 80 run their
     // CholeskyQR passes on the tensor cores (a rule on the dtype, the
@@ -1174,8 +1206,19 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
   bp.off_status = take(sizeof(DevStatus) * count);
   bp.off_err = take(sizeof(int));
   bp.total = off;
-  ruqlp_status s = ensure_arena(h, bp.total);
-  if (s != RUQLP_OK) return s;
+  ruqlp_status s = RUQLP_OK;
+  if (bp.img) {
+    if (bp.total >= h->img_limit || ensure_arena(h, bp.total) != RUQLP_OK) {
+      cudaGetLastError();  // not the next launch's error
+      h->err.clear();
+      h->img_limit = std::min(h->img_limit, bp.total);
+      *no_room = true;
+      return RUQLP_OK;
+    }
+  } else {
+    s = ensure_arena(h, bp.total);
+    if (s != RUQLP_OK) return s;
+  }
   char* base = (char*)h->arena;
   std::vector<int> cnts[NPF];
   for (int k = 0; k < NPF; ++k) cnts[k].assign(count, 0);
@@ -1201,7 +1244,7 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
     b.G = (double*)(base + oG[i]);
     b.Gf = (float*)(base + oGf[i]);
     b.tiles = (float*)(base + oT[i]);
-    b.Bt = b.use_tc || (h->f32_img && (b.flags & (BM_F32_AX | BM_F32_ATY)))
+    b.Bt = b.use_tc || (want_img && (b.flags & (BM_F32_AX | BM_F32_ATY)))
                ? (void*)(base + oB[i])
                : nullptr;
     b.Btl = b.use_tc ? (void*)(base + oB[i] + (size_t)b.dp * b.ldbt * 2) : nullptr;
@@ -1250,7 +1293,7 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
   tc_list(bp.table, true, bp.tc_tn);
   // signature: the launch sequence depends on shapes, q, dtype, product
   // kernels and the arena
-  std::vector<int64_t> key = {count, q0, (int64_t)ct0, (int64_t)(uintptr_t)h->arena};
+  std::vector<int64_t> key = {count, q0, (int64_t)ct0, (int64_t)(uintptr_t)h->arena, bp.img};
   for (int i = 0; i < count; ++i) {
     key.push_back(bp.table[i].m);
     key.push_back(bp.table[i].n);
@@ -1351,6 +1394,14 @@ ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const r
   run->A.assign(A, A + count);
   run->prm.assign(prm, prm + count);
   return RUQLP_OK;
+}
+
+ruqlp_status batch_begin(ruqlp_ctx* h, int count, const ruqlp_matrix* A, const ruqlp_params* prm,
+                         const ruqlp_outputs* out, bool graphs_ok, BatchRun* run) {
+  bool no_room = false;
+  ruqlp_status s =
+      batch_begin_img(h, count, A, prm, out, graphs_ok, run, h->f32_img, &no_room);
+  return no_room ? batch_begin_img(h, count, A, prm, out, graphs_ok, run, false, &no_room) : s;
 }
 
 ruqlp_status batch_end(ruqlp_ctx* h, const BatchRun& run, ruqlp_outputs* out) {
@@ -1474,6 +1525,10 @@ ruqlp_status ruqlp_set_option(ruqlp_handle h, const char* name, int64_t value) {
     h->orth_tsqr = value ? 1 : 0;
     return RUQLP_OK;
   }
+  if (strcmp(name, "test_arena_limit") == 0) {
+    h->test_arena_limit = value > 0 ? (size_t)value : 0;
+    return RUQLP_OK;
+  }
   if (strcmp(name, "test_withhold_stage") == 0) {
     h->test_withhold = value ? 1 : 0;
     return RUQLP_OK;
@@ -1512,8 +1567,10 @@ ruqlp_status ruqlp_reserve(ruqlp_handle h, int64_t m, int64_t n, int d, ruqlp_dt
   if (b == 0) return fail(h, RUQLP_ERR_INVALID, "invalid sizes for ruqlp_reserve");
   Ty ct = Ty::F32;
   ty_of(compute, &ct);
-  return ensure_arena(h, nnz < 0 ? layout_of(m, n, d, ct, -1, 0, 0, false, 0, false, h->f32_img).total
-                                 : b);
+  if (nnz >= 0) return ensure_arena(h, b);
+  bool img;
+  return ensure_arena_img(
+      h, [&](bool i) { return layout_of(m, n, d, ct, -1, 0, 0, false, 0, false, i).total; }, &img);
 }
 
 ruqlp_status ruqlp_decompose(ruqlp_handle h, const ruqlp_matrix* A, const ruqlp_params* prm,
@@ -1587,32 +1644,38 @@ static ruqlp_status decompose_host_once(ruqlp_handle h, const ruqlp_matrix* A,
   // the workspace first, then staging for A, Omega and the outputs
   const bool gen = prm->omega == nullptr;  // run_dense's layout, which comes first
   const bool ts = h->tsqr_now || h->orth_tsqr;
-  const Layout Lo = J.csr ? layout_of(m, n, d, J.ct, J.nnz, ty_size(J.tv), J.finish_paper, gen,
-                                      0, ts)
-                          : layout_of(m, n, d, J.ct, -1, 0, J.finish_paper, gen, 0, ts,
-                                      h->f32_img);
-  size_t off = align_up(Lo.total, 256);
-  auto take = [&](size_t bytes) {
-    const size_t o = off;
-    off = align_up(off + bytes, 256);
-    return o;
+  size_t oA, oRp, oCi, oV, oOm, oQ, oL, oP;
+  // TMA needs a 16-byte row pitch
+  const int64_t lds = !J.csr && J.ct == Ty::BF16 ? round8(n) : n;
+  auto place = [&](bool img) {  // after the decomposition's own workspace
+    const Layout Lo = J.csr ? layout_of(m, n, d, J.ct, J.nnz, ty_size(J.tv), J.finish_paper, gen,
+                                        0, ts)
+                            : layout_of(m, n, d, J.ct, -1, 0, J.finish_paper, gen, 0, ts, img);
+    size_t off = align_up(Lo.total, 256);
+    auto take = [&](size_t bytes) {
+      const size_t o = off;
+      off = align_up(off + bytes, 256);
+      return o;
+    };
+    oA = oRp = oCi = oV = 0;
+    if (J.csr) {
+      oRp = take((size_t)(m + 1) * sizeof(int32_t));
+      oCi = take((size_t)(J.nnz > 0 ? J.nnz : 1) * sizeof(int32_t));
+      oV = take((size_t)(J.nnz > 0 ? J.nnz : 1) * ty_size(J.tv));
+    } else {
+      oA = take((size_t)m * lds * ty_size(J.ct));
+    }
+    oOm = prm->omega ? take((size_t)n * d * sizeof(double)) : 0;
+    oQ = take((size_t)m * d * oes);
+    oL = take((size_t)d * d * oes);
+    oP = take((size_t)n * d * oes);
+    return off;
   };
-  size_t oA = 0, oRp = 0, oCi = 0, oV = 0;
-  int64_t lds = n;
-  if (J.csr) {
-    oRp = take((size_t)(m + 1) * sizeof(int32_t));
-    oCi = take((size_t)(J.nnz > 0 ? J.nnz : 1) * sizeof(int32_t));
-    oV = take((size_t)(J.nnz > 0 ? J.nnz : 1) * ty_size(J.tv));
-  } else {
-    lds = (J.ct == Ty::BF16) ? round8(n) : n;  // TMA needs a 16-byte row pitch
-    oA = take((size_t)m * lds * ty_size(J.ct));
-  }
-  const size_t oOm = prm->omega ? take((size_t)n * d * sizeof(double)) : 0;
-  const size_t oQ = take((size_t)m * d * oes);
-  const size_t oL = take((size_t)d * d * oes);
-  const size_t oP = take((size_t)n * d * oes);
-  s = ensure_arena(h, off);
+  bool img;
+  s = ensure_arena_img(h, place, &img);
   if (s != RUQLP_OK) return s;
+  place(img);
+  J.img = img;
   char* base = (char*)h->arena;
   cudaStream_t st = h->stream;
   if (J.csr) {
@@ -1702,10 +1765,14 @@ ruqlp_status ruqlp_sketch(ruqlp_handle h, const ruqlp_matrix* A, int trans, cons
   J.use_tc = !J.csr && J.ct == Ty::BF16 && !h->bf16_simt &&
              tc_supported(J.A, J.lda, std::min(J.dp, 256));
   const int64_t Mout = trans ? n : m;
-  const Layout Lo = J.csr ? layout_of(m, n, d, J.ct, J.nnz, ty_size(J.tv), false, false, J.lr_r)
-                          : layout_of(m, n, d, J.ct, -1, 0, 0, false, 0, false, h->f32_img);
-  s = ensure_arena(h, Lo.total);
+  auto layout = [&](bool img) {
+    return J.csr ? layout_of(m, n, d, J.ct, J.nnz, ty_size(J.tv), false, false, J.lr_r)
+                 : layout_of(m, n, d, J.ct, -1, 0, 0, false, 0, false, img);
+  };
+  bool img;
+  s = ensure_arena_img(h, [&](bool i) { return layout(i).total; }, &img);
   if (s != RUQLP_OK) return s;
+  const Layout Lo = layout(img);
   CK(status_reset(h->status, h->stream));
   if (J.csr) {
     s = prepare_csr(h, Lo, J);
