@@ -431,8 +431,8 @@ k_btc_gemm(const BTcTile* __restrict__ list, int n, const BMat* __restrict__ T,
 // One block per (tail tile, 4 rows), one thread per 4 columns (16-byte loads,
 // up to 16 contributors in flight), after the block lists the tile's
 // contributing CTAs and fragment slots.  WIDE (more than 256 columns): a thread
-// takes further columns too; without that loop the others need 90 registers
-// instead of 108 (3842 x 1632 transposed at d = 107, the call 57 -> 53 us).
+// takes further columns too; without that loop the others need 89 registers
+// instead of 110 (3842 x 1632 transposed at d = 107, the call 57 -> 53 us).
 template <bool WIDE>
 __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
   __shared__ int s_src[256];
@@ -469,13 +469,14 @@ __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
   // block (tt, y): rows 4 y .. 4 y + 3 of the tile, a thread per 4 columns
   const int tile = p.full_waves * P + tt;
   const int mt = tile / p.ns, col0 = (tile - mt * p.ns) * p.dpi;
-  const int q4 = p.dpi / 4, qs = min(p.dpi, p.cols - col0) / 4;  // stored
+  const int q4 = p.dpi / 4;
   const int r = blockIdx.y * 4 + threadIdx.x / 64;
+  int c4 = threadIdx.x % 64;
   const int64_t gr = (int64_t)mt * BM + r;
-  if (gr >= p.Mout) return;
+  if (gr >= p.Mout || c4 >= q4 || col0 + 4 * c4 >= p.cols) return;
   const float4* frag = reinterpret_cast<const float4*>(p.frag);
-  for (int c4 = threadIdx.x % 64; c4 < qs; c4 += 64) {
-    // sixteen 16-byte loads in flight, summed in contributor order
+  // sixteen 16-byte loads in flight, summed in contributor order
+  auto sum = [&]() {
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int i = 0; i < n; i += 16) {
       float4 v[16];
@@ -492,8 +493,10 @@ __global__ void __launch_bounds__(256) k_tc_fixup(TcParams p, int P) {
         }
     }
     *reinterpret_cast<float4*>(p.out + gr * p.ldo + col0 + 4 * c4) = s;
-    if (!WIDE) break;
-  }
+  };
+  sum();
+  if constexpr (WIDE)
+    while ((c4 += 64) < q4 && col0 + 4 * c4 < p.cols) sum();
 }
 
 // dst[c][r] = bf16(src[r][c]) for c < cols, 0 for cols <= c < dp (r < rows);
