@@ -44,19 +44,21 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // Bounded wait on an mbarrier phase; false on timeout or when another role
 // of the CTA has already given up.
 // (mbar_wait_inl: the same inlined, for kernels whose warpgroups hold different
-// register counts, where a call has no one register budget.)
+// register counts, where a call has no one register budget; it looks at the stop
+// word at every try, since 64 tries last some 240 us.)
+template <int POLL = 1>
 __device__ __forceinline__ bool mbar_wait_inl(uint32_t bar, uint32_t parity,
                                               volatile int* abort_flag) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = gtimer();
   for (uint32_t it = 1;; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;  // (64 tries last some 240 us)
+    if (it % POLL == 0 && *abort_flag) return false;
     if ((it & 63) == 0 && gtimer() - t0 > WAIT_NS) return false;
   }
 }
 __device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  return mbar_wait_inl(bar, parity, abort_flag);
+  return mbar_wait_inl<64>(bar, parity, abort_flag);
 }
 
 __device__ __forceinline__ uint64_t policy_evict_first() {
