@@ -42,16 +42,18 @@
 // the zeros together make it look at the zeros, whose row of A and column of X
 // say whether products may have underflowed there, and form the tiles again in
 // which they may (DevStatus::range; set-only bits, read after the launch, so the
-// choice is deterministic).  A zero row of A costs nothing that way: 8192 x 8192
-// with one and an element of 2^-60 elsewhere, d = 200: 4059 us for the call when
-// a zero counted as a tiny result, 470 now (295 without; the CUDA cores alone 3785).
+// choice is deterministic).  8192 x 8192 with a zero row and an element of 2^-60
+// elsewhere, d = 200: 4059 us for the call when a zero counted as a tiny result,
+// 470 now (295 without the element; the CUDA cores alone 3785).
 //
-// Bound: shared memory at wide sketches (the six products read 132 KB of
-// operands per 32-deep block at 224 columns, and the parts are written there
-// first: about 1600 clocks against the tensor cores' 1344; measured 1960), HBM
-// at narrow ones.  A^T X of a 20000 x 20000 matrix at d = 220: 0.66 ms (1.06
-// PFLOP of part products at 1.6 PFLOP/s) against 15.7 ms on the CUDA cores; the
-// relative error against FP64 4.5e-7 against 6.4e-7.  Measured slower: FP32
+// Bound: at wide sketches the tensor cores and their operands' shared memory (a
+// 32-deep block at 224 columns is 1344 clocks of tensor work and 132 KB of operand
+// reads, beside the parts' writes; measured 1960 clocks a block at K = 20000; at K
+// = 2048, launch and drain included, the tensor pipe is active 55 % and the LSU's
+// shared-memory pipe 33 % of the time), HBM at narrow ones.  A^T X of a 20000 x
+// 20000 matrix at d = 220: 0.66 ms (1.06 TFLOP of part products at 1.6 PFLOP/s)
+// against 15.7 ms on the CUDA cores; the relative error against FP64 4.5e-7
+// against 6.4e-7.  Measured slower: FP32
 // blocks through registers (2.8k clocks a block whatever its width: the loads
 // were waited for as soon as they were issued), X split by every CTA's
 // converters (1.04 ms), eight accumulator columns per TMEM load (3.9k clocks of

@@ -118,12 +118,15 @@ __device__ __forceinline__ void gram_tile(const float* __restrict__ X, int64_t l
   }
 }
 
-// The same for a single matrix (fewer than 8192 rows: few slabs, each a chain of
-// 512 rows per entry, so latency counts): 32 x 32 tiles, 4 x 4 entries per
+// The same for a single matrix that the tensor-core Gram does not take (fewer than
+// 8192 rows, or more than 256 columns): 32 x 32 tiles, 4 x 4 entries per
 // thread (a row takes 16 multiply-adds of a thread instead of 64, and a
 // 30-column Gram is one tile), the chunks four ahead in a cp.async ring.
-// Every entry is the same sum.  1000 x 30: 39 us with 64 x 64 tiles, 21 with
-// 32 x 32 ones prefetched one chunk ahead, 10 with the ring.
+// Every entry is the same sum.  1000 x 30 (few slabs, each a chain of 512 rows per
+// entry, so latency counts): 39 us with 64 x 64 tiles, 21 with 32 x 32 ones
+// prefetched one chunk ahead, 10 with the ring.  Where the tiles fill the chip the
+// ring still gains over 64 x 64 ones: 16384 x 272 84 -> 62 us, 100000 x 272 408 ->
+// 275, 100000 x 512 811 -> 791.
 constexpr int TMS = 32, GST = 5;
 __device__ __forceinline__ void gram_tile32(const float* __restrict__ X, int64_t ldx,
                                             const float* __restrict__ W, int64_t ldw, int64_t M,

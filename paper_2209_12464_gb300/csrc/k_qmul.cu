@@ -617,8 +617,9 @@ cudaError_t qmul_tc(const float* Y, int64_t ldy, const float* tiles, int64_t M, 
   // Without the transposed BF16 copy, narrow Q = Y S is an FP32 product
   // (k_f32tc.cu), whose load ring and separate epilogue warps keep more of Y in
   // flight (200000 x 110: 9 us less per pass, with a third of the rounding
-  // error); at 20000 x 220 its 157 tiles make two rounds over 152 SMs (40 us
-  // against 28 with k_qmul_tc's equal ranges), so wider Y stays here
+  // error; three passes at d = 128: 19456 rows, one round of tiles over the SMs, 200
+  // -> 179 us, 20000, two rounds, 210 -> 200).  Wider, the second round costs more
+  // than that (20000 x 220: 40 us a pass against 28 with k_qmul_tc's equal ranges)
   const bool plain = Bt == nullptr && dp <= 128 && f32_img_bytes(d, dp) <= qmul_st_bytes(d);
   auto trinv = plain ? k_trinv<true> : k_trinv<false>;
   cudaError_t e =
