@@ -160,6 +160,17 @@ def make_inputs(torch, device, dtype, m, n, gen="haar"):
     return A, A32, Om, sig
 
 
+def f32_tc_roofline(flops, ms, peaks, kernel):
+    """FP32 products on the tensor cores: six BF16 part products per product
+    (whole product phases, the operand's split and the fix-up included)."""
+    peak = peaks.get("bf16_tflops_sustained", 1700.0)
+    achieved = 6.0 * flops / (ms * 1e-3) / 1e12
+    return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            "frac": achieved / peak, "traffic": None,
+            "kernel": f"{kernel} (FP32 product as six BF16 part products, tcgen05)",
+            "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (of measured)"}
+
+
 def tc_traffic(m, n, d):
     """DRAM bytes per product launch from the committed ncu summary (a
     10240^2 capture scaled to the 20000^2 launch), for that workload only."""
@@ -536,15 +547,18 @@ def run_batch(args, torch, dev, local, world, rank, dist):
         cnt = prof["ax"][0] + prof["atx"][0]
         avg = (prof["ax"][1] + prof["atx"][1]) / max(cnt, 1)
         flops = 2.0 * sum(m * n * (k + p) for m, n, k, p in shapes)
-        alu_peak = 152 * 256 * sm_mhz * 1e6 / 1e12
-        achieved = flops / (avg * 1e-3) / 1e12
-        roofline = {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "TFLOP/s",
-                    "frac": achieved / alu_peak, "traffic": None,
-                    "kernel": "k_bgemm (batched CUDA-core product, one pass over every A_i per "
-                              "launch)",
-                    "alg_flops_per_launch": flops, "avg_launch_ms": avg, "launches": cnt,
-                    "peak_source": "derived: 152 SMs x 128 FP32 FMA/clk x 2 x median SM clock",
-                    **common}
+        if args.dtype == "f32":
+            roofline = f32_tc_roofline(flops, avg, peaks, "k_bf32_tc")
+        else:
+            alu_peak = 152 * 256 * sm_mhz * 1e6 / 1e12
+            achieved = flops / (avg * 1e-3) / 1e12
+            roofline = {"bound": "alu", "achieved": achieved, "peak": alu_peak,
+                        "unit": "TFLOP/s", "frac": achieved / alu_peak, "traffic": None,
+                        "kernel": "k_bgemm (batched CUDA-core product, one pass over every A_i "
+                                  "per launch)",
+                        "peak_source": "derived: 152 SMs x 128 FP32 FMA/clk x 2 x median SM "
+                                       "clock"}
+        roofline.update(alg_flops_per_launch=flops, avg_launch_ms=avg, launches=cnt, **common)
 
     # end to end: pinned host inputs -> device, batched call, outputs -> host.
     # The batch's inputs and outputs each live in one packed buffer (every
@@ -1057,8 +1071,13 @@ def main():
         if prof["tc_atx2"][0]:
             roofline["two_part_launch"] = two_part_roofline(
                 prof["tc_atx2"], 4.0 * m * n * dp, bytes_a + 4 * m * dp + 4 * n * dp, peaks)
+    elif args.dtype == "f32":
+        dom = max(("ax", "atx"), key=lambda ph: prof[ph][1])
+        cnt, tot = prof[dom]
+        roofline = f32_tc_roofline(2.0 * m * n * d, tot / max(cnt, 1), peaks, "k_f32_tc")
+        roofline.update(phase_ms=phase_ms, phase_share=share)
     else:
-        # CUDA-core products: FP32 (or FP64) multiply-add bound
+        # CUDA-core products: FP64 (or FP32) multiply-add bound
         dom = max(("ax", "atx"), key=lambda ph: prof[ph][1])
         cnt, tot = prof[dom]
         avg = tot / max(cnt, 1)

@@ -877,7 +877,8 @@ cudaError_t f32_gemm_tc(bool trans, const float* A, int64_t lda, int64_t m, int6
                         const float* X, int64_t ldx, int xcols, int d, int dp, float* out,
                         int64_t ldo, int ocols, float* frag, void* img, DevStatus* st,
                         cudaStream_t stream) {
-  if (ocols < d || ocols > dp || (ocols & 3) || xcols < d || xcols > ldx || (xcols & 3) || (ldx & 3) || ((uintptr_t)X & 15) || (ldo & 3) || ((uintptr_t)out & 15))
+  if (ocols < d || ocols > dp || (ocols & 3) || xcols < d || xcols > ldx || (xcols & 3) ||
+      (ldx & 3) || ((uintptr_t)X & 15) || (ldo & 3) || ((uintptr_t)out & 15))
     return cudaErrorInvalidValue;
   FtParams p{};
   p.A = A;

@@ -350,7 +350,8 @@ cudaError_t copy_cast_2d(Ty ts, const void* src, int64_t lds, Ty td, void* dst, 
                          int64_t rows, int64_t cols, cudaStream_t st) {
   if (rows <= 0 || cols <= 0) return cudaSuccess;
   const size_t as = 4 * ty_size(ts), ad = 4 * ty_size(td);
-  const bool vec = cols % 4 == 0 && lds % 4 == 0 && ldd % 4 == 0 && (uintptr_t)src % as == 0 && (uintptr_t)dst % ad == 0;
+  const bool vec = cols % 4 == 0 && lds % 4 == 0 && ldd % 4 == 0 && (uintptr_t)src % as == 0 &&
+                   (uintptr_t)dst % ad == 0;
   const int grid = ceil_div(rows * cols, vec ? 1024 : 256);
 #define RUQLP_CC(TS_, TD_, CS, CD)                                                           \
   if (ts == TS_ && td == TD_) {                                                              \
