@@ -525,15 +525,15 @@ __device__ __forceinline__ void ft_body(const W& w, int NX, int wmax, int* err) 
           if (++sx == NX) { sx = 0; ph ^= 1u; }
         }
       }
-      if (!ok) {
-        leave();
-        // the copies already issued land before the CTA gives up its shared memory
-        for (; issued > 0; --issued) {
-          if (sx == 0) { sx = NX; ph ^= 1u; }
-          --sx;
-          volatile int never = 0;
-          mbar_wait_inl(fx(sx), ph ^ 1u, &never);
-        }
+      if (!ok) leave();
+      // the copies already issued land before the CTA gives up its shared memory
+      // (also when none is left to issue: the other roles may stop before they use
+      // them)
+      for (; issued > 0; --issued) {
+        if (sx == 0) { sx = NX; ph ^= 1u; }
+        --sx;
+        volatile int never = 0;
+        mbar_wait_inl(fx(sx), ph ^ 1u, &never);
       }
     }
   } else if (wg < 3) {
