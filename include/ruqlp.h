@@ -137,8 +137,10 @@ typedef struct {
  * BF16 inputs use the tensor cores when A's leading dimension is a multiple
  * of 8 elements and A is 16-byte aligned (sketches wider than 256 columns
  * run as column chunks, one pass over A each; up to 384 in one pass when A
- * exceeds 128 MB); otherwise CUDA cores.  FP32 products over 128 rows or more take the tensor
- * cores too, each value split exactly into three BF16 parts (FP32 accuracy).
+ * exceeds 128 MB); otherwise CUDA cores.  FP32 products over 128 rows or more
+ * take the tensor cores too, each value split exactly into three BF16 parts
+ * (FP32 accuracy); ruqlp_sketch over less than 176 rows with less than 40000 of
+ * result stays on the CUDA cores when its operands' rows are not on 16 bytes.
  * omega: n x d row-major FP64 Gaussian test matrix (device memory for
  * ruqlp_decompose / ruqlp_submit; host memory for ruqlp_decompose_host), or
  * NULL: then the library generates it on the device from omega_seed with
